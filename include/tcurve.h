@@ -119,6 +119,8 @@ ts_status ts_real_schemes(const ts_tri *tri, const uint64_t *signs, uint64_t n,
 /* Kernel families (ts_set_kernel).  All compute the same codes.
  *   TS_KERNEL_TABLE: one generic kernel per degree; the triangulation's
  *     tables are staged into shared memory by a bulk copy in every block.
+ *     Blocks classify 64 or 128 sign vectors together, bit-sliced (with
+ *     TS_SCRATCH_GLOBAL: one thread per sign vector).
  *   TS_KERNEL_SPECIALIZED: a kernel generated for this triangulation (its
  *     structure compiled into the instruction stream) with NVRTC on first use;
  *     d <= 9 only (one sign word), TS_EUNSUPPORTED above.
@@ -128,8 +130,8 @@ ts_status ts_real_schemes(const ts_tri *tri, const uint64_t *signs, uint64_t n,
  *     no global scratch).  ts_real_schemes and ts_enumerate; batches run
  *     it as the warp tile of their fused launch (ts_batch_set_fused_tile);
  *     ts_enumerate_noalloc runs the table-driven family.
- *   TS_KERNEL_AUTO (default): specialised for ts_enumerate and for batches of
- *     at least 65536 instances when d <= 9, table-driven otherwise or if the
+ *   TS_KERNEL_AUTO (default): specialised for ts_enumerate (but not for
+ *     TS_ENUM_SPLITMIX) when 4 <= d <= 9, table-driven otherwise or if the
  *     specialised kernel cannot be built. */
 #define TS_KERNEL_AUTO 0
 #define TS_KERNEL_TABLE 1
@@ -143,7 +145,9 @@ ts_status ts_set_kernel(ts_tri *tri, int kind);
  *   TS_SCRATCH_GLOBAL: device memory, L1/L2-resident, allocated per launch
  *     with cudaMallocAsync on the launch's stream and freed after it (the
  *     device's default memory pool is set to keep freed memory).
- *   TS_SCRATCH_AUTO (default): global from d = 7, shared below.
+ *   TS_SCRATCH_AUTO (default): shared for the table-driven kernels, which
+ *     then run bit-sliced as with TS_SCRATCH_SHARED; global from d = 7 for the
+ *     specialised kernels, shared below.
  * Changing it drops the specialised kernels already built for tri (they are
  * rebuilt on next use).  Results are identical. */
 #define TS_SCRATCH_AUTO 0
@@ -262,7 +266,9 @@ void ts_batch_free(ts_batch *batch);
  * with shared scratch the block's scratch must fit shared memory), sign
  * vectors per work item (a multiple of threads) and scratch placement
  * (TS_SCRATCH_*; global scratch is allocated here, grid x threads x
- * scratch words).  Returns TS_EINVAL for tiles that do not fit, and for a
+ * scratch words).  Blocks of 128 threads without TS_SCRATCH_GLOBAL (the
+ * default tile) run bit-sliced; the other tiles run one thread per sign
+ * vector, with global scratch from d = 7 for TS_SCRATCH_AUTO.  Returns TS_EINVAL for tiles that do not fit, and for a
  * specialised group (ts_batch_info) any block size but 128 or shared
  * scratch: its code is compiled for 128-thread blocks and global scratch.
  * Waits for
@@ -275,26 +281,24 @@ ts_status ts_batch_set_tile(ts_batch *batch, int d, int threads, int chunk, int 
  * filling the whole GPU.  Takes effect at the next run (a new graph is
  * captured).  TS_EINVAL for other values. */
 ts_status ts_batch_set_serial(ts_batch *batch, int serial);
-/* One persistent launch for the whole batch (an engine facility against the
- * kernel-dispatch overhead that Sec. 3 names as a cost at scale): with
- * fused = 1, ts_batch_run launches a single kernel that pulls the work items
- * of every job of every degree from one counter (jobs in degree order, so
- * the degrees follow one another without a gap), stages a job's tables with
- * cp.async.bulk when it moves to another triangulation, and runs each job
- * with its degree's fused tile (ts_batch_set_fused_tile).  The kernel is
- * compiled per range of degrees with the register budget of that range's
- * table-driven sweep (degrees up to 6, 9, 11, 16: 40, 48, 64, 80
- * registers); a batch takes the range of its largest degree, or the widest
- * one when a degree has a warp tile.  Specialised groups do not apply in
- * this mode.  fused = 0 (default) returns to one persistent kernel per
- * degree group (ts_batch_set_serial).  Allocates the job table and global
- * scratch of the launch here (grid x 128 threads x scratch words), after
- * waiting for all work on the device; the next run with use_graph captures
- * a new graph.  TS_EINVAL for other values. */
+/* One persistent kernel per tier of degrees for the whole batch (an engine
+ * facility against the kernel-dispatch overhead that Sec. 3 names as a cost at
+ * scale): with fused = 1, ts_batch_run launches one kernel for the jobs of
+ * degrees up to 6, one for 7 and 8, one for 9 and 10 and one above (as many
+ * as the batch has degrees for), and one for the degrees with a warp tile,
+ * the largest degrees first, the others on streams forked from the run's.
+ * Each pulls the work items of its jobs from one counter, stages a job's
+ * tables with cp.async.bulk when it moves to another triangulation, and runs
+ * each job with its degree's fused tile (ts_batch_set_fused_tile).
+ * Specialised groups do not apply in this mode.  fused = 0 (default) returns
+ * to one persistent kernel per degree group (ts_batch_set_serial).  Allocates
+ * the job table of the launches here, after waiting for all work on the
+ * device; the next run with use_graph captures a new graph.  TS_EINVAL for
+ * other values. */
 ts_status ts_batch_set_fused(ts_batch *batch, int fused);
 /* Tile of degree d in the fused launch: kind TS_KERNEL_TABLE or
- * TS_KERNEL_AUTO (default: one thread per sign vector, the table-driven
- * sweep, per-thread scratch in global memory) or TS_KERNEL_WARP (d >= 7:
+ * TS_KERNEL_AUTO (default: blocks of 128 sign vectors, bit-sliced, all in
+ * shared memory) or TS_KERNEL_WARP (d >= 7:
  * the 32 lanes of a warp classify one sign vector together, the state in
  * shared memory), and chunk sign vectors per work item (a multiple of 128,
  * at most 2^24; default 1024).  May be set in either mode; in fused mode it
@@ -334,8 +338,8 @@ ts_status ts_batch_run(ts_batch *batch, int use_graph, void *stream);
  * (ts_batch_set_tile accepts only those; the chunk may vary).  In fused
  * mode (ts_batch_set_fused) info describes the degree's fused tile instead:
  * kernel TS_KERNEL_TABLE or TS_KERNEL_WARP, 128 threads, its chunk, scratch
- * TS_SCRATCH_GLOBAL (thread tiles) or TS_SCRATCH_SHARED (warp tiles), and
- * the registers, resident blocks and grid of the one fused kernel.
+ * TS_SCRATCH_SHARED, and the registers, resident blocks and grid of its
+ * tier's kernel.
  *   info  receives kernel (TS_KERNEL_*), threads per block, chunk (sign
  *         vectors per work item), scratch (TS_SCRATCH_*), registers per
  *         thread, local_bytes (per-thread local memory: spills, call

@@ -31,12 +31,11 @@
 
 #include "engine.h"
 #include "tc_layout.h"
+#include "tc_stage.cuh"
 #include "tc_table_sweep.cuh"
 
 namespace tcurve {
 namespace {
-
-constexpr long kWaitIters = 1L << 22;
 
 // Largest table of degree d: 2V + |E(T^diamond)| words, V = 2d^2 + 2d + 1 and
 // |E(T^diamond)| = 6d^2 + 2d, padded to 16 bytes.
@@ -53,27 +52,11 @@ struct JobK : TcTableK<D_, T_, true> {
                                                  227 * 1024;
 };
 
-struct DevJob {
-  const u32 *tab;
-  u64 n;              // sign vectors
-  u64 base;           // splitmix64 counter base of the sign vectors
-  u64 *codes;         // per-instance codes, code_words each (or null)
-  u64 *hkeys;         // job histogram (open addressing, code_words per key, 0 = empty)
-  unsigned long long *hcnt;
-  u64 hslots;
-  u64 chunk0;         // first work item of the job
-  u32 fn, pad;        // specialised groups: index of the job's function in the module
-};
-static_assert(sizeof(DevJob) == 72, "the job table layout of the generated batch kernels");
 
 // Degree groups of at least this many sign vectors run specialised code
 // (TS_KERNEL_AUTO): the compile at creation (about a second per
 // triangulation, in parallel) pays for itself.
 constexpr uint64_t kJitGroupMin = 1ull << 22;
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
 
 template <int D, int T, bool G>
 __global__ void __launch_bounds__(T)
@@ -256,6 +239,9 @@ struct ts_batch {
   struct Group {  // all jobs of one degree
     int d = 0, threads = 64, chunk = 1024;
     bool global = false;        // per-thread scratch in global memory
+    bool sliced = false;        // the bit-sliced kernel (kSlicedThreads threads, shared memory)
+    uint32_t stable_words = 0;  // its tables (largest of the group's) and areas
+    size_t sarea = 0;
     std::shared_ptr<JitJobsModule> jit;  // specialised kernel (null: table-driven)
     std::string jit_log;        // why the specialised kernel could not be built
     JobsFn fn = nullptr;        // the kernel of this tile, its launch shape
@@ -291,17 +277,20 @@ struct ts_batch {
   std::vector<ts_tri *> tris;  // triangulation of every job
   std::vector<const uint64_t *> signs;  // caller sign vectors of every job (null: splitmix64)
   bool serial = false;         // degree groups one after the other (else concurrent streams)
-  // fused launch (ts_batch_set_fused): one persistent kernel over all jobs
+  // fused plan (ts_batch_set_fused): one persistent kernel per tier of degrees
+  struct Tier {
+    int tier = -1;
+    uint32_t job0 = 0, njobs = 0, toff = 0, ws = 0;
+    uint64_t items = 0;
+    unsigned grid = 1;
+    size_t smem = 0;
+  };
   bool fused = false;
-  FusedJob *d_fjobs = nullptr;  // jobs sorted by degree
-  uint64_t fitems = 0;
-  int ftier = -1;
-  unsigned fgrid = 1;
-  size_t fsmem = 0;
-  uint32_t ftoff = 0, fls = 0, fws = 0;
-  uint32_t *fscratch = nullptr;
-  size_t fscratch_bytes = 0;
-  unsigned long long *d_fwork = nullptr;
+  std::vector<Tier> tiers;     // largest degrees first
+  FusedJob *d_fjobs = nullptr;  // jobs tier by tier
+  unsigned long long *d_fwork = nullptr;  // one counter per tier
+  cudaStream_t fstream[kFusedTiers + 1] = {};  // of the tiers after the first
+  cudaEvent_t fdone[kFusedTiers + 1] = {};
 };
 
 namespace {
@@ -329,7 +318,16 @@ cudaError_t upload_group(ts_batch *b, ts_batch::Group &g) {
 cudaError_t prepare_group(ts_batch::Group &g) {
   int per_sm = 0, sms = 0, dev = 0;
   cudaError_t e = cudaSuccess;
-  if (g.jit) {  // specialised: 128-thread blocks, global scratch, grid from its occupancy
+  if (!g.jit && g.sliced) {
+    const void *fn = sliced_jobs_fn(g.d);
+    if (!fn) return cudaErrorInvalidConfiguration;
+    g.fn = nullptr;
+    g.smem = ((size_t)g.stable_words * 4 + 127) / 128 * 128 + 128 + g.sarea;
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxBlockSmem);
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, g.threads, g.smem);
+    if (e != cudaSuccess) return e;
+  } else if (g.jit) {  // specialised: 128-thread blocks, global scratch, grid from its occupancy
     g.fn = nullptr;
     g.smem = 0;
     per_sm = jit_jobs_blocks_per_sm(*g.jit);
@@ -337,8 +335,9 @@ cudaError_t prepare_group(ts_batch::Group &g) {
     g.fn = jobs_fn_dt(g.d, g.threads, g.global);
     if (!g.fn) return cudaErrorInvalidConfiguration;
     g.smem = jobs_smem(g.d, g.threads, g.table_words, g.ls_words, g.global);
+    // whichever batch was planned last, every launch may have its own size
     e = cudaFuncSetAttribute((const void *)g.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)g.smem);
+                             kMaxBlockSmem);
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)g.fn, g.threads, g.smem);
     if (e != cudaSuccess) return e;
@@ -364,9 +363,13 @@ cudaError_t prepare_group(ts_batch::Group &g) {
 }
 
 cudaError_t launch_group(ts_batch *b, ts_batch::Group &g, cudaStream_t st) {
-  if (!g.fn && !g.jit) return cudaErrorInvalidConfiguration;
+  if (!g.fn && !g.jit && !g.sliced) return cudaErrorInvalidConfiguration;
   cudaError_t e = cudaMemsetAsync(g.d_work, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
+  if (!g.jit && g.sliced)
+    return sliced_jobs_launch(g.d, g.grid, g.smem, (g.stable_words * 4 + 127) / 128 * 128, g.d_jobs,
+                              (uint32_t)g.jobs.size(), g.items, (uint32_t)g.chunk, g.d_work, b->d_err,
+                              b->d_failed, st);
   if (g.jit)
     return jit_jobs_launch(*g.jit, g.grid, g.d_jobs, (uint32_t)g.jobs.size(), g.items,
                            (uint32_t)g.chunk, g.d_work, b->d_err, b->d_failed, g.scratch, st);
@@ -376,97 +379,78 @@ cudaError_t launch_group(ts_batch *b, ts_batch::Group &g, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Job table, kernel tier, shared memory, persistent grid and global scratch
-// of the fused launch (host work only, never while a stream is captured):
-// the jobs in degree order, each with its degree's tile; the tier of the
-// largest degree, or the warp tier when a degree has a warp tile.
+// Job table and launches of the fused plan (host work only, never while a
+// stream is captured): the jobs tier by tier, each with its degree's tile,
+// and per tier the shared memory of its largest job and a persistent grid.
 cudaError_t prepare_fused(ts_batch *b) {
-  std::vector<const ts_batch::Group *> gs;
-  for (const auto &g : b->groups) gs.push_back(&g);
-  std::sort(gs.begin(), gs.end(), [](const ts_batch::Group *x, const ts_batch::Group *y) {
-    return x->d < y->d;
-  });
   std::vector<FusedJob> fj;
-  uint64_t items = 0;
-  uint32_t maxtab = 0, wsw = 0, lsw = 0;
-  int dmax = 0;
-  bool anywarp = false;
-  for (const ts_batch::Group *g : gs) {
-    for (int j : g->jobs) {
-      const DevJob &dj = b->jobs[j];
-      const ts_tri *t = b->tris[j];
-      FusedJob x{};
-      x.n = dj.n;
-      x.base = dj.base;
-      x.codes = dj.codes;
-      x.hkeys = dj.hkeys;
-      x.hcnt = dj.hcnt;
-      x.hslots = dj.hslots;
-      x.item0 = items;
-      x.signs = reinterpret_cast<const unsigned long long *>(b->signs[j]);
-      x.d = (uint32_t)g->d;
-      x.chunk = (uint32_t)g->fchunk;
-      x.warp = (uint32_t)g->fwarp;
-      if (x.warp) {
-        x.tab = t->d_wtables;
-        x.tab_words = t->wlay.words;
-        x.wl = t->wlay;
-        wsw = std::max(wsw, fused_warp_words(g->d));
-        anywarp = true;
-      } else {
-        x.tab = t->d_tables;
-        x.tab_words = t->lay.words;
-        x.off_fan = t->lay.off_fan;
-        x.off_vext = t->lay.off_vext;
-        const uint32_t epw = tc_layout(g->d, true, kFusedThreads).epw;
-        lsw = std::max(lsw, (t->lay.nslots + epw - 1) / epw);
-      }
-      maxtab = std::max(maxtab, x.tab_words);
-      items += (x.n + x.chunk - 1) / x.chunk;
-      dmax = std::max(dmax, g->d);
-      fj.push_back(x);
-    }
-  }
-  const int tier = anywarp ? kFusedWarpTier : fused_tier(dmax);
-  if (tier < 0 || fj.empty()) return cudaErrorInvalidConfiguration;
-  const uint32_t toff = (maxtab * 4 + 127) / 128 * 128;
-  const size_t smem = (size_t)toff + 128 + (size_t)kFusedThreads * lsw * 4 +
-                      (anywarp ? (size_t)4 * wsw * 4 : 0);
-  if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  int per_sm = 0, sms = 0, dev = 0;
-  cudaError_t e = fused_occupancy(tier, smem, &per_sm);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  std::vector<ts_batch::Tier> tiers;
+  int sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint64_t cap = (uint64_t)per_sm * sms;
-  const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(cap, items));
-  const size_t need = (size_t)grid * kFusedThreads * fused_slab_words(tier) * 4;
-  if (need > b->fscratch_bytes) {
-    if (b->fscratch) cudaFree(b->fscratch);
-    b->fscratch = nullptr;
-    b->fscratch_bytes = 0;
-    e = cudaMalloc(&b->fscratch, need);
+  for (int tier = kFusedTiers; tier >= 0; --tier) {
+    ts_batch::Tier T;
+    T.tier = tier;
+    T.job0 = (uint32_t)fj.size();
+    uint32_t maxtab = 0;
+    size_t area = 0;
+    for (const auto &g : b->groups) {
+      if ((g.fwarp ? kFusedWarpTier : fused_tier(g.d)) != tier) continue;
+      for (int j : g.jobs) {
+        const DevJob &dj = b->jobs[j];
+        const ts_tri *t = b->tris[j];
+        FusedJob x{};
+        x.n = dj.n;
+        x.base = dj.base;
+        x.codes = dj.codes;
+        x.hkeys = dj.hkeys;
+        x.hcnt = dj.hcnt;
+        x.hslots = dj.hslots;
+        x.item0 = T.items;
+        x.signs = reinterpret_cast<const unsigned long long *>(b->signs[j]);
+        x.d = (uint32_t)g.d;
+        x.chunk = (uint32_t)g.fchunk;
+        x.sl = t->slay;
+        x.wl = t->wlay;
+        if (g.fwarp) {
+          x.tab = t->d_wtables;
+          x.tab_words = t->wlay.words;
+          T.ws = std::max(T.ws, fused_warp_words(g.d));
+          area = std::max(area, (size_t)4 * T.ws * 4);
+        } else {
+          x.tab = t->d_stables;
+          x.tab_words = t->slay.words;
+          area = std::max(area, fused_area_bytes(g.d, t->slay));
+        }
+        maxtab = std::max(maxtab, x.tab_words);
+        T.items += (x.n + x.chunk - 1) / x.chunk;
+        fj.push_back(x);
+      }
+    }
+    T.njobs = (uint32_t)fj.size() - T.job0;
+    if (!T.njobs) continue;
+    T.toff = (maxtab * 4 + 127) / 128 * 128;
+    T.smem = (size_t)T.toff + 128 + area;
+    if (T.smem > (size_t)kMaxBlockSmem) return cudaErrorInvalidConfiguration;
+    int per_sm = 0;
+    cudaError_t e = fused_occupancy(tier, T.smem, &per_sm);
     if (e != cudaSuccess) return e;
-    b->fscratch_bytes = need;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    T.grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)per_sm * sms, T.items));
+    tiers.push_back(T);
   }
-  if (!b->d_fjobs) {
-    e = cudaMalloc(&b->d_fjobs, sizeof(FusedJob) * fj.size());
-    if (e != cudaSuccess) return e;
+  if (fj.empty()) return cudaErrorInvalidConfiguration;
+  cudaError_t e = cudaSuccess;
+  for (size_t k = 1; k < tiers.size() && e == cudaSuccess; ++k) {
+    if (!b->fstream[k]) e = cudaStreamCreateWithFlags(&b->fstream[k], cudaStreamNonBlocking);
+    if (e == cudaSuccess && !b->fdone[k]) e = cudaEventCreateWithFlags(&b->fdone[k], cudaEventDisableTiming);
   }
-  if (!b->d_fwork) {
-    e = cudaMalloc(&b->d_fwork, sizeof(unsigned long long));
-    if (e != cudaSuccess) return e;
-  }
-  e = cudaMemcpy(b->d_fjobs, fj.data(), sizeof(FusedJob) * fj.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && !b->d_fjobs) e = cudaMalloc(&b->d_fjobs, sizeof(FusedJob) * fj.size());
+  if (e == cudaSuccess && !b->d_fwork) e = cudaMalloc(&b->d_fwork, sizeof(unsigned long long) * (kFusedTiers + 1));
+  if (e == cudaSuccess)
+    e = cudaMemcpy(b->d_fjobs, fj.data(), sizeof(FusedJob) * fj.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return e;
-  b->fitems = items;
-  b->ftier = tier;
-  b->fgrid = grid;
-  b->fsmem = smem;
-  b->ftoff = toff;
-  b->fls = lsw;
-  b->fws = wsw;
+  b->tiers = tiers;
   return cudaSuccess;
 }
 
@@ -477,12 +461,20 @@ cudaError_t enqueue(ts_batch *b, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_counts, 0, b->count_words * 8, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_err, 0, 4, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_failed, 0, 8, st);
-  if (b->fused) {  // one persistent kernel for every job of every degree
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_fwork, 0, sizeof(unsigned long long), st);
+  if (b->fused) {  // one persistent kernel per tier, the later ones on forked streams
     if (e == cudaSuccess)
-      e = fused_launch(b->ftier, b->fgrid, b->fsmem, b->ftoff, b->fls, b->fws, b->d_fjobs,
-                       (uint32_t)b->jobs.size(), b->fitems, b->d_fwork, b->d_err, b->d_failed,
-                       b->fscratch, st);
+      e = cudaMemsetAsync(b->d_fwork, 0, sizeof(unsigned long long) * (kFusedTiers + 1), st);
+    if (e == cudaSuccess && b->tiers.size() > 1) e = cudaEventRecord(b->fork, st);
+    for (size_t k = 0; k < b->tiers.size(); ++k) {
+      const auto &T = b->tiers[k];
+      cudaStream_t s = k ? b->fstream[k] : st;
+      if (e == cudaSuccess && k) e = cudaStreamWaitEvent(s, b->fork, 0);
+      if (e == cudaSuccess)
+        e = fused_launch(T.tier, T.grid, T.smem, T.toff, T.ws, b->d_fjobs + T.job0, T.njobs, T.items,
+                         b->d_fwork + k, b->d_err, b->d_failed, s);
+      if (e == cudaSuccess && k) e = cudaEventRecord(b->fdone[k], s);
+      if (e == cudaSuccess && k) e = cudaStreamWaitEvent(st, b->fdone[k], 0);
+    }
     return e;
   }
   if (b->serial) {  // one degree after the other, each persistent kernel on the whole GPU
@@ -500,14 +492,20 @@ cudaError_t enqueue(ts_batch *b, cudaStream_t st) {
   return e;
 }
 
-// Table-driven tile of a group at creation: global scratch from d = 7 with
-// 128-thread blocks, shared scratch below (64-thread blocks from d = 8).
+// Tile of a table-driven group: the bit-sliced kernel for blocks of 128
+// threads unless global scratch is asked for, else the sweep with one thread
+// per sign vector, its scratch placed as asked (TS_SCRATCH_AUTO: global from
+// d = 7).
+void table_tile(ts_batch::Group &g, int threads, int chunk, int scratch) {
+  g.sliced = threads == kSlicedThreads && scratch != TS_SCRATCH_GLOBAL;
+  g.global = !g.sliced && (scratch == TS_SCRATCH_GLOBAL ||
+                           (scratch == TS_SCRATCH_AUTO && g.d >= kGlobalScratchFrom));
+  g.threads = threads;
+  g.chunk = chunk;
+}
 void table_defaults(ts_batch::Group &g) {
   g.jit.reset();
-  g.global = g.d >= kGlobalScratchFrom;
-  g.threads = g.global ? 128 : (g.d >= 8 ? 64 : 128);
-  while (g.threads > 32 && !jobs_fn_dt(g.d, g.threads, g.global)) g.threads -= 32;
-  g.chunk = g.threads * 8;
+  table_tile(g, kSlicedThreads, kSlicedThreads * 8, TS_SCRATCH_AUTO);
 }
 
 // TS_KERNEL_AUTO at creation: specialised code for groups of at least
@@ -559,6 +557,7 @@ bool make_specialised(ts_batch *b, const std::vector<int> &gids) {
       g.jit = mods[k];
       g.jit_log.clear();
       g.global = true;
+      g.sliced = false;
       g.threads = jit_jobs_threads();
       g.chunk = g.threads * 16;
     } else {
@@ -616,10 +615,13 @@ ts_status ts_batch_create(int njobs, ts_tri *const *tris, const uint64_t *counts
     x.tab = t->d_tables;
     x.n = counts[j];
     x.base = bases[j];
-    x.codes = code_outputs ? reinterpret_cast<u64 *>(code_outputs[j]) : nullptr;
-    x.hkeys = reinterpret_cast<u64 *>(b->d_keys + b->kofs[j]);
+    x.codes = code_outputs ? reinterpret_cast<unsigned long long *>(code_outputs[j]) : nullptr;
+    x.hkeys = reinterpret_cast<unsigned long long *>(b->d_keys + b->kofs[j]);
     x.hcnt = b->d_counts + b->cofs[j];
     x.hslots = b->jslots[j];
+    x.stab = t->d_stables;
+    x.swords = t->slay.words;
+    x.schunks = t->slay.chunks;
     b->jobs.push_back(x);
     b->degree.push_back(t->d);
     b->tris.push_back(tris[j]);
@@ -639,6 +641,8 @@ ts_status ts_batch_create(int njobs, ts_tri *const *tris, const uint64_t *counts
     grp.table_words = std::max(grp.table_words, t->lay.words);
     const uint32_t epw = (uint32_t)tc_layout(t->d, true, 32).epw;
     grp.ls_words = std::max(grp.ls_words, (t->lay.nslots + epw - 1) / epw);
+    grp.stable_words = std::max(grp.stable_words, t->slay.words);
+    grp.sarea = std::max(grp.sarea, fused_area_bytes(t->d, t->slay));
   }
   if (e == cudaSuccess) {
     std::vector<int> spec;
@@ -672,8 +676,11 @@ void ts_batch_free(ts_batch *b) {
     if (g.done) cudaEventDestroy(g.done);
   }
   if (b->fork) cudaEventDestroy(b->fork);
+  for (auto &f : b->fstream)
+    if (f) cudaStreamDestroy(f);
+  for (auto &f : b->fdone)
+    if (f) cudaEventDestroy(f);
   if (b->d_fjobs) cudaFree(b->d_fjobs);
-  if (b->fscratch) cudaFree(b->fscratch);
   if (b->d_fwork) cudaFree(b->d_fwork);
   if (b->d_keys) cudaFree(b->d_keys);
   if (b->d_counts) cudaFree(b->d_counts);
@@ -688,20 +695,22 @@ ts_status ts_batch_set_tile(ts_batch *b, int d, int threads, int chunk, int scra
     return TS_EINVAL;
   for (auto &g : b->groups) {
     if (g.d != d) continue;
-    bool global = scratch == TS_SCRATCH_AUTO ? d >= kGlobalScratchFrom : scratch == TS_SCRATCH_GLOBAL;
+    const bool global = scratch == TS_SCRATCH_AUTO ? d >= kGlobalScratchFrom : scratch == TS_SCRATCH_GLOBAL;
     if (g.jit) {  // specialised: the block size and global scratch are fixed at compile time
       if (threads != jit_jobs_threads() || scratch == TS_SCRATCH_SHARED) return TS_EINVAL;
-      global = true;
-    } else if (!jobs_fn_dt(d, threads, global)) {
+    } else if (!(threads == kSlicedThreads && scratch != TS_SCRATCH_GLOBAL) && !jobs_fn_dt(d, threads, global)) {
       return TS_EINVAL;  // block does not fit shared memory
     }
     // runs already launched (graph launches included) read the job table and
     // the scratch that this call rewrites or frees: let them finish first
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_st(e);
-    g.threads = threads;
-    g.chunk = chunk;
-    g.global = global;
+    if (g.jit) {
+      g.threads = threads;
+      g.chunk = chunk;
+    } else {
+      table_tile(g, threads, chunk, scratch);
+    }
     if (b->exec) {
       cudaGraphExecDestroy(b->exec);
       b->exec = nullptr;
@@ -848,10 +857,13 @@ ts_status ts_batch_info(const ts_batch *b, int d, ts_batch_group_info *info, cha
       x.kernel = g.fwarp ? TS_KERNEL_WARP : TS_KERNEL_TABLE;
       x.threads = kFusedThreads;
       x.chunk = g.fchunk;
-      x.scratch = g.fwarp ? TS_SCRATCH_SHARED : TS_SCRATCH_GLOBAL;
-      x.grid = (int)b->fgrid;
-      fused_attrs(b->ftier, &x.registers, &x.local_bytes);
-      fused_occupancy(b->ftier, b->fsmem, &x.blocks_per_sm);
+      x.scratch = TS_SCRATCH_SHARED;
+      for (const auto &T : b->tiers)
+        if (T.tier == (g.fwarp ? kFusedWarpTier : fused_tier(g.d))) {
+          x.grid = (int)T.grid;
+          fused_attrs(T.tier, &x.registers, &x.local_bytes);
+          fused_occupancy(T.tier, T.smem, &x.blocks_per_sm);
+        }
       *info = x;
       if (log && len) log[0] = 0;
       return TS_OK;
@@ -864,14 +876,13 @@ ts_status ts_batch_info(const ts_batch *b, int d, ts_batch_group_info *info, cha
     if (g.jit) {
       jit_jobs_attrs(*g.jit, &x.registers, &x.local_bytes);
       x.blocks_per_sm = jit_jobs_blocks_per_sm(*g.jit);
-    } else if (g.fn) {
+    } else if (const void *fn = g.sliced ? sliced_jobs_fn(g.d) : (const void *)g.fn) {
       cudaFuncAttributes fa{};
-      if (cudaFuncGetAttributes(&fa, (const void *)g.fn) == cudaSuccess) {
+      if (cudaFuncGetAttributes(&fa, fn) == cudaSuccess) {
         x.registers = fa.numRegs;
         x.local_bytes = (int)fa.localSizeBytes;
       }
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x.blocks_per_sm, (const void *)g.fn, g.threads,
-                                                    g.smem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x.blocks_per_sm, fn, g.threads, g.smem);
     }
     *info = x;
     if (log && len) {

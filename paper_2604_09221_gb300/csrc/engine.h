@@ -2,6 +2,7 @@
 // CUDA kernels (kernels.cu).  Not part of the public ABI (include/tcurve.h).
 #pragma once
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include <memory>
@@ -46,6 +47,12 @@ struct WarpLayout {
   uint32_t off_v, off_e, off_anti, off_bedge;
   uint32_t words;  // padded to a multiple of 4
 };
+// Tables of the bit-sliced kernels (format at the top of tc_sliced.cuh).
+struct SlicedLayout {
+  uint32_t words;   // padded to a multiple of 4
+  uint32_t chunks;  // event chunks of 32: label starts, joins, boundary edges
+  uint32_t far;     // steps of four fan entries beyond a vertex's row of planes
+};
 // Device error word bits.
 enum : uint32_t {
   kErrInternal = 1u,   // invariant violated (root, tree, scratch)
@@ -72,6 +79,8 @@ struct JitModule;  // compiled specialised kernels (jit.cpp)
 bool pack_diamond_tables(const Diamond &D, std::vector<uint32_t> &tables, TableLayout &lay);
 // Tables of the warp-per-instance kernels (host.cpp; format at WarpLayout).
 bool pack_warp_tables(const Diamond &D, std::vector<uint32_t> &tables, WarpLayout &lay);
+// Tables of the bit-sliced kernels (host.cpp; format in tc_sliced.cuh).
+bool pack_sliced_tables(const Diamond &D, std::vector<uint32_t> &tables, SlicedLayout &lay);
 // Label slot of every vertex in the table-driven sweep (a slot is reused once
 // its vertex has no later reader) and, in *nslots, how many slots are used.
 std::vector<int> lab_slots(const Diamond &D, int *nslots);
@@ -96,6 +105,9 @@ struct ts_tri {
   tcurve::WarpLayout wlay{};
   std::vector<uint32_t> host_wtables;
   uint32_t *d_wtables = nullptr;  // wlay.words words (warp-per-instance kernels)
+  tcurve::SlicedLayout slay{};
+  std::vector<uint32_t> host_stables;
+  uint32_t *d_stables = nullptr;  // slay.words words (bit-sliced kernels)
   uint32_t *d_err = nullptr;     // device error word (scratch, owned here)
   tcurve::Diamond dia;
   int kernel = 0;                // TS_KERNEL_*
@@ -187,40 +199,63 @@ cudaError_t jit_jobs_launch(const JitJobsModule &m, unsigned grid, const void *j
                             uint64_t items, uint32_t chunk, unsigned long long *work, uint32_t *err,
                             unsigned long long *failed, uint32_t *scratch, cudaStream_t st);
 
-// Fused batch kernel (fused.cu): one persistent launch over the jobs of all
-// degrees of a batch, each degree with its own tile (one thread or one warp
-// per sign vector, sign vectors per work item).
+constexpr int kMaxBlockSmem = 227 * 1024;  // dynamic shared memory a block can have
+
+// A batch's job as the degree-group kernels read it (the generated kernels of
+// jit.cpp name the same fields).
+struct DevJob {
+  const uint32_t *tab;
+  unsigned long long n;      // sign vectors
+  unsigned long long base;   // splitmix64 counter base of the sign vectors
+  unsigned long long *codes;  // per-instance codes, code_words each (or null)
+  unsigned long long *hkeys;  // job histogram (open addressing, code_words per key, 0 = empty)
+  unsigned long long *hcnt;
+  unsigned long long hslots;
+  unsigned long long chunk0;  // first work item of the job
+  uint32_t fn, pad;           // specialised groups: index of the job's function in the module
+  const uint32_t *stab;       // tables of the bit-sliced kernel, their words and event chunks
+  uint32_t swords, schunks;
+};
+static_assert(sizeof(DevJob) == 88 && offsetof(DevJob, fn) == 64,
+              "the job table layout of the generated batch kernels");
+
+// The bit-sliced kernel of a degree group (sliced_jobs.cu): smem = toff (the
+// tables, 128-byte aligned) + 128 + fused_area_bytes.
+constexpr int kSlicedThreads = 128;  // threads and sign vectors per block
+const void *sliced_jobs_fn(int d);
+cudaError_t sliced_jobs_launch(int d, unsigned grid, size_t smem, uint32_t toff, const DevJob *jobs,
+                               uint32_t njobs, uint64_t items, uint32_t chunk, unsigned long long *work,
+                               uint32_t *err, unsigned long long *failed, cudaStream_t st);
+
+// Fused batch plan (fused.cu): one persistent kernel per tier of degrees over
+// the batch's jobs, each degree with its own tile (bit-sliced or one warp per
+// sign vector, sign vectors per work item).
 constexpr int kFusedThreads = 128;  // threads per block (4 warps)
-constexpr int kFusedTiers = 4;      // register tiers: degrees up to 6, 9, 11, 16
-constexpr int kFusedWarpTier = 4;   // the tier-3 kernel with warp-per-instance bodies
+constexpr int kFusedTiers = 4;      // bit-sliced tiers: degrees up to 6, 8, 10, 16
+constexpr int kFusedWarpTier = 4;   // the kernel of the warp-per-instance tiles
 constexpr int kFusedWarpFrom = 7;   // warp-per-instance bodies from this degree
 struct FusedJob {
-  const uint32_t *tab;   // tables staged for the job: table-driven or warp layout (tile)
+  const uint32_t *tab;   // tables staged for the job: bit-sliced or warp layout (tile)
   uint64_t n, base;      // sign vectors, splitmix64 counter base
   unsigned long long *codes;  // per-instance codes or null
   unsigned long long *hkeys;  // the job's histogram
   unsigned long long *hcnt;
   uint64_t hslots;
-  uint64_t item0;        // first work item of the job
+  uint64_t item0;        // first work item of the job in its tier
   uint32_t d, chunk;     // degree; sign vectors per work item (a multiple of kFusedThreads)
-  uint32_t warp;         // 1: warp per instance (warp tables), 0: thread per instance
   uint32_t tab_words;    // words staged (a multiple of 4)
-  uint32_t off_fan, off_vext;  // table-driven layout
-  WarpLayout wl;               // warp layout
-  uint32_t pad;
+  SlicedLayout sl;       // bit-sliced layout
+  WarpLayout wl;         // warp layout
   const unsigned long long *signs;  // the caller's sign vectors (n x words), or null: splitmix64
 };
-int fused_tier(int dmax);          // tier of a batch whose largest degree is dmax (-1: none)
-int fused_tier_degree(int tier);   // largest degree of a tier
-uint32_t fused_slab_words(int tier);  // global scratch words per thread of a tier's kernel
+int fused_tier(int d);  // bit-sliced tier of a degree (-1: none)
+size_t fused_area_bytes(int d, const SlicedLayout &l);  // a block's areas behind the tables
 uint32_t fused_warp_words(int d);     // shared words of one warp of a degree-d warp tile
 cudaError_t fused_occupancy(int tier, size_t smem, int *blocks_per_sm);
 cudaError_t fused_attrs(int tier, int *regs, int *local_bytes);
-// smem = toff (the tables, 128-byte aligned) + 128 + kFusedThreads x
-// ls_words words (label slots of the thread tiles) + 4 x ws_stride words
-// (warp tiles); scratch: grid x kFusedThreads x fused_slab_words(tier) words.
-cudaError_t fused_launch(int tier, unsigned grid, size_t smem, uint32_t toff, uint32_t ls_words,
-                         uint32_t ws_stride, const FusedJob *jobs, uint32_t njobs, uint64_t items,
-                         unsigned long long *work, uint32_t *err, unsigned long long *failed,
-                         uint32_t *scratch, cudaStream_t st);
+// smem = toff (the tables, 128-byte aligned) + 128 + the largest area, or
+// 4 x ws_stride words (warp tier).
+cudaError_t fused_launch(int tier, unsigned grid, size_t smem, uint32_t toff, uint32_t ws_stride,
+                         const FusedJob *jobs, uint32_t njobs, uint64_t items, unsigned long long *work,
+                         uint32_t *err, unsigned long long *failed, cudaStream_t st);
 }  // namespace tcurve

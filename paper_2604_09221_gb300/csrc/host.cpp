@@ -334,12 +334,120 @@ bool pack_warp_tables(const Diamond &D, std::vector<uint32_t> &tables, WarpLayou
   lay = L;
   return true;
 }
+// Tables of the bit-sliced kernels (format in tc_sliced.cuh).  The vertices
+// of the logic phase are listed by fan length, so that the threads of a warp
+// run fans of one length; a join site is a fan entry that can start a second
+// run (the second entry only if it is not linked to the first).  Returns
+// false if a field does not fit.
+bool pack_sliced_tables(const Diamond &D, std::vector<uint32_t> &tables, SlicedLayout &lay) {
+  const int V = D.V, d = D.d, H = d * d;  // [0, H) lower half, [H, 2H) upper half, then the middle row
+  const uint32_t ncb = ((uint32_t)V + 31) / 32;
+  std::vector<uint32_t> fan, vd(V), first(V), site0(V, 0), half_sites, mid_sites;
+  uint32_t half_steps[2] = {0, 0}, far = 0, half_far[2] = {0, 0};
+  // steps whose takes fit the vertex's row of label planes (TcSlK::TW / 4)
+  const size_t near = V <= 256 ? 2 : 4;
+  auto can_join = [&](int v, size_t i) { return i >= 2 || (i == 1 && !D.link[v][1]); };
+  for (int v = 0; v < V; ++v) {
+    if (v == H || v == 2 * H) {
+      half_steps[v / H - 1] = (uint32_t)fan.size() / 4;
+      half_far[v / H - 1] = far;
+    }
+    const size_t len = D.fan[v].size(), padded = len ? (len + 3) / 4 * 4 : 4;
+    if (len > 255 || fan.size() > 0xFFFF || D.k[v] > 255) return false;
+    first[v] = (uint32_t)fan.size();
+    vd[v] = (len ? (uint32_t)D.fan[v][0] | 1u << 15 : 0u) | (far << 16);
+    if (padded / 4 > near) far += (uint32_t)(padded / 4 - near);
+    for (size_t i = 0; i < D.fan[v].size(); ++i) {
+      const int u = D.fan[v][i];
+      if (v < 2 * H && (u < H) != (v < H)) return false;  // no edge leaves a half-diamond
+      fan.push_back((uint32_t)D.k[u] | ((uint32_t)u << 8) | (can_join(v, i) ? 1u << 24 : 0u) |
+                    (i % 4 == 0 && i + 4 < len ? 1u << 25 : 0u) | ((uint32_t)D.link[v][i] << 30) |
+                    ((uint32_t)(D.c[u] ^ D.c[v] ^ 1) << 31));
+      if (can_join(v, i))
+        (v < 2 * H ? half_sites : mid_sites).push_back((uint32_t)v | ((uint32_t)u << 16));
+    }
+    for (size_t i = len; i < padded; ++i) fan.push_back((uint32_t)D.k[v]);
+  }
+  // the half-diamonds are mirror images: as many steps each
+  if (half_steps[1] != 2 * half_steps[0] || half_far[1] != 2 * half_far[0] || far > 0xFFFF) return false;
+  // chunks of joins: the half-diamonds', one of boundary pairs, the middle
+  // row's (with the corner pair of even d); at least as many as start chunks
+  if (d % 2 == 0) mid_sites.push_back(0);  // the corner pair, below
+  uint32_t nc1 = ((uint32_t)half_sites.size() + 31) / 32;
+  const uint32_t ncm = ((uint32_t)mid_sites.size() + 31) / 32;
+  nc1 = std::max(nc1, ncb > ncm + 1 ? ncb - ncm - 1 : 0u);
+  uint32_t next_half = 32 * ncb, next_mid = 32 * (ncb + nc1 + 1);
+  for (int v = 0; v < V; ++v) {
+    uint32_t &next = v < 2 * H ? next_half : next_mid;
+    site0[v] = next;
+    for (size_t i = 0; i < D.fan[v].size(); ++i) next += can_join(v, i) ? 1 : 0;
+  }
+  std::vector<uint32_t> site(32 * (nc1 + 1 + ncm), 0), bx(2 * d), be(2 * d);
+  std::copy(half_sites.begin(), half_sites.end(), site.begin());
+  std::copy(mid_sites.begin(), mid_sites.end(), site.begin() + 32 * (nc1 + 1));
+  // the boundary in cyclic order, p[t + 2d] antipodal to p[t]
+  std::map<std::pair<int, int>, int> pos;
+  for (int v = 0; v < V; ++v) pos[{D.x[v], D.y[v]}] = v;
+  std::vector<int> p;
+  for (int t = 0; t < d; ++t) p.push_back(pos.at({d - t, t}));
+  for (int t = 0; t < d; ++t) p.push_back(pos.at({-t, d - t}));
+  for (int t = 0; t <= 2 * d; ++t) {  // the other half
+    const int q = t < 2 * d ? p[t] : p[0];
+    p.push_back(t < 2 * d ? pos.at({-D.x[q], -D.y[q]}) : q);
+  }
+  for (int t = 0; t < 2 * d; ++t) {
+    const int a = p[t], b = p[t + 1];            // edge t; if crossed, it joins
+    const int x = p[t + 1], y = p[t + 1 + 2 * d];  // the pair behind it
+    uint32_t slot = 32 * (ncb + nc1) + (uint32_t)t;
+    uint32_t pair = (uint32_t)std::min(x, y) | ((uint32_t)std::max(x, y) << 16);
+    if (d % 2 == 0 && D.y[x] == 0) {  // the corner pair goes with the middle row, parity 1
+      slot = next_mid;
+      pair |= 1u << 31;
+    }
+    if (slot > 0x7FFF) return false;
+    bx[t] = (uint32_t)D.k[a] | ((uint32_t)D.k[b] << 8) | ((uint32_t)(D.c[a] ^ D.c[b]) << 16) | (slot << 17);
+    be[t] = (uint32_t)a | ((uint32_t)b << 16);
+    site[slot - 32 * ncb] = pair;
+  }
+  std::vector<int> order(V);
+  for (int v = 0; v < V; ++v) order[v] = v;
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int a, int b) { return D.fan[a].size() > D.fan[b].size(); });
+  tables.assign(12, 0);
+  for (int v : order) {
+    tables.push_back((uint32_t)D.k[v] | ((uint32_t)std::max<size_t>(1, (D.fan[v].size() + 3) / 4) << 8) |
+                     (first[v] << 16));
+    tables.push_back((uint32_t)v | (site0[v] << 16));
+  }
+  auto put = [&](const std::vector<uint32_t> &w) {
+    while (tables.size() % 4) tables.push_back(0);  // the fan's steps are read four words at a time
+    const uint32_t at = (uint32_t)tables.size();
+    tables.insert(tables.end(), w.begin(), w.end());
+    return at;
+  };
+  tables[0] = half_steps[0];
+  tables[8] = (uint32_t)fan.size() / 4;
+  tables[9] = half_far[0];
+  tables[1] = nc1;
+  tables[2] = ncb + nc1 + 1 + ncm;
+  tables[3] = put(fan);
+  tables[4] = put(vd);
+  tables[5] = put(site);
+  tables[6] = put(bx);
+  tables[7] = put(be);
+  while (tables.size() % 4) tables.push_back(0);
+  lay.words = (uint32_t)tables.size();
+  lay.chunks = ncb + nc1 + 1 + ncm;
+  lay.far = far;
+  return true;
+}
 }  // namespace tcurve
 
 namespace {
 
 bool pack_tables(const Diamond &D, ts_tri *t) {
   if (!pack_diamond_tables(D, t->host_tables, t->lay)) return false;
+  if (!pack_sliced_tables(D, t->host_stables, t->slay)) return false;
   if (!pack_warp_tables(D, t->host_wtables, t->wlay)) return false;
   t->V = D.V;
   return true;
@@ -427,6 +535,10 @@ ts_status ts_load_triangulation(int d, const int32_t *edges_ij, int n_edges, ts_
   if (e == cudaSuccess)
     e = cudaMemcpy(t->d_wtables, t->host_wtables.data(), t->wlay.words * sizeof(uint32_t),
                    cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMalloc(&t->d_stables, t->slay.words * sizeof(uint32_t));
+  if (e == cudaSuccess)
+    e = cudaMemcpy(t->d_stables, t->host_stables.data(), t->slay.words * sizeof(uint32_t),
+                   cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&t->d_err, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(t->d_err, 0, sizeof(uint32_t));
   if (e != cudaSuccess) {
@@ -443,6 +555,7 @@ void ts_free_triangulation(ts_tri *t) {
   jit_release(t);
   if (t->d_tables) cudaFree(t->d_tables);
   if (t->d_wtables) cudaFree(t->d_wtables);
+  if (t->d_stables) cudaFree(t->d_stables);
   if (t->d_err) cudaFree(t->d_err);
   delete t;
 }
@@ -453,13 +566,17 @@ int ts_sign_words(const ts_tri *t) { return t ? t->sw : 0; }
 int ts_code_words(const ts_tri *t) { return t ? t->cw : 0; }
 
 namespace {
-// Kernel choice: the specialised kernel for sweeps and large batches (AUTO),
-// the table-driven kernel otherwise or when specialisation is unavailable.
-bool want_specialised(ts_tri *t, uint64_t n, bool sweep) {
+// Kernel choice (AUTO): the specialised block sweep for sweeps whose masks
+// share their high bits; the table-driven (bit-sliced) kernels for queries
+// and sampled sweeps, which the specialised per-mask kernels lose to (d = 7,
+// random sign vectors: 1.8 against 4.2e9 schemes/s), for d < 4, where a block
+// has fewer masks than a warp has lanes, and when specialisation is
+// unavailable.
+bool want_specialised(ts_tri *t, bool sweep) {
   if (t->kernel == TS_KERNEL_TABLE || t->kernel == TS_KERNEL_WARP || t->d > kMaxSpecialized)
     return false;
   if (t->kernel == TS_KERNEL_SPECIALIZED) return true;
-  if (!sweep && n < (1u << 16)) return false;
+  if (!sweep || t->d < 4) return false;
   return jit_prepare(t) == cudaSuccess;
 }
 }  // namespace
@@ -471,7 +588,7 @@ ts_status ts_real_schemes(const ts_tri *tc, const uint64_t *signs, uint64_t n, u
   ts_tri *t = const_cast<ts_tri *>(tc);  // only the lazily compiled kernel cache changes
   if (t->kernel == TS_KERNEL_WARP)
     return cuda_status(launch_real_schemes_warp(t, signs, n, codes, (cudaStream_t)stream));
-  if (want_specialised(t, n, false))
+  if (want_specialised(t, false))
     return cuda_status(launch_real_schemes_jit(t, signs, n, codes, (cudaStream_t)stream));
   return cuda_status(launch_real_schemes(t, signs, n, codes, (cudaStream_t)stream));
 }
@@ -671,7 +788,7 @@ ts_status ts_enumerate(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags
   ts_tri *tm = const_cast<ts_tri *>(t);
   if (tm->kernel == TS_KERNEL_WARP)
     return cuda_status(launch_enumerate_warp(tm, lo, hi, flags, h, (cudaStream_t)stream));
-  if (want_specialised(tm, hi - lo, true))
+  if (want_specialised(tm, !(flags & TS_ENUM_SPLITMIX)))
     return cuda_status(launch_enumerate_jit(tm, lo, hi, flags, h, (cudaStream_t)stream));
   return cuda_status(launch_enumerate(t, lo, hi, flags, h, (cudaStream_t)stream));
 }

@@ -694,6 +694,8 @@ struct TcjJob {
   unsigned long long *hcnt;
   unsigned long long hslots, chunk0;   // its slots; its first work item
   unsigned fn, pad;                    // index of its specialised function
+  const unsigned *stab;                // (the bit-sliced kernel's tables)
+  unsigned swords, schunks;
 };
 )TCJS";
 

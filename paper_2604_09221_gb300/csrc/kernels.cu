@@ -27,6 +27,7 @@
 
 #include "engine.h"
 #include "tc_layout.h"
+#include "tc_sliced.cuh"
 #include "tc_stage.cuh"
 #include "tc_table_sweep.cuh"
 
@@ -96,6 +97,11 @@ __device__ __forceinline__ void fan_offsets(u32 *tab, const TableLayout &L) {
   tc_fan_to_offsets(tab + L.off_fan, L.NF, TcScratch<K>::EPW, K::LBYTES, K::THREADS, threadIdx.x,
                     K::THREADS);
   __syncthreads();
+}
+
+// Bytes of a bit-sliced kernel's tables in shared memory.
+__host__ __device__ constexpr uint32_t sliced_table_bytes(uint32_t words) {
+  return (words * 4 + 127) / 128 * 128;
 }
 
 // ----------------------------------------------------- query kernel ----
@@ -178,6 +184,97 @@ __global__ void __launch_bounds__(TableK<D, G>::THREADS)
   if (failed) atomicAdd(h.d_failed, failed);
 }
 
+// ------------------------------------------------ bit-sliced kernels ----
+//
+// Blocks of 128 threads classify 128 sign vectors at a time (tc_sliced.cuh).
+// smem: tables (toff bytes) | mbarrier, work slot (128 bytes) | the block's
+// areas | hash table (sweeps of one-word codes).
+template <int D>
+using SlicedK = TcSlK<D, 4>;
+
+template <class K>
+__global__ void __launch_bounds__(K::T)
+    sliced_real_schemes_kernel(SlicedLayout L, const uint32_t *__restrict__ gtab,
+                               const uint64_t *__restrict__ signs, uint64_t n, uint64_t *codes,
+                               uint32_t *err_word) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  const uint32_t toff = sliced_table_bytes(L.words);
+  u32 *const tab = reinterpret_cast<u32 *>(smem);
+  if (!stage_tables(tab, gtab, L.words * 4, reinterpret_cast<uint64_t *>(smem + toff), err_word)) return;
+  const TcSlMem M = tc_sl_carve<K>(tab, reinterpret_cast<u32 *>(smem + toff + 128), L.chunks);
+  const u32 t = threadIdx.x, mine = tc_sl_instance<K>(t);
+  const u64 *sg = reinterpret_cast<const u64 *>(signs);
+  uint32_t err = 0;
+  for (uint64_t base = (uint64_t)blockIdx.x * K::T; base < n; base += (uint64_t)gridDim.x * K::T) {
+    TcSig<K::W> s{};
+    if (base + t < n) s = tc_load_sig<K>(sg, base + t);
+    u32 e = 0;
+    u64 code[K::CW];
+    tc_sl_classify<K>(M, s, t, e, code);
+    if (base + mine < n) {
+      err |= e;
+#pragma unroll
+      for (u32 w = 0; w < K::CW; ++w) codes[(base + mine) * K::CW + w] = code[w];
+    }
+    __syncthreads();
+  }
+  if (err) atomicOr(err_word, err);
+}
+
+template <class K>
+__global__ void __launch_bounds__(K::T)
+    sliced_enumerate_kernel(SlicedLayout L, const uint32_t *__restrict__ gtab, uint64_t lo, uint64_t total,
+                            uint32_t flags, ts_hist h) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  const uint32_t toff = sliced_table_bytes(L.words);
+  u32 *const tab = reinterpret_cast<u32 *>(smem);
+  u32 *const area = reinterpret_cast<u32 *>(smem + toff + 128);
+  unsigned long long *const slot = reinterpret_cast<unsigned long long *>(smem + toff + 64);
+  u64 *const hkeys = reinterpret_cast<u64 *>(area + tc_sl_words<K>(L.chunks, L.far));
+  unsigned long long *const hcnt = reinterpret_cast<unsigned long long *>(hkeys + K::HASH);
+  const u32 t = threadIdx.x, mine = tc_sl_instance<K>(t);
+  for (u32 s = t; s < K::HASH; s += K::T) {
+    hkeys[s] = 0;
+    hcnt[s] = 0;
+  }
+  if (t == 0) *slot = atomicAdd(h.d_work, (unsigned long long)K::T);
+  if (!stage_tables(tab, gtab, L.words * 4, reinterpret_cast<uint64_t *>(smem + toff), h.d_err)) return;
+  const TcSlMem M = tc_sl_carve<K>(tab, area, L.chunks);
+  uint32_t err = 0;
+  unsigned long long failed = 0;
+  for (;;) {
+    const uint64_t base = *slot;
+    if (base >= total) break;
+    __syncthreads();
+    // the next work item is fetched while this one runs
+    if (t == 0) *slot = atomicAdd(h.d_work, (unsigned long long)K::T);
+    u32 e = 0;
+    u64 code[K::CW];
+    tc_sl_classify<K>(M, tc_enum_sig<K::W>(lo + base + t, flags, K::D), t, e, code);
+    u64 any = 0;
+    const bool live = base + mine < total;
+#pragma unroll
+    for (u32 w = 0; w < K::CW; ++w) {
+      code[w] = live ? code[w] : 0ull;
+      any |= code[w];
+    }
+    err |= live ? e : 0u;
+    failed += live && any == 0;
+    if constexpr (K::CW == 1)
+      tc_hist_add<K::HASH>(code[0], hkeys, hcnt, reinterpret_cast<u64 *>(h.d_keys), h.d_counts, h.slots,
+                           h.d_err);
+    else
+      tc_hist_add_wide<K::CW>(code, reinterpret_cast<u64 *>(h.d_keys), h.d_counts, h.slots, h.d_err);
+    __syncthreads();
+  }
+  __syncthreads();
+  for (u32 s = t; s < K::HASH; s += K::T)
+    if (hkeys[s])
+      tc_global_add(reinterpret_cast<u64 *>(h.d_keys), h.d_counts, h.slots, h.d_err, hkeys[s], hcnt[s]);
+  if (err) atomicOr(h.d_err, err);
+  if (failed) atomicAdd(h.d_failed, failed);
+}
+
 // Word w of sign vector i is splitmix64((base + i) * W + w); the top word is
 // cut to the |A| - 64 (W - 1) bits that exist.
 __global__ void splitmix_masks_kernel(uint64_t base, uint64_t n, uint32_t npoints, uint64_t *out) {
@@ -251,7 +348,8 @@ int sm_count() {
 // Grid of a persistent launch: resident blocks per SM x SMs, at most `want`.
 template <class F>
 cudaError_t persistent_grid(F fn, int threads, size_t smem, uint64_t want, unsigned *grid) {
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the most a block can have: launches of other sizes may come from other threads
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxBlockSmem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
@@ -272,6 +370,34 @@ struct GlobalScratch {
     if (p) cudaFreeAsync(p, st);
   }
 };
+
+template <int D>
+cudaError_t real_schemes_sliced(const ts_tri *t, const uint64_t *signs, uint64_t n, uint64_t *codes,
+                                cudaStream_t st) {
+  typedef SlicedK<D> K;
+  const size_t smem = sliced_table_bytes(t->slay.words) + 128 + (size_t)tc_sl_words<K>(t->slay.chunks, t->slay.far) * 4;
+  unsigned grid = 0;
+  cudaError_t e = persistent_grid(sliced_real_schemes_kernel<K>, K::T, smem, (n + K::T - 1) / K::T, &grid);
+  if (e != cudaSuccess) return e;
+  sliced_real_schemes_kernel<K><<<grid, K::T, smem, st>>>(t->slay, t->d_stables, signs, n, codes, t->d_err);
+  return cudaGetLastError();
+}
+
+template <int D>
+cudaError_t enumerate_sliced(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *h,
+                             cudaStream_t st) {
+  typedef SlicedK<D> K;
+  const size_t smem = sliced_table_bytes(t->slay.words) + 128 + (size_t)tc_sl_words<K>(t->slay.chunks, t->slay.far) * 4 +
+                      (size_t)K::HASH * 16;
+  const uint64_t total = hi - lo;
+  unsigned grid = 0;
+  cudaError_t e = persistent_grid(sliced_enumerate_kernel<K>, K::T, smem, (total + K::T - 1) / K::T, &grid);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(h->d_work, 0, sizeof(unsigned long long), st);
+  if (e != cudaSuccess) return e;
+  sliced_enumerate_kernel<K><<<grid, K::T, smem, st>>>(t->slay, t->d_stables, lo, total, flags, *h);
+  return cudaGetLastError();
+}
 
 template <int D, bool G>
 cudaError_t real_schemes_dg(const ts_tri *t, const uint64_t *signs, uint64_t n, uint64_t *codes,
@@ -309,25 +435,21 @@ cudaError_t enumerate_dg(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t fla
   return cudaGetLastError();
 }
 
-// Global scratch from d = 7 unless the triangulation asks otherwise.
-bool global_scratch(const ts_tri *t) {
-  if (t->scratch == TS_SCRATCH_SHARED) return false;
-  if (t->scratch == TS_SCRATCH_GLOBAL) return true;
-  return t->d >= kGlobalScratchFrom;
-}
+// One thread per sign vector, scratch in global memory, only when asked for.
+bool global_scratch(const ts_tri *t) { return t->scratch == TS_SCRATCH_GLOBAL; }
 
 template <int D>
 cudaError_t real_schemes_d(const ts_tri *t, const uint64_t *signs, uint64_t n, uint64_t *codes,
                            cudaStream_t st) {
   return global_scratch(t) ? real_schemes_dg<D, true>(t, signs, n, codes, st)
-                           : real_schemes_dg<D, false>(t, signs, n, codes, st);
+                           : real_schemes_sliced<D>(t, signs, n, codes, st);
 }
 
 template <int D>
 cudaError_t enumerate_d(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *h,
                         cudaStream_t st, bool allow_global) {
   return allow_global && global_scratch(t) ? enumerate_dg<D, true>(t, lo, hi, flags, h, st)
-                                           : enumerate_dg<D, false>(t, lo, hi, flags, h, st);
+                                           : enumerate_sliced<D>(t, lo, hi, flags, h, st);
 }
 
 }  // namespace

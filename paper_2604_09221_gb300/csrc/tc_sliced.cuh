@@ -1,0 +1,783 @@
+// tc_sliced.cuh -- Algorithm 1 for a block of sign vectors at once, bit-sliced
+// (the table-driven query, sweep and batch kernels).
+//
+// A block of NG warps classifies T = 32 NG sign vectors together.  The part
+// of the method that looks at every edge of T^diamond (crossing tests, which
+// earlier neighbour gives a vertex its label, where two runs of a fan have to
+// be joined) is plain logic, so it runs on 32 sign vectors per instruction:
+// bit i of a word is instance i of a group of 32.  Only the few events it
+// leaves (about one vertex in eight starts a label, about one in eight joins
+// two) are handled one instance per thread.  Phases, a barrier between each:
+//
+//   planes   sign vectors -> one word per lattice point and group (32 x 32
+//            bit transposes across the warp)
+//   logic    (vertex, group) per thread, vertices in order of fan length:
+//            for every fan entry the mask of the instances that take their
+//            label from it (first same-sign entry), per vertex the mask of
+//            the instances in which it starts a label, per entry that can
+//            start a second run the mask of the instances that have to join
+//   labels   the labels as bit planes, vertices in sweep order (the two
+//            half-diamonds side by side, then the middle row):
+//            L(v) = start(v) ? id(v) : OR over entries of take & L(u); a
+//            label's id is the vertex that starts it.  The takes of v lie
+//            where its planes will be (steps of longer fans: "far" steps, in
+//            the last area)
+//   tiles    planes -> one byte (d >= 11: half-word) per vertex and
+//            instance, in place; event masks -> one word per instance
+//   trees    one instance per thread: joins in a union-find over the label
+//            bytes themselves (a vertex that starts a label points at itself),
+//            regions, region tree, root and code
+//
+// Everything a block touches is in shared memory; nothing is allocated.
+//
+// Orientation parity (even d, Alg. 1 lines 6-7).  Before the middle row a set
+// of labels can mix the two half-diamonds only through antipodal pairs
+// (parity 1), so the parity between two labels is whether their halves
+// differ.  Links are stored relative to that: the half joins and the
+// antipodal joins need no parity at all, and only joins of the middle row
+// (and its corner pair) carry a "twist" bit.
+//
+// Antipodal joins.  Consecutive boundary vertices of one sign are joined by
+// their boundary edge, and so are their antipodes; so a pair is joined only
+// where the boundary edge in front of it is crossed.  Those crossed edges are
+// also the pseudoline's candidates (odd d).
+#pragma once
+
+#include "tc_layout.h"
+#include "tc_runtime.cuh"
+
+// Table words (host.cpp, pack_sliced_tables), staged into shared memory:
+//   header   [0] steps of a half-diamond  [1] event chunks of half-diamond
+//            joins  [2] event chunks in all  [3] off_fan  [4] off_vd
+//            [5] off_site  [6] off_bx  [7] off_be  [8] steps in all
+//            [9] far steps of a half-diamond
+//   task[V]  two words per vertex, in order of fan length: k(v) (8 bits) |
+//            fan steps << 8 (8 bits) | first fan entry << 16, and
+//            v | first join site << 16
+//   fan[]    in steps of four entries, vertices in sweep order, a vertex's
+//            last step padded (one step for an empty fan): k(u) (8 bits) |
+//            u << 8 (16 bits) | "can start a second run" << 24 | "another step
+//            of this vertex follows" << 25 | link << 30 |
+//            (c(u) ^ c(v) ^ 1) << 31; padding: k(v), never of v's sign
+//   vd[V]    u of the first fan entry | "the fan is not empty" << 15 |
+//            first far step << 16
+//   site[]   32 per chunk of join events: v | u << 16 (| parity << 31 for the
+//            corner pair of even d): the half-diamonds' sites, one chunk of
+//            boundary pairs, the middle row's sites
+//   bx[2d]   k(a) | k(b) << 8 | (c(a) ^ c(b)) << 16 | event slot << 17 of the
+//            boundary edges of half the boundary, in cyclic order
+//   be[2d]   a | b << 16 of the same edges
+#define TC_SL_HEADER 12u
+#define TC_SL_GROUP 40u  // words of one group's event chunk: 32 and a pad
+                         // (the trees phase reads it conflict-free)
+
+template <int D_, int NG_>
+struct TcSlK {
+  static constexpr TcLayout L = tc_layout(D_, true, 32);
+  static constexpr u32 D = D_, NG = NG_, T = 32 * NG_, V = L.V, NPOINTS = L.np, W = L.sw,
+                       CW = L.cw, RMAX = L.rmax, WIDE = L.wide, HASH = L.hash, CODE64 = L.code64;
+  static constexpr u32 H = D * D;                 // vertices of one half-diamond
+  static constexpr u32 LB = V <= 256 ? 1 : 2;     // bytes per label
+  static constexpr u32 NPL = V <= 128 ? 7 : V <= 256 ? 8 : V <= 512 ? 9 : 10;  // label planes
+  static constexpr u32 TW = 8 * LB;               // words of a vertex's tile per group
+  static constexpr u32 PP = NG >= 8 ? 4 : 2;      // planes per thread in the labels phase
+  static constexpr u32 PS = TW / PP;              // threads per group there
+  static constexpr u32 NCB = (V + 31) / 32;       // birth chunks
+  static constexpr bool EVEN = D % 2 == 0;
+  static constexpr bool TWTOP = LB == 2 || V <= 128;   // twist bit in the label's top bit
+  static constexpr u32 TWWORDS = EVEN && !TWTOP ? NCB : 0;  // else in words of their own
+  static constexpr u32 LABW = V * TW * NG;        // words of the label area
+  static constexpr u32 PAR_WORDS = (RMAX * T + 3) / 4;  // region parents, a byte each
+  static constexpr u32 PLANES = (NPOINTS * NG + 3) & ~3u;
+  static constexpr u32 BW = PAR_WORDS + TWWORDS * T;
+  // tree codes: the wide back end's scratch lies over the label area
+  static constexpr u32 THREADS = T;
+  static constexpr u32 WB = (RMAX + 3) / 4, WARENA = L.warena_words;
+  static constexpr u32 OFF_WPAR = 0, OFF_WFC = WB, OFF_WNS = 2 * WB, OFF_WENT = 3 * WB,
+                       OFF_WARENA = 3 * WB + (RMAX / 2 + 2 + 1) / 2,
+                       OFF_WTEMP = OFF_WARENA + WARENA, WIDE_WORDS = OFF_WTEMP + WARENA;
+  static_assert(!WIDE || WIDE_WORDS * T <= LABW, "the wide back end's scratch fits the label area");
+  // unused members TcScratch names
+  static constexpr u32 LBYTES = LB, OFF_LPAR = 0, OFF_CAND = 0;
+};
+
+// Shared-memory areas of a block.
+struct TcSlMem {
+  const u32 *tab;  // staged tables
+  u32 *lab;        // label planes, then label bytes (K::LABW words)
+  u32 *ev;         // event chunks (chunks x NG x TC_SL_GROUP words)
+  u32 *x;          // sign planes and takes, then region parents and twists
+};
+
+// Words of the last area: sign planes and the takes of far steps (four per
+// step and group); in the trees phase region parents and twists.
+template <class K>
+__host__ __device__ constexpr u32 tc_sl_xwords(u32 far) {
+  return ((K::PLANES + 4 * far * K::NG > K::BW ? K::PLANES + 4 * far * K::NG : K::BW) + 3) & ~3u;
+}
+
+// Words of a block's areas behind the tables (chunks of events, far steps).
+template <class K>
+__host__ __device__ constexpr u32 tc_sl_words(u32 chunks, u32 far) {
+  return K::LABW + chunks * K::NG * TC_SL_GROUP + tc_sl_xwords<K>(far);
+}
+
+template <class K>
+__device__ __forceinline__ TcSlMem tc_sl_carve(const u32 *tab, u32 *area, u32 chunks) {
+  TcSlMem m;
+  m.tab = tab;
+  m.lab = area;
+  m.ev = m.lab + K::LABW;
+  m.x = m.ev + chunks * K::NG * TC_SL_GROUP;
+  return m;
+}
+
+struct alignas(16) TcQuad {
+  u32 a, b, c, d;
+};
+struct alignas(8) TcPair {
+  u32 a, b;
+};
+
+// 32 x 32 bit transpose across a warp: lane r's word is row r; lane r gets
+// column r.  Stage j exchanges words with the lane at distance j and swaps the
+// off-diagonal j x j blocks: one shuffle, one rotate (by the lane's side), one
+// bitwise select.
+#ifndef TC_SL_EMULATE
+struct TcTranspose {
+  u32 keep[5], rot[5];
+  __device__ __forceinline__ explicit TcTranspose(u32 lane) {
+#pragma unroll
+    for (u32 s = 0; s < 5; ++s) {
+      const u32 j = 16u >> s, m = 0xFFFFFFFFu / ((1u << j) + 1u);  // low halves of the 2j-bit blocks
+      keep[s] = (lane & j) ? ~m : m;
+      rot[s] = (lane & j) ? 32u - j : j;
+    }
+  }
+  __device__ __forceinline__ u32 operator()(u32 x) const {
+#pragma unroll
+    for (u32 s = 0; s < 5; ++s) {
+      const u32 y = __shfl_xor_sync(0xffffffffu, x, 16u >> s);
+      x = (x & keep[s]) | (__funnelshift_l(y, y, rot[s]) & ~keep[s]);
+    }
+    return x;
+  }
+};
+#endif
+
+// Instance (of the block's T) that thread t holds in the trees phase: label
+// bytes of one vertex are T consecutive bytes, four instances to a word, and
+// a warp's threads read 32 different words, so that any mix of vertices is
+// free of bank conflicts.
+template <class K>
+__device__ __forceinline__ u32 tc_sl_instance(u32 t) {
+  constexpr u32 WR = K::TW * K::NG;  // words per vertex
+  const u32 word = t % WR, part = t / WR, g = word / K::TW, q = word % K::TW;
+  return 32u * g + (K::LB == 1 ? 8u * part + q : 8u * (2u * (q >> 3) + part) + (q & 7u));
+}
+
+// ---- planes: clear the event chunks; transpose the sign words ----
+template <class K>
+__device__ __forceinline__ void tc_sl_clear(const TcSlMem &m, u32 t) {
+  const u32 n = m.tab[2] * K::NG * TC_SL_GROUP;
+  for (u32 i = t; i < n; i += K::T) m.ev[i] = 0;
+}
+
+// sg: the sign vector of instance t of the block (warp t / 32 is a group).
+#ifndef TC_SL_EMULATE
+template <class K>
+__device__ __forceinline__ void tc_sl_planes(const TcSlMem &m, const TcSig<K::W> &sg, u32 t) {
+  const u32 g = t >> 5, lane = t & 31u;
+  const TcTranspose transpose(lane);
+#pragma unroll
+  for (u32 j = 0; j < (K::NPOINTS + 31) / 32; ++j) {
+    const u32 half = (u32)(sg.w[j / 2] >> (32 * (j & 1)));
+    const u32 p = transpose(half);
+    if (32 * j + lane < K::NPOINTS) m.x[(32 * j + lane) * K::NG + g] = p;
+  }
+}
+#endif
+
+// All ones if bit b of f is set, else zero.
+__device__ __forceinline__ u32 tc_bitmask(u32 f, u32 b) { return (u32)((int)(f << (31u - b)) >> 31); }
+
+template <class K>
+__device__ __forceinline__ u32 *tc_sl_event(const TcSlMem &m, u32 slot, u32 g) {
+  return m.ev + ((slot >> 5) * K::NG + g) * TC_SL_GROUP + (slot & 31u);
+}
+
+// ---- logic: one (vertex, group) at a time, four fan entries a step ----
+template <class K>
+__device__ __forceinline__ void tc_sl_logic(const TcSlMem &m, u32 t) {
+  const u32 g = t % K::NG;
+  const u32 *const P = m.x + g;
+  const TcPair *task = reinterpret_cast<const TcPair *>(m.tab + TC_SL_HEADER) + t / K::NG;
+  const u32 *const fan = m.tab + m.tab[3];
+  for (u32 k = t / K::NG; k < K::V; k += 32u, task += 32) {
+    const TcPair w = *task;
+    const u32 sv = P[(w.a & 255u) * K::NG], steps = (w.a >> 8) & 255u, v = w.b & 0xFFFFu;
+    u32 site = w.b >> 16, any = 0, prev = 0;
+    const TcQuad *f = reinterpret_cast<const TcQuad *>(fan + (w.a >> 16));
+    TcQuad *take = reinterpret_cast<TcQuad *>(m.lab + (v * K::NG + g) * K::TW);
+    for (u32 j = 0; j < steps; ++j, ++f) {
+      if (j >= K::TW / 4)  // a far step
+        take = reinterpret_cast<TcQuad *>(m.x + K::PLANES) +
+               ((m.tab[m.tab[4] + v] >> 16) + j - K::TW / 4) * K::NG + g;
+      const TcQuad q = *f;
+      // the four entries' masks "same sign as v"
+      const u32 ea = P[(q.a & 255u) * K::NG] ^ sv ^ (u32)((int)q.a >> 31);
+      const u32 eb = P[(q.b & 255u) * K::NG] ^ sv ^ (u32)((int)q.b >> 31);
+      const u32 ec = P[(q.c & 255u) * K::NG] ^ sv ^ (u32)((int)q.c >> 31);
+      const u32 ed = P[(q.d & 255u) * K::NG] ^ sv ^ (u32)((int)q.d >> 31);
+      TcQuad o;
+      auto entry = [&](u32 f, u32 e) -> u32 {
+        if (f & (1u << 24)) {  // a run that may follow another one
+          *tc_sl_event<K>(m, site, g) = e & any & ~(prev & tc_bitmask(f, 30));
+          ++site;
+        }
+        const u32 x = e & ~any;
+        any |= e;
+        prev = e;
+        return x;
+      };
+      o.a = entry(q.a, ea);
+      o.b = entry(q.b, eb);
+      o.c = entry(q.c, ec);
+      o.d = entry(q.d, ed);
+      *take = o;
+      ++take;
+    }
+    *tc_sl_event<K>(m, v, g) = ~any;  // v starts a label
+  }
+  // crossed boundary edges
+  const u32 *const bx = m.tab + m.tab[6];
+  for (u32 k = t / K::NG; k < 2 * K::D; k += 32u) {
+    const u32 w = bx[k];
+    *tc_sl_event<K>(m, w >> 17, g) = P[(w & 255u) * K::NG] ^ P[((w >> 8) & 255u) * K::NG] ^ tc_bitmask(w, 16);
+  }
+}
+
+// ---- labels: steps [s0, s1), vertices from v and far steps from `far` on,
+// K::PP planes per thread ----
+// A serial chain from vertex to vertex: the fan entries and takes of the next
+// step, which do not depend on it, are loaded a step ahead.  The threads of a
+// group are in one warp: they have all read a vertex's takes before one of
+// them writes its planes over them (mask: the warp's threads in this call).
+template <u32 PP>
+struct TcPlanes;
+template <>
+struct TcPlanes<2> {
+  typedef TcPair T;
+  static __device__ __forceinline__ void acc(u32 (&a)[2], u32 s, const T &p) {
+    a[0] |= s & p.a;
+    a[1] |= s & p.b;
+  }
+  static __device__ __forceinline__ T out(const u32 (&a)[2]) { return T{a[0], a[1]}; }
+};
+template <>
+struct TcPlanes<4> {
+  typedef TcQuad T;
+  static __device__ __forceinline__ void acc(u32 (&a)[4], u32 s, const T &p) {
+    a[0] |= s & p.a;
+    a[1] |= s & p.b;
+    a[2] |= s & p.c;
+    a[3] |= s & p.d;
+  }
+  static __device__ __forceinline__ T out(const u32 (&a)[4]) { return T{a[0], a[1], a[2], a[3]}; }
+};
+
+template <class K>
+__device__ __forceinline__ void tc_sl_label_run(const TcSlMem &m, u32 g, u32 part, u32 s0, u32 s1, u32 v,
+                                                u32 far, u32 mask) {
+  typedef TcPlanes<K::PP> PL;
+  typedef typename PL::T plane_t;
+  constexpr u32 ROW = K::TW * K::NG * 4;  // bytes per vertex
+  constexpr u32 NEAR = K::TW / 4;         // steps whose takes lie in the vertex's row
+  const TcQuad *fan = reinterpret_cast<const TcQuad *>(m.tab + m.tab[3]) + s0;
+  u8 *const L = reinterpret_cast<u8 *>(m.lab + g * K::TW + K::PP * part);
+  const TcQuad *ft = reinterpret_cast<const TcQuad *>(m.x + K::PLANES) + far * K::NG + g;
+  u32 row = v * ROW;
+  const u8 *const T = reinterpret_cast<const u8 *>(m.lab + g * K::TW);
+  auto planes = [&](u32 f) -> const plane_t & {
+    return *reinterpret_cast<const plane_t *>(L + ((f >> 8) & 0xFFFFu) * ROW);
+  };
+  TcQuad f = fan[0], s = *reinterpret_cast<const TcQuad *>(T + row);
+  u32 a[K::PP] = {}, any = 0, j = 0;
+  for (u32 n = s1 - s0; n; --n) {
+    const TcQuad sc = s;
+    const bool more = f.a & (1u << 25);  // another step of this vertex
+    const plane_t p0 = planes(f.a), p1 = planes(f.b), p2 = planes(f.c), p3 = planes(f.d);
+    const u32 here = row;
+    j = more ? j + 1 : 0;
+    row += more ? 0 : ROW;
+    // one step past the last one read here is still inside the areas (the
+    // tables' next part; the event chunks behind the labels)
+    f = *++fan;
+    if (j < NEAR) {
+      s = *reinterpret_cast<const TcQuad *>(T + row + 16 * j);
+    } else {
+      s = *ft;
+      ft += K::NG;
+    }
+    __syncwarp(mask);
+    PL::acc(a, sc.a, p0);
+    PL::acc(a, sc.b, p1);
+    PL::acc(a, sc.c, p2);
+    PL::acc(a, sc.d, p3);
+    any |= sc.a | sc.b | sc.c | sc.d;
+    if (!more) {
+#pragma unroll
+      for (u32 i = 0; i < K::PP; ++i) a[i] |= tc_bitmask(v, K::PP * part + i) & ~any;
+      *reinterpret_cast<plane_t *>(L + here) = PL::out(a);
+#pragma unroll
+      for (u32 i = 0; i < K::PP; ++i) a[i] = 0;
+      ++v;
+      any = 0;
+    }
+  }
+}
+
+// Thread t's planes, group and half-diamond (half > 1: none).
+template <class K>
+__device__ __forceinline__ void tc_sl_label_thread(u32 t, u32 &half, u32 &g, u32 &pair) {
+  pair = t % K::PS;
+  g = (t / K::PS) % K::NG;
+  half = t / (K::PS * K::NG);
+}
+__device__ __forceinline__ constexpr u32 tc_lanes(u32 n) { return n >= 32 ? 0xffffffffu : (1u << n) - 1u; }
+
+template <class K>
+__device__ __forceinline__ void tc_sl_labels_halves(const TcSlMem &m, u32 t) {
+  u32 half, g, pair;
+  tc_sl_label_thread<K>(t, half, g, pair);
+  if (half < 2)
+    tc_sl_label_run<K>(m, g, pair, half * m.tab[0], (half + 1) * m.tab[0], half * K::H, half * m.tab[9],
+                       tc_lanes(2 * K::PS * K::NG));
+}
+template <class K>
+__device__ __forceinline__ void tc_sl_labels_middle(const TcSlMem &m, u32 t) {
+  u32 half, g, pair;
+  tc_sl_label_thread<K>(t, half, g, pair);
+  if (half == 0)
+    tc_sl_label_run<K>(m, g, pair, 2 * m.tab[0], m.tab[8], 2 * K::H, 2 * m.tab[9], tc_lanes(K::PS * K::NG));
+}
+
+// ---- tiles ----
+// Bytes c = 0..3 of the words p[0..7] as four 8 x 8 bit matrices, transposed:
+// byte c of word r gets bit s of p[s]'s byte c, bit r.
+__device__ __forceinline__ void tc_transpose8(u32 (&p)[8]) {
+#pragma unroll
+  for (u32 j = 4, mk = 0x0F0F0F0Fu; j; j >>= 1, mk ^= mk << j) {
+#pragma unroll
+    for (u32 r = 0; r < 8; ++r)
+      if (!(r & j)) {
+        const u32 x = ((p[r] >> j) ^ p[r + j]) & mk;
+        p[r + j] ^= x;
+        p[r] ^= x << j;
+      }
+  }
+}
+
+template <class K>
+__device__ __forceinline__ void tc_sl_tiles(const TcSlMem &m, u32 t) {
+  for (u32 k = t; k < K::V * K::NG; k += K::T) {
+    TcQuad *const q = reinterpret_cast<TcQuad *>(m.lab + k * K::TW);
+    const TcQuad x = q[0], y = q[1];
+    u32 lo[8] = {x.a, x.b, x.c, x.d, y.a, y.b, y.c, K::NPL > 7 ? y.d : 0u};
+    tc_transpose8(lo);
+    if constexpr (K::LB == 1) {
+      q[0] = TcQuad{lo[0], lo[1], lo[2], lo[3]};
+      q[1] = TcQuad{lo[4], lo[5], lo[6], lo[7]};
+    } else {  // planes 8 and 9: two more bits per label
+      const TcQuad z = q[2];
+      u32 h[8] = {z.a, K::NPL > 9 ? z.b : 0u, 0, 0, 0, 0, 0, 0};
+      tc_transpose8(h);
+      u32 o[16];
+#pragma unroll
+      for (u32 r = 0; r < 8; ++r) {  // bytes 0, 1 and bytes 2, 3 with their high bytes
+        o[r] = (lo[r] & 0xFFu) | ((h[r] & 0xFFu) << 8) | ((lo[r] & 0xFF00u) << 8) | ((h[r] & 0xFF00u) << 16);
+        o[8 + r] = ((lo[r] >> 16) & 0xFFu) | (((h[r] >> 16) & 0xFFu) << 8) | (((lo[r] >> 24) & 0xFFu) << 16) |
+                   (h[r] & 0xFF000000u);
+      }
+#pragma unroll
+      for (u32 r = 0; r < 4; ++r) q[r] = TcQuad{o[4 * r], o[4 * r + 1], o[4 * r + 2], o[4 * r + 3]};
+    }
+  }
+}
+
+#ifndef TC_SL_EMULATE
+template <class K>
+__device__ __forceinline__ void tc_sl_events(const TcSlMem &m, u32 t) {
+  const TcTranspose transpose(t & 31u);
+  u32 *p = m.ev + (t >> 5) * TC_SL_GROUP + (t & 31u);
+  u32 *const end = m.ev + m.tab[2] * K::NG * TC_SL_GROUP;
+  for (; p < end; p += K::NG * TC_SL_GROUP) *p = transpose(*p);
+}
+#endif
+
+// ---- trees: one instance per thread ----
+template <u32 LB>
+struct TcSlLab;
+template <>
+struct TcSlLab<1> {
+  typedef u8 T;
+};
+template <>
+struct TcSlLab<2> {
+  typedef u16 T;
+};
+
+// One thread's labels, event words and region parents.
+template <class K>
+struct TcSlInst {
+  typedef typename TcSlLab<K::LB>::T lab_t;
+  static constexpr u32 TOP = K::LB == 1 ? 0x80u : 0x8000u;
+  static constexpr u32 LOW = K::EVEN && K::TWTOP ? TOP - 1u : 2u * TOP - 1u;
+  static constexpr u32 ROW = K::T;  // labels per vertex
+  lab_t *l;
+  const u32 *ev;
+  u8 *par;
+  u32 *tw;
+  __device__ __forceinline__ TcSlInst(const TcSlMem &m, u32 t) {
+    constexpr u32 WR = K::TW * K::NG;
+    const u32 i = tc_sl_instance<K>(t);
+    l = reinterpret_cast<lab_t *>(m.lab + t % WR) + t / WR;
+    ev = m.ev + (i >> 5) * TC_SL_GROUP + (i & 31u);
+    par = reinterpret_cast<u8 *>(m.x) + t;
+    tw = m.x + K::PAR_WORDS + t;
+  }
+  __device__ __forceinline__ u32 *event_word(u32 v) const {
+    return const_cast<u32 *>(ev) + (v >> 5) * (K::NG * TC_SL_GROUP);
+  }
+  // label start x is no root any more
+  __device__ __forceinline__ void drop(u32 x) const { *event_word(x) &= ~(1u << (x & 31u)); }
+  // region of root x: the roots before it (rank kept per chunk in the first
+  // join chunks)
+  __device__ __forceinline__ u32 region(u32 x) const {
+    return event(K::NCB + (x >> 5)) + (u32)__popc(event(x >> 5) & ((1u << (x & 31u)) - 1u));
+  }
+  __device__ __forceinline__ u32 raw(u32 v) const { return l[v * ROW]; }
+  __device__ __forceinline__ void set(u32 v, u32 x) const { l[v * ROW] = (lab_t)x; }
+  __device__ __forceinline__ u32 lab(u32 v) const { return raw(v) & LOW; }
+  __device__ __forceinline__ u32 event(u32 chunk) const { return ev[chunk * (K::NG * TC_SL_GROUP)]; }
+  __device__ __forceinline__ void set_event(u32 chunk, u32 w) const {
+    const_cast<u32 *>(ev)[chunk * (K::NG * TC_SL_GROUP)] = w;
+  }
+  __device__ __forceinline__ u32 root(u32 x) const {
+    u32 y = lab(x);
+    while (y != x) {
+      x = y;
+      y = lab(x);
+    }
+    return x;
+  }
+  // Whether vertex x's label started in the upper half-diamond; starts: the
+  // middle row's vertices that start a label themselves (their entries may be
+  // links by now).
+  __device__ __forceinline__ u32 upper(u32 x, u64 starts) const {
+    if (x >= 2 * K::H) x = (starts >> (x - 2 * K::H)) & 1ull ? x : lab(x);
+    return x - K::H < K::H ? 1u : 0u;
+  }
+  __device__ __forceinline__ u64 middle_starts() const {
+    constexpr u32 c = 2 * K::H / 32, sh = 2 * K::H % 32;
+    u64 b = event(c) >> sh;
+    if constexpr (c + 1 < K::NCB) b |= (u64)event(c + 1) << (32 - sh);
+    if constexpr (c + 2 < K::NCB) b |= sh ? (u64)event(c + 2) << (64 - sh) : 0ull;
+    return b;
+  }
+  // root of vertex x's set and the twist of the path to it
+  __device__ __forceinline__ u32 root_twist(u32 x, u32 &q) const {
+    for (;;) {
+      const u32 e = raw(x), y = e & LOW;
+      if (y == x) return x;
+      if constexpr (K::TWTOP)
+        q ^= (e & TOP) ? 1u : 0u;
+      else
+        q ^= (tw[(x >> 5) * K::T] >> (x & 31u)) & 1u;
+      x = y;
+    }
+  }
+  __device__ __forceinline__ void link(u32 hi, u32 lo, u32 q) const {
+    drop(hi);
+    if constexpr (K::TWTOP) {
+      set(hi, lo | (q ? TOP : 0u));
+    } else {
+      set(hi, lo);
+      if (q) tw[(hi >> 5) * K::T] |= 1u << (hi & 31u);
+    }
+  }
+};
+
+// Joins of the event chunks [c0, c1) without parity.  The next event and its
+// two labels are loaded before the present join's roots are known (a label
+// read early is still a label of the same set).
+template <class K>
+__device__ __forceinline__ void tc_sl_joins(const TcSlInst<K> &I, const u32 *site, u32 c0, u32 c1) {
+  u32 c = c0, w = 0;
+  while (w == 0 && c < c1) w = I.event(K::NCB + c++);
+  if (w == 0) return;
+  u32 s = site[32u * (c - 1u) + (u32)__ffs(w) - 1u];
+  w &= w - 1u;
+  u32 na = I.raw(s & 0xFFFFu), nb = I.raw(s >> 16);
+  for (;;) {
+    u32 a = na, b = nb, pa, pb;
+    while (w == 0 && c < c1) w = I.event(K::NCB + c++);
+    const bool more = w != 0;
+    if (more) {
+      s = site[32u * (c - 1u) + (u32)__ffs(w) - 1u];
+      w &= w - 1u;
+      na = I.raw(s & 0xFFFFu);
+      nb = I.raw(s >> 16);
+    }
+    do {
+      pa = a;
+      pb = b;
+      a = I.raw(pa);
+      b = I.raw(pb);
+    } while (a != pa || b != pb);
+    if (a != b) {
+      const u32 hi = a < b ? b : a;
+      I.set(hi, a < b ? a : b);
+      I.drop(hi);
+    }
+    if (!more) return;
+  }
+}
+
+// The middle row's joins of even degree, with parity: odd1 / odd2 receive
+// labels of the first and last set found to hold an odd antipodal cycle.
+template <class K>
+__device__ __forceinline__ void tc_sl_joins_twisted(const TcSlInst<K> &I, const u32 *site, u32 c0, u32 c1,
+                                                    u32 &odd1, u32 &odd2) {
+  const u64 starts = I.middle_starts();
+  u32 c = c0, w = 0;
+  for (;;) {
+    while (w == 0) {
+      if (c == c1) return;
+      w = I.event(K::NCB + c++);
+    }
+    const u32 s = site[32u * (c - 1u) + (u32)__ffs(w) - 1u];
+    w &= w - 1u;
+    const u32 v = s & 0xFFFFu, u = (s >> 16) & 0x7FFFu;
+    // parity asked for, relative to the halves of the two labels
+    u32 q = (s >> 31) ^ I.upper(v, starts) ^ I.upper(u, starts);
+    const u32 ra = I.root_twist(v, q), rb = I.root_twist(u, q);
+    if (ra != rb) {
+      I.link(ra < rb ? rb : ra, ra < rb ? ra : rb, q);
+    } else if (q) {
+      if (odd1 == ~0u) odd1 = ra;
+      odd2 = ra;
+    }
+  }
+}
+
+// Joins, regions and the region tree of one instance.  Returns the number of
+// regions R (0: failed, err set) with their parents in I.par (par[r] < r,
+// r >= 1) and the region the tree is rooted at; star: every oval is
+// outermost.
+template <class K>
+__device__ __forceinline__ u32 tc_sl_regions(const TcSlMem &m, const TcSlInst<K> &I, u32 &root, bool &star,
+                                             u32 &err) {
+  const u32 *const tab = m.tab;
+  const u32 *const site = tab + tab[5];
+  const u32 nc1 = tab[1], nc = tab[2] - K::NCB;
+  u32 rv = ~0u;  // a label of the root's set
+  if constexpr (K::EVEN) {
+#pragma unroll
+    for (u32 w = 0; w < K::TWWORDS; ++w) I.tw[w * K::T] = 0;
+    tc_sl_joins<K>(I, site, 0, nc1 + 1);
+    u32 odd2 = ~0u;
+    tc_sl_joins_twisted<K>(I, site, nc1 + 1, nc, rv, odd2);
+    if (rv == ~0u || I.root(rv) != I.root(odd2)) {  // exactly one odd set
+      err |= TC_ERR_INTERNAL;
+      return 0;
+    }
+    rv = I.root(rv);
+  } else {
+    tc_sl_joins<K>(I, site, 0, nc);
+    // the pseudoline's region: both ends of a crossed boundary edge in one
+    // region; the near end of a crossed edge is in the region of the far end
+    // of the one before
+    const u32 *const be = tab + tab[7];
+    u32 prev = I.root(be[0] & 0xFFFFu);
+    bool two = false;
+    for (u32 w = I.event(K::NCB + nc1); w; w &= w - 1u) {
+      const u32 a = I.root(be[(u32)__ffs(w) - 1u] >> 16);
+      if (a == prev) {
+        two |= rv != ~0u && rv != a;
+        rv = a;
+      }
+      prev = a;
+    }
+    if (two) {
+      err |= TC_ERR_INTERNAL;
+      return 0;
+    }
+    if (rv == ~0u) {
+      err |= TC_ERR_INTERNAL;
+      return 0;
+    }
+  }
+  // regions in the order of their smallest label: the starts that are still
+  // roots, counted chunk by chunk (the join chunks are used up)
+  u32 R = 0;
+#pragma unroll
+  for (u32 c = 0; c < K::NCB; ++c) {
+    I.set_event(K::NCB + c, R);
+    R += (u32)__popc(I.event(c));
+  }
+  if (R > K::RMAX) {
+    err |= TC_ERR_OVERFLOW;
+    return 0;
+  }
+  root = I.region(rv);
+  // the tree hanging from region 0: the parent of region r is the region of
+  // the first earlier neighbour of its smallest label's vertex
+  const u32 *const vd = tab + tab[4];
+  star = true;
+  bool bad = false;
+  u32 c = 0, w = 0;
+  for (u32 r = 0; r < R; ++r) {
+    while (w == 0) w = I.event(c++);
+    const u32 v = 32u * (c - 1u) + (u32)__ffs(w) - 1u;
+    w &= w - 1u;
+    if (r) {
+      const u32 d = vd[v], p = I.region(I.root(d & 0x7FFFu));
+      bad |= !(d & 0x8000u) || p >= r;  // no earlier neighbour, or not a tree
+      I.par[r * K::T] = (u8)p;
+      star &= p == (r == root ? 0u : root);
+    }
+  }
+  if (bad) {
+    err |= TC_ERR_INTERNAL;
+    return 0;
+  }
+  return R;
+}
+
+// Canonical code of a region tree of at most 32 regions that is no star.
+// adj: this thread's children masks, word r at adj[r * T] (over the label
+// area, free by then).  The tree is re-rooted by reversing the path from the
+// root to region 0; AHU codes follow for the regions with children, those off
+// the path by falling index (children have larger ones), then along the path.
+// A code is left-aligned in 64 bits with its length in the low byte (at most
+// 56 bits: fewer than 29 ovals); a leaf's code '10' is the smallest.
+template <class K>
+__device__ __forceinline__ u64 tc_sl_tree_code(const TcSlInst<K> &I, u32 *adj, u32 R, u32 root, u32 &err) {
+  static_assert(2 * K::RMAX <= 58 && K::RMAX * K::T <= K::LABW, "narrow tree codes");
+  for (u32 r = 0; r < R; ++r) adj[r * K::T] = 0;
+  u32 internal = 0, path = 0;
+  for (u32 r = 1; r < R; ++r) {
+    const u32 p = I.par[r * K::T];
+    adj[p * K::T] |= 1u << r;
+    internal |= 1u << p;
+  }
+  for (u32 x = root, prev = 32;;) {  // reverse the path root -> 0
+    const u32 up = I.par[x * K::T];
+    u32 kids = adj[x * K::T];
+    if (prev < 32) kids &= ~(1u << prev);
+    if (x) kids |= 1u << up;
+    adj[x * K::T] = kids;
+    internal = kids ? internal | (1u << x) : internal & ~(1u << x);
+    path |= 1u << x;
+    I.par[x * K::T] = (u8)prev;
+    if (x == 0) break;
+    prev = x;
+    x = up;
+  }
+  u64 node[(K::RMAX + 1) / 2];  // codes of the regions with children, by rank among them
+  auto rank = [&](u32 x) -> u32 { return (u32)__popc(internal & ((1u << x) - 1u)); };
+  for (u32 off = internal & ~path, x = 0;;) {
+    if (off) {
+      x = 31u - (u32)__clz(off);
+      off &= ~(1u << x);
+    } else if (path) {  // from region 0 towards the root
+      x = (path & 1u) ? 0u : (u32)I.par[x * K::T];
+      path &= ~(1u << x);
+      if (!((internal >> x) & 1u)) continue;
+    } else {
+      break;
+    }
+    const u32 kids = adj[x * K::T];
+    u64 v = 0;
+    u32 len = 0;
+    for (u32 big = kids & internal; big;) {  // larger codes first
+      u32 best = 0;
+      u64 bv = 0;
+      for (u32 y = big; y; y &= y - 1u) {
+        const u32 k = (u32)__ffs(y) - 1u;
+        const u64 cv = node[rank(k)];
+        if (cv > bv) {
+          bv = cv;
+          best = k;
+        }
+      }
+      v |= (bv & ~255ull) >> len;
+      len += (u32)bv & 255u;
+      big &= ~(1u << best);
+    }
+    const u32 nl = 2u * (u32)__popc(kids & ~internal);
+    if (nl) v |= (0xAAAAAAAAAAAAAAAAull & ~(~0ull >> nl)) >> len;
+    len += nl;
+    if (x == root) {
+      if (len != 2 * (R - 1)) {
+        err |= TC_ERR_INTERNAL;
+        return 0;
+      }
+      return (1ull << len) | (v >> (64u - len));
+    }
+    node[rank(x)] = (1ull << 63) | (v >> 1) | (u64)(len + 2u);
+  }
+  err |= TC_ERR_INTERNAL;
+  return 0;
+}
+
+// Code of thread t's instance from tc_sl_regions' result (all zero if it
+// failed).  The tree codes work over the label area, so every thread of the
+// block must be done with tc_sl_regions.
+template <class K>
+__device__ __forceinline__ void tc_sl_finish(const TcSlMem &m, const TcSlInst<K> &I, u32 t, u32 R, u32 root,
+                                             bool star, u32 &err, u64 *code) {
+  if constexpr (K::WIDE) {
+#pragma unroll
+    for (u32 w = 0; w < K::CW; ++w) code[w] = 0;
+    if (R == 0) return;
+    const TcScratch<K> S{m.lab + t};
+    for (u32 r = 1; r < R; ++r) *S.byte(K::OFF_WPAR, r) = I.par[r * K::T];
+    tc_wide_tree_code(S, R, (int)root, err, code);
+  } else {
+    const u32 q = 2 * (R - 1);
+    code[0] = R == 0 ? 0ull
+              : star ? (1ull << q) | (0xAAAAAAAAAAAAAAAAull & ((1ull << q) - 1))
+                     : tc_sl_tree_code<K>(I, m.lab + t, R, root, err);
+  }
+}
+
+#ifndef TC_SL_EMULATE
+// The whole classification: sg is the sign vector of instance t of the block,
+// code receives that of instance tc_sl_instance<K>(t) (zero if it failed).
+// All T threads call it, after a barrier behind the last use of the areas.
+template <class K>
+__device__ __forceinline__ void tc_sl_classify(const TcSlMem &m, const TcSig<K::W> &sg, u32 t, u32 &err,
+                                               u64 *code) {
+  tc_sl_clear<K>(m, t);
+  tc_sl_planes<K>(m, sg, t);
+  __syncthreads();
+  tc_sl_logic<K>(m, t);
+  __syncthreads();
+  tc_sl_labels_halves<K>(m, t);
+  if constexpr (2 * K::PS * K::NG <= 32) __syncwarp();  // one warp holds both halves
+  else __syncthreads();
+  tc_sl_labels_middle<K>(m, t);
+  __syncthreads();
+  tc_sl_tiles<K>(m, t);
+  tc_sl_events<K>(m, t);
+  __syncthreads();
+  const TcSlInst<K> I(m, t);
+  u32 root = 0;
+  bool star = false;
+  const u32 R = tc_sl_regions<K>(m, I, root, star, err);
+  __syncthreads();  // tree codes are made over the label area
+  tc_sl_finish<K>(m, I, t, R, root, star, err, code);
+}
+#endif

@@ -1,0 +1,52 @@
+"""The bit-sliced classification (tc_sliced.cuh) compiled for the host, all
+threads of a block phase by phase, against the oracle (no GPU needed)."""
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+import tcurve_inputs as ti
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+CUDA = "/usr/local/cuda"
+
+
+@pytest.fixture(scope="module")
+def sliced_exe(tmp_path_factory):
+    if not shutil.which("g++") or not os.path.exists(os.path.join(CUDA, "include", "cuda_runtime.h")):
+        pytest.skip("needs g++ and the CUDA headers")
+    csrc = os.path.join(ROOT, "paper_2604_09221_gb300", "csrc")
+    out = {}
+    for groups in (2, 4):
+        exe = tmp_path_factory.mktemp("sliced") / f"run{groups}"
+        cmd = ["g++", "-std=c++17", "-O1", "-w", f"-DTC_SL_GROUPS={groups}", f"-I{csrc}",
+               f"-I{os.path.join(HERE, 'host')}", f"-I{os.path.join(ROOT, 'oracle')}",
+               f"-I{CUDA}/include", "-o", str(exe), os.path.join(HERE, "host", "run_sliced_sweep.cpp"),
+               "-x", "c", os.path.join(ROOT, "oracle", "tcurve_oracle.c"), "-x", "none",
+               f"-L{CUDA}/lib64", f"-Wl,-rpath,{CUDA}/lib64", "-lcudart", "-lpthread"]
+        subprocess.run(cmd, check=True, capture_output=True)
+        out[groups] = exe
+    return out
+
+
+@pytest.mark.parametrize("d", list(range(1, 17)))
+def test_sliced_sweep_on_the_host(sliced_exe, tmp_path, d):
+    """Random and special sign vectors on the standard, (d >= 3) a regular and
+    (d >= 2) the fan triangulation, whose origin has more earlier neighbours
+    than a vertex's row of label planes holds takes for: one- and two-byte
+    labels, both back ends, blocks of 64 and 128 sign vectors, every area of
+    exactly the kernels' size."""
+    cases = [("standard", ti.standard_triangulation(d))]
+    if d >= 3:
+        cases.append(("regular", ti.regular_triangulation(d, seed=300 + d)))
+    if d >= 2:
+        cases.append(("fan", ti.fan_triangulation(d)))
+    for name, edges in cases:
+        np.savetxt(tmp_path / "tri.txt", edges, fmt="%d")
+        for groups, exe in sliced_exe.items():
+            out = subprocess.run([str(exe), str(d), str(tmp_path / "tri.txt"), "3"],
+                                 capture_output=True, text=True)
+            assert out.returncode == 0, (name, groups, out.stdout + out.stderr)
