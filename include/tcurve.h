@@ -130,9 +130,11 @@ ts_status ts_real_schemes(const ts_tri *tri, const uint64_t *signs, uint64_t n,
  *     no global scratch).  ts_real_schemes and ts_enumerate; batches run
  *     it as the warp tile of their fused launch (ts_batch_set_fused_tile);
  *     ts_enumerate_noalloc runs the table-driven family.
- *   TS_KERNEL_AUTO (default): specialised for ts_enumerate (but not for
- *     TS_ENUM_SPLITMIX) when 4 <= d <= 9, table-driven otherwise or if the
- *     specialised kernel cannot be built. */
+ *     Sweeps of at least 2^19 masks that differ in the middle row block by
+ *     block (4 <= d <= 9, not TS_ENUM_SPLITMIX) share the half-diamonds of
+ *     each block.
+ *   TS_KERNEL_AUTO (default): table-driven; batches may specialise small
+ *     degrees (ts_batch_info). */
 #define TS_KERNEL_AUTO 0
 #define TS_KERNEL_TABLE 1
 #define TS_KERNEL_SPECIALIZED 2
@@ -165,9 +167,9 @@ ts_status ts_set_scratch(ts_tri *tri, int where);
 ts_status ts_set_occupancy(ts_tri *tri, int blocks_per_sm);
 
 /* Build the specialised kernels now (NVRTC compile and module load on the
- * current device; about a second).  Call it before capturing launches of
- * this triangulation in a CUDA graph, since the first specialised launch
- * otherwise compiles.  Returns TS_ECUDA if compilation or loading fails
+ * current device; about a second), for TS_KERNEL_SPECIALIZED.  Call it before
+ * capturing launches of such a triangulation in a CUDA graph, since the first
+ * specialised launch otherwise compiles.  Returns TS_ECUDA if compilation or loading fails
  * (ts_specialized_log then holds the compiler log), TS_EUNSUPPORTED for
  * d > 9. */
 ts_status ts_prepare(ts_tri *tri);
@@ -216,9 +218,8 @@ ts_status ts_hist_clear(ts_hist *hist, void *stream);
  * Except with TS_ENUM_SPLITMIX, m(hi-1) < 2^|A| (a bound only for d <= 9
  * and, with TS_ENUM_REDUCED, d = 10).  Persistent launches on `stream`
  * (whole blocks of middle-row patterns, and a ragged head and tail mask by
- * mask); asynchronous.  With TS_ENUM_FLIP the specialised kernels take a
- * block of masks and the block of their complements (every bit flipped)
- * together, evaluating the complements of half of them instead: the global
+ * mask); asynchronous.  With TS_ENUM_FLIP whole blocks are swept with the
+ * blocks of their complements (every bit flipped) together, evaluating the complements of half of them instead: the global
  * sign flip keeps the curve, so the histogram is the one of the masks m(k).
  * Failed instances are counted, not inserted, and set the histogram's
  * error word. */

@@ -17,9 +17,10 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libtcurve.so")
 SOURCES = ["host.cpp", "kernels.cu", "warp_kernels.cu", "jit.cpp", "noalloc.cu", "batch.cu", "sliced_jobs.cu",
-           "fused.cu", "int_peak.cu"]
+           "block_sweep.cu", "fused.cu", "int_peak.cu"]
 HEADERS = ["engine.h", "tc_layout.h", "tc_runtime.cuh", "tc_table_sweep.cuh", "tc_warp_sweep.cuh",
-           "tc_stage.cuh", "tc_sliced.cuh", "jit_kernels.cuh",
+           "tc_stage.cuh", "tc_sliced.cuh", "tc_block_sweep.cuh",
+           "jit_kernels.cuh",
            os.path.join("..", "..", "include", "tcurve.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -139,6 +139,13 @@ cudaError_t launch_real_schemes(const ts_tri *tri, const uint64_t *signs, uint64
 // allow_global = false keeps the scratch in shared memory (no allocation).
 cudaError_t launch_enumerate(const ts_tri *tri, uint64_t lo, uint64_t hi, uint32_t flags,
                              ts_hist *hist, cudaStream_t stream, bool allow_global = true);
+// The bit-sliced block sweep (block_sweep.cu), 4 <= d <= 9: whether a range
+// holds enough whole blocks of middle-row patterns, which it is (sweep indexes
+// [a, b)), and the sweep of such a range.
+constexpr uint64_t kBlockSweepMin = 1ull << 19;
+bool block_range(const ts_tri *tri, uint64_t lo, uint64_t hi, uint32_t flags, uint64_t *a, uint64_t *b);
+cudaError_t launch_block_sweep(const ts_tri *tri, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *hist,
+                               cudaStream_t stream);
 // Warp-per-instance kernels (warp_kernels.cu, TS_KERNEL_WARP): the whole
 // scratch in shared memory, so they allocate nothing either.
 cudaError_t launch_real_schemes_warp(const ts_tri *tri, const uint64_t *signs, uint64_t n,

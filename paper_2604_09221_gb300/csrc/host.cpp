@@ -566,19 +566,11 @@ int ts_sign_words(const ts_tri *t) { return t ? t->sw : 0; }
 int ts_code_words(const ts_tri *t) { return t ? t->cw : 0; }
 
 namespace {
-// Kernel choice (AUTO): the specialised block sweep for sweeps whose masks
-// share their high bits; the table-driven (bit-sliced) kernels for queries
-// and sampled sweeps, which the specialised per-mask kernels lose to (d = 7,
-// random sign vectors: 1.8 against 4.2e9 schemes/s), for d < 4, where a block
-// has fewer masks than a warp has lanes, and when specialisation is
-// unavailable.
-bool want_specialised(ts_tri *t, bool sweep) {
-  if (t->kernel == TS_KERNEL_TABLE || t->kernel == TS_KERNEL_WARP || t->d > kMaxSpecialized)
-    return false;
-  if (t->kernel == TS_KERNEL_SPECIALIZED) return true;
-  if (!sweep || t->d < 4) return false;
-  return jit_prepare(t) == cudaSuccess;
-}
+// Kernel choice: the specialised kernels only when asked for.  AUTO takes the
+// table-driven (bit-sliced) kernels: on random sign vectors at d = 7 they
+// classify 4.2e9/s against the specialised query kernel's 1.8e9, and the
+// bit-sliced block sweep beats the specialised one at every degree.
+bool want_specialised(const ts_tri *t) { return t->kernel == TS_KERNEL_SPECIALIZED; }
 }  // namespace
 
 ts_status ts_real_schemes(const ts_tri *tc, const uint64_t *signs, uint64_t n, uint64_t *codes,
@@ -588,7 +580,7 @@ ts_status ts_real_schemes(const ts_tri *tc, const uint64_t *signs, uint64_t n, u
   ts_tri *t = const_cast<ts_tri *>(tc);  // only the lazily compiled kernel cache changes
   if (t->kernel == TS_KERNEL_WARP)
     return cuda_status(launch_real_schemes_warp(t, signs, n, codes, (cudaStream_t)stream));
-  if (want_specialised(t, false))
+  if (want_specialised(t))
     return cuda_status(launch_real_schemes_jit(t, signs, n, codes, (cudaStream_t)stream));
   return cuda_status(launch_real_schemes(t, signs, n, codes, (cudaStream_t)stream));
 }
@@ -788,7 +780,7 @@ ts_status ts_enumerate(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags
   ts_tri *tm = const_cast<ts_tri *>(t);
   if (tm->kernel == TS_KERNEL_WARP)
     return cuda_status(launch_enumerate_warp(tm, lo, hi, flags, h, (cudaStream_t)stream));
-  if (want_specialised(tm, !(flags & TS_ENUM_SPLITMIX)))
+  if (want_specialised(tm))
     return cuda_status(launch_enumerate_jit(tm, lo, hi, flags, h, (cudaStream_t)stream));
   return cuda_status(launch_enumerate(t, lo, hi, flags, h, (cudaStream_t)stream));
 }

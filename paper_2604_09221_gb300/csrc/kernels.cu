@@ -448,8 +448,15 @@ cudaError_t real_schemes_d(const ts_tri *t, const uint64_t *signs, uint64_t n, u
 template <int D>
 cudaError_t enumerate_d(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *h,
                         cudaStream_t st, bool allow_global) {
-  return allow_global && global_scratch(t) ? enumerate_dg<D, true>(t, lo, hi, flags, h, st)
-                                           : enumerate_sliced<D>(t, lo, hi, flags, h, st);
+  if (allow_global && global_scratch(t)) return enumerate_dg<D, true>(t, lo, hi, flags, h, st);
+  // whole blocks of middle-row patterns by the block sweep, the ragged ends
+  // (or everything, if there are few blocks) mask by mask
+  uint64_t a = hi, b = hi;
+  cudaError_t e = cudaSuccess;
+  if (block_range(t, lo, hi, flags, &a, &b)) e = launch_block_sweep(t, a, b, flags, h, st);
+  if (e == cudaSuccess && lo < a) e = enumerate_sliced<D>(t, lo, a, flags, h, st);
+  if (e == cudaSuccess && b < hi) e = enumerate_sliced<D>(t, b, hi, flags, h, st);
+  return e;
 }
 
 }  // namespace

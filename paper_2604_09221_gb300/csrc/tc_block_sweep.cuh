@@ -1,0 +1,441 @@
+// tc_block_sweep.cuh -- exhaustive sweeps in whole blocks of middle-row
+// patterns, bit-sliced twice (d <= 9; block_sweep.cu).
+//
+// The masks of a block share their high bits (the lattice points off the
+// x-axis); its 2^ib masks differ in the middle row only.  No edge of
+// T^diamond crosses the x-axis, so the two half-diamonds depend on the high
+// bits alone, and what they leave to the middle row is small: the components
+// ("comps") that touch it, which of them are next to which middle vertex with
+// which sign, and the tree they hang in.  A thread block takes 128 high parts:
+//
+//   halves   the half-diamonds of 128 high parts by the phases of
+//            tc_sliced.cuh, then one high part per thread: the half joins, and
+//            a record of the comps (TcSb below)
+//   middle   32 middle-row patterns of one high part per thread, one bit each.
+//            The open comps (about d + 1 of them) are the nodes of a graph;
+//            the middle row is walked once, joining all nodes of a run of one
+//            sign, and the graph is closed transitively (Warshall): a region
+//            is a class of nodes, or a closed comp.  The root needs no
+//            orientation parity: a region X other than the root is a disk with
+//            holes, so chi(X) + (its neighbours in the region tree) is even,
+//            and it is odd for the root (one Moebius band more, or the
+//            pseudoline's two sides), where chi counts label starts minus join
+//            events.  Both are sums over nodes, kept modulo 2 as bit planes.
+//            Patterns whose regions all border the root (a star) are counted
+//            by their number of regions; the codes of the others are made one
+//            by one from their classes.
+//
+// Every middle vertex has half-diamond neighbours of both signs: the triangle
+// over an edge of the x-axis has its apex at height 1, and the reflections
+// (x, 1) and (x, -1) have opposite signs (Eq. 2).  So no region lies in the
+// middle row alone, and every run has a node.
+//
+// High parts with more than K::NB open comps or more than 32 comps (none on
+// the seeded regular triangulations) take the per-mask phases of tc_sliced.cuh.
+#pragma once
+
+#include "tc_sliced.cuh"
+
+// Traits: TcSlK's, two sizes of the middle phase (nodes), the areas.
+template <int D_>
+struct TcSbK : TcSlK<D_, 4> {
+  typedef TcSlK<D_, 4> Base;
+  static constexpr u32 D = D_, M = 2 * D_ + 1;  // middle vertices
+  static constexpr u32 NA = D_ <= 8 ? D_ + 1 : 13, NB = D_ + 6 < 16 ? D_ + 6 : 16;
+  // record of a high part (words, one column per thread)
+  static constexpr u32 R_HDR = 0,          // comps | nodes << 8 | closed comps << 16 | star impossible << 24
+                                           // | valid << 25 | corner edge signs << 26, 27
+                       R_NODE = 1,         // nodes that must be in the root | chi parities << 16
+                       R_ADJ = 2,          // per middle vertex: nodes next to it with sigma 0 | with sigma 1 << 16
+                       R_TOG = R_ADJ + M,  // per middle vertex 4 bits: chi changes by an odd number; bit
+                                           // sigma + 2 * (same sign as the vertex before)
+                       R_NPAR = R_TOG + (4 * M + 31) / 32,  // parent of a node (byte): node, 254 closed, 255 none
+                       R_NCOMP = R_NPAR + 4,                // comp of a node (byte)
+                       R_CPAR = R_NCOMP + 4,                // parent of a comp (byte)
+                       R_CNODE = R_CPAR + 8,                // node of a comp (byte; 255: closed)
+                       R_WORDS = R_CNODE + 8;
+  static constexpr u32 T = Base::T;
+  // areas (words): the label area also holds the tree codes' children masks
+  // and parents (32 + 8 words per thread); scratch: M words per thread
+  static constexpr u32 LAB = Base::LABW > 40 * T ? Base::LABW : 40 * T;
+  static constexpr u32 SW = (M > 16 ? M : 16) * T;
+  static constexpr u32 STARS = 48;  // star patterns by number of regions (64-bit counts)
+};
+
+struct TcSbMem {
+  TcSlMem s;     // tables, labels, events, sign planes
+  u32 *chi;      // K::NCB words per thread
+  u32 *rec;      // K::R_WORDS words per thread
+  u32 *scr;      // K::SW words
+  unsigned long long *stars;  // K::STARS counters
+};
+
+template <class K>
+__host__ __device__ constexpr u32 tc_sb_words(u32 chunks, u32 far) {
+  return K::LAB + chunks * K::NG * TC_SL_GROUP + tc_sl_xwords<typename K::Base>(far) + K::NCB * K::T +
+         K::R_WORDS * K::T + K::SW + 2 * K::STARS;
+}
+
+template <class K>
+__device__ __forceinline__ TcSbMem tc_sb_carve(const u32 *tab, u32 *area, u32 chunks, u32 far) {
+  TcSbMem m;
+  m.s.tab = tab;
+  m.s.lab = area;
+  m.s.ev = m.s.lab + K::LAB;
+  m.s.x = m.s.ev + chunks * K::NG * TC_SL_GROUP;
+  m.chi = m.s.x + tc_sl_xwords<typename K::Base>(far);
+  m.rec = m.chi + K::NCB * K::T;
+  m.scr = m.rec + K::R_WORDS * K::T;
+  m.stars = reinterpret_cast<unsigned long long *>(m.scr + K::SW);
+  return m;
+}
+
+template <class K>
+__device__ __forceinline__ u8 *tc_sb_byte(u32 *rec, u32 off, u32 i, u32 t) {
+  return reinterpret_cast<u8 *>(rec + (off + (i >> 2)) * K::T + t) + (i & 3u);
+}
+
+// ---- halves: one high part per thread (thread t: instance
+// tc_sl_instance<K>(t) of the block), after the phases of tc_sliced.cuh up to
+// the tiles.  sig: its mask, middle-row bits zero.
+template <class K>
+__device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
+  typedef TcSlInst<typename K::Base> Inst;
+  const Inst I(m.s, t);
+  const u32 *const tab = m.s.tab;
+  const u32 nc1 = tab[1];
+  // label starts and joins of the half-diamonds only.  The first pair behind
+  // a corner is joined whatever the corner's sign; the corner pair is not.
+  constexpr u32 HB = 2 * K::H;
+  if constexpr (HB % 32 != 0) I.set_event(HB / 32, I.event(HB / 32) & ((1u << (HB % 32)) - 1u));
+  for (u32 c = (HB + 31) / 32; c < K::NCB; ++c) I.set_event(c, 0);
+  const u32 be = (I.event(K::NCB + nc1) | 1u) & ((1u << (2 * K::D - 1)) - 1u);
+  I.set_event(K::NCB + nc1, be);
+  for (u32 c = 0; c < K::NCB; ++c) m.chi[c * K::T + t] = I.event(c);  // label starts, before joins drop some
+  tc_sl_joins<typename K::Base>(I, tab + tab[5], 0, nc1 + 1);
+  // chi of every comp modulo 2, at its root: label starts plus join events
+  auto toggle = [&](u32 r) { m.chi[(r >> 5) * K::T + t] ^= 1u << (r & 31u); };
+  {
+    u32 starts[K::NCB];  // (the starts that are roots keep their own bit)
+#pragma unroll
+    for (u32 c = 0; c < K::NCB; ++c) {
+      starts[c] = m.chi[c * K::T + t] & ~I.event(c);
+      m.chi[c * K::T + t] = I.event(c);
+    }
+#pragma unroll
+    for (u32 c = 0; c < K::NCB; ++c)
+      for (u32 w = starts[c]; w; w &= w - 1u) toggle(I.root(32u * c + (u32)__ffs(w) - 1u));
+    const u32 *const site = tab + tab[5];
+    for (u32 c = 0; c <= nc1; ++c)
+      for (u32 w = I.event(K::NCB + c); w; w &= w - 1u)
+        toggle(I.root(site[32u * c + (u32)__ffs(w) - 1u] & 0xFFFFu));
+  }
+  u32 C = 0;  // comps, numbered by their roots; the join chunks are used up
+#pragma unroll
+  for (u32 c = 0; c < K::NCB; ++c) {
+    I.set_event(K::NCB + c, C);
+    C += (u32)__popc(I.event(c));
+  }
+  u32 *const rec = m.rec + t;
+  rec[K::R_HDR * K::T] = 0;
+  if (C > 32) return;  // not valid: the block's masks one by one
+  // the middle vertices' neighbours: comps next to them by sign, and whether
+  // chi changes by an odd number when the vertex joins: 1 minus the runs of
+  // its same-sign earlier neighbours, for either sign and with or without the
+  // vertex before it
+  u32 open = 0, tog = 0, vi = 0;
+  {
+    u32 m0 = 0, m1 = 0, bits = 0, links = 0, left = 0, n = 0;
+    const TcQuad *f = reinterpret_cast<const TcQuad *>(tab + tab[3]) + 2 * tab[0];
+    for (u32 s = 2 * tab[0]; s < tab[8]; ++s, ++f) {
+      const TcQuad q = *f;
+#pragma unroll
+      for (u32 i = 0; i < 4; ++i) {
+        const u32 e = i == 0 ? q.a : i == 1 ? q.b : i == 2 ? q.c : q.d, u = (e >> 8) & 0xFFFFu;
+        if (u == 0) continue;  // padding: vertex 0 is never next to the middle row
+        links |= ((e >> 30) & 1u) << n;
+        if (u >= 2 * K::H) {
+          left = 1u << n;
+        } else {
+          // sigma of the middle vertex for which the two have one sign
+          const u32 b = ((u32)(sig >> (e & 63u)) ^ (e >> 31) ^ 1u) & 1u;
+          const u32 c = 1u << I.region(I.root(u));
+          m0 |= b ? 0u : c;
+          m1 |= b ? c : 0u;
+          bits |= b << n;
+        }
+        ++n;
+      }
+      if (q.a & (1u << 25)) continue;  // another step of this vertex
+      const u32 all = ((1u << n) - 1u) & ~left;
+#pragma unroll
+      for (u32 k = 0; k < 4; ++k) {
+        const u32 e = ((k & 1u) ? bits : ~bits & all) | ((k & 2u) ? left : 0u);
+        tog |= ((1u + (u32)__popc(e & ~((e << 1) & links))) & 1u) << ((4u * vi + k) & 31u);
+      }
+      rec[(K::R_ADJ + vi) * K::T] = m0;
+      m.scr[vi * K::T + t] = m1;
+      open |= m0 | m1;
+      if ((vi & 7u) == 7u || vi + 1u == K::M) {
+        rec[(K::R_TOG + (vi >> 3)) * K::T] = tog;
+        tog = 0;
+      }
+      ++vi;
+      m0 = m1 = bits = links = left = n = 0;
+    }
+  }
+  const u32 N = (u32)__popc(open);
+  if (N > K::NB) return;
+  // neighbours in node numbers
+  for (u32 v = 0; v < K::M; ++v) {
+    const u32 a = rec[(K::R_ADJ + v) * K::T], b = m.scr[v * K::T + t];
+    u32 x = 0, k = 0;
+    for (u32 o = open; o; o &= o - 1u, ++k) {
+      const u32 c = (u32)__ffs(o) - 1u;
+      x |= (((a >> c) & 1u) | (((b >> c) & 1u) << 16)) << k;
+    }
+    rec[(K::R_ADJ + v) * K::T] = x;
+  }
+  // comps in order: parents, chi, what a star needs
+  auto node_of = [&](u32 c) -> u32 { return (open >> c) & 1u ? (u32)__popc(open & ((1u << c) - 1u)) : 255u; };
+  u32 need = 0, chi = 0, nostar = 0;
+  const u32 *const vd = tab + tab[4];
+  {
+    u32 ch = 0, w = 0;
+    for (u32 c = 0; c < C; ++c) {
+      while (w == 0) w = I.event(ch++);
+      const u32 v = 32u * (ch - 1u) + (u32)__ffs(w) - 1u;
+      w &= w - 1u;
+      const u32 p = c ? I.region(I.root(vd[v] & 0x7FFFu)) : 255u, nc = node_of(c),
+                np = c ? node_of(p) : 255u;
+      *tc_sb_byte<K>(m.rec, K::R_CPAR, c, t) = (u8)p;
+      *tc_sb_byte<K>(m.rec, K::R_CNODE, c, t) = (u8)nc;
+      if (nc != 255u) {
+        *tc_sb_byte<K>(m.rec, K::R_NPAR, nc, t) = (u8)(c == 0 ? 255u : np == 255u ? 254u : np);
+        *tc_sb_byte<K>(m.rec, K::R_NCOMP, nc, t) = (u8)c;
+        chi ^= ((m.chi[(v >> 5) * K::T + t] >> (v & 31u)) & 1u) << nc;
+        need |= c && np == 255u ? 1u << nc : 0u;
+      } else if (c) {  // a closed comp: one more neighbour of its parent
+        if (np == 255u) {
+          nostar = 1;
+        } else {
+          chi ^= 1u << np;
+          need |= 1u << np;
+        }
+      }
+    }
+  }
+  // sigma of each corner for which its half-diamond boundary edge is not
+  // crossed: edge 0 at (d, 0), edge 2d - 1 at (-d, 0)
+  const u32 *const bx = tab + tab[6];
+  const u32 e0 = bx[0], e1 = bx[2 * K::D - 1];
+  const u32 s0 = ((u32)(sig >> ((e0 >> 8) & 63u)) ^ (e0 >> 16)) & 1u;
+  const u32 s1 = ((u32)(sig >> (e1 & 63u)) ^ (e1 >> 16)) & 1u;
+  rec[K::R_NODE * K::T] = need | (chi << 16);
+  rec[K::R_HDR * K::T] = C | (N << 8) | ((C - N) << 16) | (nostar << 24) | (1u << 25) | (s0 << 26) | (s1 << 27);
+}
+
+// ---- middle: 32 patterns per thread ----
+
+// Bit plane of pattern bit j of the 32 patterns of word w.
+__device__ __forceinline__ u32 tc_sb_plane(u32 j, u32 w) {
+  switch (j) {
+    case 0: return 0xAAAAAAAAu;
+    case 1: return 0xCCCCCCCCu;
+    case 2: return 0xF0F0F0F0u;
+    case 3: return 0xFF00FF00u;
+    case 4: return 0xFFFF0000u;
+    default: return (w >> (j - 5u)) & 1u ? ~0u : 0u;
+  }
+}
+
+// Add cnt to key in the block's hash table, or in the device's if that is full.
+template <u32 HASH>
+__device__ __forceinline__ void tc_sb_insert(u64 key, unsigned long long cnt, u64 *hkeys,
+                                             unsigned long long *hcnt, u64 *gkeys, unsigned long long *gcnt,
+                                             u64 gslots, u32 *gerr) {
+  u32 s = tc_hash_slot(key, HASH - 1);
+  for (u32 probe = 0; probe < HASH; ++probe) {
+    unsigned long long *kp = reinterpret_cast<unsigned long long *>(hkeys + s);
+    unsigned long long k = *reinterpret_cast<volatile unsigned long long *>(kp);
+    if (k == 0) k = atomicCAS(kp, 0ull, (unsigned long long)key);
+    if (k == 0 || k == key) {
+      atomicAdd(hcnt + s, cnt);
+      return;
+    }
+    s = (s + 1) & (HASH - 1);
+  }
+  tc_global_add(gkeys, gcnt, gslots, gerr, key, cnt);
+}
+
+// Code of a star: R - 1 ovals, none in another.
+__device__ __forceinline__ u64 tc_sb_star_code(u32 R) {
+  const u32 q = 2 * (R - 1);
+  return (1ull << q) | (0xAAAAAAAAAAAAAAAAull & ((1ull << q) - 1));
+}
+
+// Where the codes of a sweep go.
+struct TcSbOut {
+  u64 *hkeys;
+  unsigned long long *hcnt;
+  u64 *gkeys;
+  unsigned long long *gcnt;
+  u64 gslots;
+  u32 *gerr;
+};
+
+// Word w of the patterns of high part hl (a column of the records), at most
+// NN nodes; ishift: the lowest middle-row bit that varies.
+template <class K, u32 NN>
+__device__ __forceinline__ void tc_sb_middle(const TcSbMem &m, u32 t, u32 hl, u32 w, u32 ishift,
+                                             const TcSbOut &out, u32 &err, unsigned long long &failed) {
+  const u32 *const rec = m.rec + hl;
+  const u32 hdr = rec[K::R_HDR * K::T], N = (hdr >> 8) & 255u, nd = rec[K::R_NODE * K::T];
+  u32 *const tg = m.scr + t;  // chi + degree of the nodes, modulo 2, one plane each
+  u32 conn[NN * (NN - 1) / 2], T[NN], n[NN], first[NN];
+  auto pair = [](u32 a, u32 b) constexpr -> u32 { return b * (b - 1) / 2 + a; };  // a < b
+#pragma unroll
+  for (u32 i = 0; i < NN * (NN - 1) / 2; ++i) conn[i] = 0;
+#pragma unroll
+  for (u32 c = 0; c < NN; ++c) {
+    T[c] = 0;
+    tg[c * K::T] = tc_bitmask(nd, 16 + c);
+  }
+  u32 prev = 0, S = 0, sfirst = 0, togw = 0, adj = 0;
+  for (u32 v = 0; v < K::M; ++v) {
+    const u32 x = v < K::D ? K::D - v : v - K::D;
+    S = x < ishift ? 0u : tc_sb_plane(x - ishift, w);
+    // same sign as the vertex before: left of the origin Eq. 2's constant
+    // |x| mod 2 changes from vertex to vertex, up to (-1, 0) -> (0, 0)
+    const u32 same = v ? ~(S ^ prev ^ (v <= K::D ? ~0u : 0u)) : 0u;
+    adj = rec[(K::R_ADJ + v) * K::T];
+#pragma unroll
+    for (u32 c = 0; c < NN; ++c) {
+      n[c] = (tc_bitmask(adj, c) & ~S) | (tc_bitmask(adj, 16 + c) & S);
+      T[c] = (T[c] & same) | n[c];
+    }
+#pragma unroll
+    for (u32 b = 1; b < NN; ++b)
+#pragma unroll
+      for (u32 a = 0; a < b; ++a) conn[pair(a, b)] |= (n[a] & T[b]) | (n[b] & T[a]);
+    if ((v & 7u) == 0) togw = rec[(K::R_TOG + (v >> 3)) * K::T];
+    const u32 tb = togw >> (4u * (v & 7u));
+    const u32 od0 = (tc_bitmask(tb, 0) & ~same) | (tc_bitmask(tb, 2) & same),
+              od1 = (tc_bitmask(tb, 1) & ~same) | (tc_bitmask(tb, 3) & same);
+    tg[((u32)__ffs(adj & 0xFFFFu) - 1u) * K::T] ^= od0 & ~S;
+    tg[((u32)__ffs(adj >> 16) - 1u) * K::T] ^= od1 & S;
+    if (v == 0) {
+      sfirst = S;
+#pragma unroll
+      for (u32 c = 0; c < NN; ++c) first[c] = n[c];
+    }
+    prev = S;
+  }
+  // the corners (d, 0) and (-d, 0) are one point; identifying them and the
+  // uncrossed boundary edges next to them changes chi by -1 + those edges
+#pragma unroll
+  for (u32 b = 1; b < NN; ++b)
+#pragma unroll
+    for (u32 a = 0; a < b; ++a) conn[pair(a, b)] |= (first[a] & n[b]) | (first[b] & n[a]);
+  {
+    const u32 od = ~(tc_bitmask(hdr, 26) ^ S) ^ ~(tc_bitmask(hdr, 27) ^ sfirst) ^ ~0u;
+    tg[((u32)__ffs(adj & 0xFFFFu) - 1u) * K::T] ^= od & ~S;
+    tg[((u32)__ffs(adj >> 16) - 1u) * K::T] ^= od & S;
+  }
+#pragma unroll
+  for (u32 k = 0; k < NN; ++k)
+#pragma unroll
+    for (u32 b = 1; b < NN; ++b)
+#pragma unroll
+      for (u32 a = 0; a < b; ++a)
+        if (a != k && b != k)
+          conn[pair(a, b)] |= conn[a < k ? pair(a, k) : pair(k, a)] & conn[b < k ? pair(b, k) : pair(k, b)];
+  // region roots (the smallest node of a class), the tree edges they hang on,
+  // the number of regions as a 5-bit number per pattern
+  u32 cnt[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+  for (u32 c = 0; c < NN; ++c) {
+    u32 r = c < N ? ~0u : 0u;
+#pragma unroll
+    for (u32 a = 0; a < c; ++a) r &= ~conn[pair(a, c)];
+    const u32 p = c < N ? (u32)*tc_sb_byte<K>(m.rec, K::R_NPAR, c, hl) : 255u;
+    if (p != 255u) tg[c * K::T] ^= r;
+    if (p < 254u) tg[p * K::T] ^= r;
+    u32 carry = r;
+#pragma unroll
+    for (u32 i = 0; i < 5; ++i) {
+      const u32 s = cnt[i] & carry;
+      cnt[i] ^= carry;
+      carry = s;
+    }
+  }
+  // the root region's nodes: chi + degree of their class is odd
+#pragma unroll
+  for (u32 c = 0; c < NN; ++c) n[c] = tg[c * K::T];
+#pragma unroll
+  for (u32 c = 0; c < NN; ++c) {
+    u32 x = n[c];
+#pragma unroll
+    for (u32 a = 0; a < NN; ++a)
+      if (a != c) x ^= conn[a < c ? pair(a, c) : pair(c, a)] & n[a];
+    T[c] = c < N ? x : 0u;
+  }
+#pragma unroll
+  for (u32 c = 0; c < NN; ++c) tg[c * K::T] = T[c];
+  u32 star = (hdr >> 24) & 1u ? 0u : ~0u, any = 0;
+#pragma unroll
+  for (u32 c = 0; c < NN; ++c) {
+    any |= T[c];
+    if (c < N) {
+      const u32 p = *tc_sb_byte<K>(m.rec, K::R_NPAR, c, hl);
+      if ((nd >> c) & 1u) star &= T[c];
+      if (p < 254u) star &= T[c] | tg[p * K::T];
+    }
+  }
+  const u32 closed = (hdr >> 16) & 255u;
+#pragma unroll
+  for (u32 k = 1; k <= NN; ++k) {
+    u32 x = star & any;
+#pragma unroll
+    for (u32 i = 0; i < 5; ++i) x &= (k >> i) & 1u ? cnt[i] : ~cnt[i];
+    if (x) atomicAdd(m.stars + closed + k, (unsigned long long)__popc(x));
+  }
+  if (~any) {  // no root: counted as failed, not inserted
+    failed += (u32)__popc(~any);
+    err |= TC_ERR_INTERNAL;
+  }
+  // the other patterns, one by one
+  u8 *const par = reinterpret_cast<u8 *>(m.s.lab + 32 * K::T + t);  // byte i: word i / 4 of the thread
+  for (u32 rest = any & ~star; rest; rest &= rest - 1u) {
+    const u32 i = (u32)__ffs(rest) - 1u, C = hdr & 255u;
+    u64 low = 0;  // smallest node of every node's class, 4 bits each
+    u32 rootn = 0, have = 0;
+#pragma unroll
+    for (u32 c = 0; c < NN; ++c) {
+      u32 row = 1u << c;
+#pragma unroll
+      for (u32 a = 0; a < c; ++a) row |= ((conn[pair(a, c)] >> i) & 1u) << a;
+      low |= (u64)((u32)__ffs(row) - 1u) << (4 * c);
+      if (!have && ((T[c] >> i) & 1u)) {
+        have = 1;
+        rootn = c;
+      }
+    }
+    auto comp = [&](u32 c) -> u32 {  // the region of comp c: its smallest comp
+      const u32 k = *tc_sb_byte<K>(m.rec, K::R_CNODE, c, hl);
+      return k == 255u ? c : (u32)*tc_sb_byte<K>(m.rec, K::R_NCOMP, (u32)(low >> (4 * k)) & 15u, hl);
+    };
+    u32 alive = 0;
+    for (u32 c = 0; c < C; ++c) {
+      if (comp(c) != c) continue;
+      alive |= 1u << c;
+      if (c) par[(c >> 2) * 4 * K::T + (c & 3u)] = (u8)comp(*tc_sb_byte<K>(m.rec, K::R_CPAR, c, hl));
+    }
+    const u32 root = *tc_sb_byte<K>(m.rec, K::R_NCOMP, rootn, hl);
+    const u64 key = tc_sl_tree_code<K::T, 4 * K::T, K::RMAX>(par, m.s.lab + t, alive, root, err);
+    if (key)
+      tc_sb_insert<K::HASH>(key, 1, out.hkeys, out.hcnt, out.gkeys, out.gcnt, out.gslots, out.gerr);
+    else
+      ++failed;
+  }
+}

@@ -87,7 +87,7 @@ struct TcSlK {
   static constexpr bool TWTOP = LB == 2 || V <= 128;   // twist bit in the label's top bit
   static constexpr u32 TWWORDS = EVEN && !TWTOP ? NCB : 0;  // else in words of their own
   static constexpr u32 LABW = V * TW * NG;        // words of the label area
-  static constexpr u32 PAR_WORDS = (RMAX * T + 3) / 4;  // region parents, a byte each
+  static constexpr u32 PAR_WORDS = (RMAX + 3) / 4 * T;  // region parents, a byte each
   static constexpr u32 PLANES = (NPOINTS * NG + 3) & ~3u;
   static constexpr u32 BW = PAR_WORDS + TWWORDS * T;
   // tree codes: the wide back end's scratch lies over the label area
@@ -96,6 +96,7 @@ struct TcSlK {
   static constexpr u32 OFF_WPAR = 0, OFF_WFC = WB, OFF_WNS = 2 * WB, OFF_WENT = 3 * WB,
                        OFF_WARENA = 3 * WB + (RMAX / 2 + 2 + 1) / 2,
                        OFF_WTEMP = OFF_WARENA + WARENA, WIDE_WORDS = OFF_WTEMP + WARENA;
+  static_assert(WIDE || RMAX * T <= LABW, "the narrow tree code's children masks fit the label area");
   static_assert(!WIDE || WIDE_WORDS * T <= LABW, "the wide back end's scratch fits the label area");
   // unused members TcScratch names
   static constexpr u32 LBYTES = LB, OFF_LPAR = 0, OFF_CAND = 0;
@@ -436,16 +437,17 @@ struct TcSlInst {
   static constexpr u32 ROW = K::T;  // labels per vertex
   lab_t *l;
   const u32 *ev;
-  u8 *par;
+  u8 *par;  // region r: byte r % 4 of word r / 4
   u32 *tw;
   __device__ __forceinline__ TcSlInst(const TcSlMem &m, u32 t) {
     constexpr u32 WR = K::TW * K::NG;
     const u32 i = tc_sl_instance<K>(t);
     l = reinterpret_cast<lab_t *>(m.lab + t % WR) + t / WR;
     ev = m.ev + (i >> 5) * TC_SL_GROUP + (i & 31u);
-    par = reinterpret_cast<u8 *>(m.x) + t;
+    par = reinterpret_cast<u8 *>(m.x + t);
     tw = m.x + K::PAR_WORDS + t;
   }
+  __device__ __forceinline__ u8 &parent(u32 r) const { return par[(r >> 2) * 4 * K::T + (r & 3u)]; }
   __device__ __forceinline__ u32 *event_word(u32 v) const {
     return const_cast<u32 *>(ev) + (v >> 5) * (K::NG * TC_SL_GROUP);
   }
@@ -644,7 +646,7 @@ __device__ __forceinline__ u32 tc_sl_regions(const TcSlMem &m, const TcSlInst<K>
     if (r) {
       const u32 d = vd[v], p = I.region(I.root(d & 0x7FFFu));
       bad |= !(d & 0x8000u) || p >= r;  // no earlier neighbour, or not a tree
-      I.par[r * K::T] = (u8)p;
+      I.parent(r) = (u8)p;
       star &= p == (r == root ? 0u : root);
     }
   }
@@ -655,50 +657,55 @@ __device__ __forceinline__ u32 tc_sl_regions(const TcSlMem &m, const TcSlInst<K>
   return R;
 }
 
-// Canonical code of a region tree of at most 32 regions that is no star.
-// adj: this thread's children masks, word r at adj[r * T] (over the label
-// area, free by then).  The tree is re-rooted by reversing the path from the
-// root to region 0; AHU codes follow for the regions with children, those off
-// the path by falling index (children have larger ones), then along the path.
-// A code is left-aligned in 64 bits with its length in the low byte (at most
-// 56 bits: fewer than 29 ovals); a leaf's code '10' is the smallest.
-template <class K>
-__device__ __forceinline__ u64 tc_sl_tree_code(const TcSlInst<K> &I, u32 *adj, u32 R, u32 root, u32 &err) {
-  static_assert(2 * K::RMAX <= 58 && K::RMAX * K::T <= K::LABW, "narrow tree codes");
-  for (u32 r = 0; r < R; ++r) adj[r * K::T] = 0;
+// Canonical code of a region tree of at most 29 regions that is no star (28
+// ovals).  alive: the regions' numbers (below 32, region 0 the smallest);
+// parent of region r: byte r % 4 of par's group r / 4 (PW bytes apart), for
+// r > 0, smaller than r; adj: children masks, word r at adj[r * AW], written
+// here.  The tree is re-rooted by reversing the path from the root to region
+// 0; AHU codes follow for the regions with children, those off the path by
+// falling number (children have larger ones), then along the path.  A code is
+// left-aligned in 64 bits with its length in the low byte (at most 56 bits);
+// a leaf's code '10' is the smallest.
+template <u32 AW, u32 PW, u32 RMAX>
+__device__ __forceinline__ u64 tc_sl_tree_code(u8 *par, u32 *adj, u32 alive, u32 root, u32 &err) {
+  static_assert(2 * RMAX <= 58, "narrow tree codes");
+  auto up_of = [&](u32 r) -> u8 & { return par[(r >> 2) * PW + (r & 3u)]; };
+  const u32 first = (u32)__ffs(alive) - 1u;
+  for (u32 a = alive; a; a &= a - 1u) adj[((u32)__ffs(a) - 1u) * AW] = 0;
   u32 internal = 0, path = 0;
-  for (u32 r = 1; r < R; ++r) {
-    const u32 p = I.par[r * K::T];
-    adj[p * K::T] |= 1u << r;
+  for (u32 a = alive & (alive - 1u); a; a &= a - 1u) {
+    const u32 r = (u32)__ffs(a) - 1u, p = up_of(r);
+    adj[p * AW] |= 1u << r;
     internal |= 1u << p;
   }
-  for (u32 x = root, prev = 32;;) {  // reverse the path root -> 0
-    const u32 up = I.par[x * K::T];
-    u32 kids = adj[x * K::T];
+  for (u32 x = root, prev = 32;;) {  // reverse the path root -> region 0
+    const u32 up = x == first ? 32u : (u32)up_of(x);
+    u32 kids = adj[x * AW];
     if (prev < 32) kids &= ~(1u << prev);
-    if (x) kids |= 1u << up;
-    adj[x * K::T] = kids;
+    if (x != first) kids |= 1u << up;
+    adj[x * AW] = kids;
     internal = kids ? internal | (1u << x) : internal & ~(1u << x);
     path |= 1u << x;
-    I.par[x * K::T] = (u8)prev;
-    if (x == 0) break;
+    up_of(x) = (u8)prev;
+    if (x == first) break;
     prev = x;
     x = up;
   }
-  u64 node[(K::RMAX + 1) / 2];  // codes of the regions with children, by rank among them
+  const u32 nb2 = 2u * ((u32)__popc(alive) - 1u);
+  u64 node[(RMAX + 1) / 2];  // codes of the regions with children, by rank among them
   auto rank = [&](u32 x) -> u32 { return (u32)__popc(internal & ((1u << x) - 1u)); };
   for (u32 off = internal & ~path, x = 0;;) {
     if (off) {
       x = 31u - (u32)__clz(off);
       off &= ~(1u << x);
     } else if (path) {  // from region 0 towards the root
-      x = (path & 1u) ? 0u : (u32)I.par[x * K::T];
+      x = (path >> first) & 1u ? first : (u32)up_of(x);
       path &= ~(1u << x);
       if (!((internal >> x) & 1u)) continue;
     } else {
       break;
     }
-    const u32 kids = adj[x * K::T];
+    const u32 kids = adj[x * AW];
     u64 v = 0;
     u32 len = 0;
     for (u32 big = kids & internal; big;) {  // larger codes first
@@ -720,7 +727,7 @@ __device__ __forceinline__ u64 tc_sl_tree_code(const TcSlInst<K> &I, u32 *adj, u
     if (nl) v |= (0xAAAAAAAAAAAAAAAAull & ~(~0ull >> nl)) >> len;
     len += nl;
     if (x == root) {
-      if (len != 2 * (R - 1)) {
+      if (len != nb2) {
         err |= TC_ERR_INTERNAL;
         return 0;
       }
@@ -743,13 +750,14 @@ __device__ __forceinline__ void tc_sl_finish(const TcSlMem &m, const TcSlInst<K>
     for (u32 w = 0; w < K::CW; ++w) code[w] = 0;
     if (R == 0) return;
     const TcScratch<K> S{m.lab + t};
-    for (u32 r = 1; r < R; ++r) *S.byte(K::OFF_WPAR, r) = I.par[r * K::T];
+    for (u32 r = 1; r < R; ++r) *S.byte(K::OFF_WPAR, r) = I.parent(r);
     tc_wide_tree_code(S, R, (int)root, err, code);
   } else {
     const u32 q = 2 * (R - 1);
     code[0] = R == 0 ? 0ull
               : star ? (1ull << q) | (0xAAAAAAAAAAAAAAAAull & ((1ull << q) - 1))
-                     : tc_sl_tree_code<K>(I, m.lab + t, R, root, err);
+                     : tc_sl_tree_code<K::T, 4 * K::T, K::RMAX>(I.par, m.lab + t, R >= 32 ? ~0u : (1u << R) - 1u,
+                                                                root, err);
   }
 }
 

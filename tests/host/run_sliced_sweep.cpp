@@ -24,6 +24,47 @@ static uint64_t special(int d, int which, u32 w) {
   return x;
 }
 
+// The logic and labels phases (middle: the middle row too).
+template <class K>
+static void emulate_labels(const TcSlMem &m, bool middle) {
+  for (u32 i = 0; i < K::T; ++i) tc_sl_logic<K>(m, i);
+  // the threads of a group share a vertex's takes before they write its
+  // planes over them: each runs on the takes as they were, and its planes
+  // are collected
+  std::vector<u32> takes(m.lab, m.lab + K::LABW), planes(K::LABW, 0);
+  for (int part = 0; part < (middle ? 2 : 1); ++part) {
+    for (u32 i = 0; i < K::T; ++i) {
+      u32 half, g, pair;
+      tc_sl_label_thread<K>(i, half, g, pair);
+      if (half > 1 || (part && half)) continue;
+      std::copy(takes.begin(), takes.end(), m.lab);
+      if (part) std::copy(planes.begin(), planes.begin() + 2 * K::H * K::TW * K::NG, m.lab);
+      if (part) tc_sl_labels_middle<K>(m, i);
+      else tc_sl_labels_halves<K>(m, i);
+      const u32 v0 = part ? 2 * K::H : half * K::H, v1 = part ? K::V : (half + 1) * K::H;
+      for (u32 v = v0; v < v1; ++v)
+        for (u32 w = 0; w < K::PP; ++w) {
+          const u32 at = (v * K::NG + g) * K::TW + K::PP * pair + w;
+          planes[at] = m.lab[at];
+        }
+    }
+  }
+  std::copy(planes.begin(), planes.begin() + (middle ? K::V : 2 * K::H) * K::TW * K::NG, m.lab);
+}
+
+template <class K>
+static void emulate_events(const TcSlMem &m, u32 chunks) {
+  for (u32 k = 0; k < chunks * K::NG; ++k) {  // tc_sl_events
+    u32 *const p = m.ev + k * TC_SL_GROUP;
+    u32 o[32];
+    for (u32 r = 0; r < 32; ++r) {
+      o[r] = 0;
+      for (u32 s = 0; s < 32; ++s) o[r] |= ((p[s] >> r) & 1u) << s;
+    }
+    for (u32 r = 0; r < 32; ++r) p[r] = o[r];
+  }
+}
+
 template <int D, int NG>
 int run_sliced(const char *edge_file, int blocks) {
   typedef TcSlK<D, NG> K;
@@ -63,40 +104,9 @@ int run_sliced(const char *edge_file, int blocks) {
         for (u32 i = 0; i < 32; ++i) x |= sig[32 * g + i].bit(k) << i;
         m.x[k * K::NG + g] = x;
       }
-    for (u32 i = 0; i < K::T; ++i) tc_sl_logic<K>(m, i);
-    // the threads of a group share a vertex's takes before they write its
-    // planes over them: each runs on the takes as they were, and its planes
-    // are collected
-    std::vector<u32> takes(m.lab, m.lab + K::LABW), planes(K::LABW, 0);
-    for (int part = 0; part < 2; ++part) {
-      for (u32 i = 0; i < K::T; ++i) {
-        u32 half, g, pair;
-        tc_sl_label_thread<K>(i, half, g, pair);
-        if (half > 1 || (part && half)) continue;
-        std::copy(takes.begin(), takes.end(), m.lab);
-        if (part) std::copy(planes.begin(), planes.begin() + 2 * K::H * K::TW * K::NG, m.lab);
-        if (part) tc_sl_labels_middle<K>(m, i);
-        else tc_sl_labels_halves<K>(m, i);
-        const u32 v0 = part ? 2 * K::H : half * K::H, v1 = part ? K::V : (half + 1) * K::H;
-        for (u32 v = v0; v < v1; ++v)
-          for (u32 w = 0; w < K::PP; ++w) {
-            const u32 at = (v * K::NG + g) * K::TW + K::PP * pair + w;
-            planes[at] = m.lab[at];
-          }
-      }
-    }
-    std::copy(planes.begin(), planes.end(), m.lab);
+    emulate_labels<K>(m, true);
     for (u32 i = 0; i < K::T; ++i) tc_sl_tiles<K>(m, i);
-    for (u32 k = 0; k < nch * K::NG; ++k) {  // tc_sl_events
-      u32 *const p = m.ev + k * TC_SL_GROUP, x[32] = {};
-      (void)x;
-      u32 o[32];
-      for (u32 r = 0; r < 32; ++r) {
-        o[r] = 0;
-        for (u32 s = 0; s < 32; ++s) o[r] |= ((p[s] >> r) & 1u) << s;
-      }
-      for (u32 r = 0; r < 32; ++r) p[r] = o[r];
-    }
+    emulate_events<K>(m, nch);
     std::vector<u64> code((size_t)K::T * K::CW, 0);
     std::vector<u32> R(K::T), root(K::T), err(K::T, 0);
     std::vector<char> star(K::T);
@@ -126,6 +136,7 @@ int run_sliced(const char *edge_file, int blocks) {
   return bad != 0;
 }
 
+#ifndef TC_SL_NO_MAIN
 int main(int argc, char **argv) {
   const int d = atoi(argv[1]), n = atoi(argv[3]);
   switch (d) {
@@ -136,3 +147,4 @@ int main(int argc, char **argv) {
   }
   return 2;
 }
+#endif

@@ -20,11 +20,12 @@ def sliced_exe(tmp_path_factory):
         pytest.skip("needs g++ and the CUDA headers")
     csrc = os.path.join(ROOT, "paper_2604_09221_gb300", "csrc")
     out = {}
-    for groups in (2, 4):
+    for groups in (2, 4, "blocks"):
         exe = tmp_path_factory.mktemp("sliced") / f"run{groups}"
+        name = "run_block_sliced.cpp" if groups == "blocks" else "run_sliced_sweep.cpp"
         cmd = ["g++", "-std=c++17", "-O1", "-w", f"-DTC_SL_GROUPS={groups}", f"-I{csrc}",
                f"-I{os.path.join(HERE, 'host')}", f"-I{os.path.join(ROOT, 'oracle')}",
-               f"-I{CUDA}/include", "-o", str(exe), os.path.join(HERE, "host", "run_sliced_sweep.cpp"),
+               f"-I{CUDA}/include", "-o", str(exe), os.path.join(HERE, "host", name),
                "-x", "c", os.path.join(ROOT, "oracle", "tcurve_oracle.c"), "-x", "none",
                f"-L{CUDA}/lib64", f"-Wl,-rpath,{CUDA}/lib64", "-lcudart", "-lpthread"]
         subprocess.run(cmd, check=True, capture_output=True)
@@ -46,7 +47,34 @@ def test_sliced_sweep_on_the_host(sliced_exe, tmp_path, d):
         cases.append(("fan", ti.fan_triangulation(d)))
     for name, edges in cases:
         np.savetxt(tmp_path / "tri.txt", edges, fmt="%d")
-        for groups, exe in sliced_exe.items():
+        for groups in (2, 4):
+            exe = sliced_exe[groups]
             out = subprocess.run([str(exe), str(d), str(tmp_path / "tri.txt"), "3"],
                                  capture_output=True, text=True)
             assert out.returncode == 0, (name, groups, out.stdout + out.stderr)
+
+
+@pytest.mark.parametrize("d", [4, 5, 6, 7, 8, 9])
+def test_block_sweep_on_the_host(sliced_exe, tmp_path, d):
+    """The bit-sliced block sweep: the halves of 128 high parts (the first,
+    the last and random ones) and every middle-row pattern of each, per mask
+    map, against the oracle's histogram of the same masks; standard, regular,
+    fan and (d = 8) the printed triangulations.  The middle phase takes every
+    high part but those of the fan triangulation at d = 9 (too many open
+    components: the kernel takes those mask by mask)."""
+    cases = [("standard", ti.standard_triangulation(d)), ("regular", ti.regular_triangulation(d, seed=d)),
+             ("fan", ti.fan_triangulation(d))]
+    if d == 8:
+        cases += [(n, np.loadtxt(os.path.join(HERE, "golden", f"fig2_{n}.edges"), dtype=np.int32, comments="#"))
+                  for n in ("rank016", "rank015")]
+    for k, (name, edges) in enumerate(cases):
+        np.savetxt(tmp_path / "tri.txt", edges, fmt="%d")
+        maps = [("plain", d + 1), ("flip", d), ("reduced", d - 1), ("orbits", d + 1)]
+        for mode, ib in maps if name == "regular" else maps[:1]:
+            if ib < 5:
+                continue
+            out = subprocess.run([str(sliced_exe["blocks"]), str(d), str(tmp_path / "tri.txt"), mode, str(k)],
+                                 capture_output=True, text=True)
+            assert out.returncode == 0, (name, mode, out.stdout + out.stderr)
+            taken = int(out.stdout.split("middle phase=")[1].split()[0])
+            assert taken == (0 if (name, d) == ("fan", 9) else 128), out.stdout
