@@ -22,7 +22,7 @@ namespace {
 // t < 2^ib.  smem: tables (toff bytes) | mbarrier, work slot (128 bytes) |
 // the areas | hash table.
 template <int D>
-__global__ void __launch_bounds__(128, 2)
+__global__ void __launch_bounds__(128, D <= 7 ? 3 : 2)
     block_sweep_kernel(SlicedLayout L, const uint32_t *__restrict__ gtab, uint64_t hi0, uint64_t n_hi,
                        uint32_t oshift, uint32_t ishift, uint32_t ib, uint32_t flags, ts_hist h) {
   typedef TcSbK<D> K;
@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(128, 2)
   unsigned long long *const slot = reinterpret_cast<unsigned long long *>(smem + toff + 64);
   const TcSbMem M = tc_sb_carve<K>(tab, area, L.chunks, L.far);
   u64 *const hkeys = reinterpret_cast<u64 *>(area + tc_sb_words<K>(L.chunks, L.far));
-  unsigned long long *const hcnt = reinterpret_cast<unsigned long long *>(hkeys + K::HASH);
+  u32 *const hcnt = reinterpret_cast<u32 *>(hkeys + K::HASH);
   const TcSbOut out{hkeys, hcnt, reinterpret_cast<u64 *>(h.d_keys), h.d_counts, h.slots, h.d_err};
   const u32 t = threadIdx.x, mine = tc_sl_instance<B>(t), lw = ib - 5u;
   for (u32 s = t; s < K::HASH; s += K::T) {
@@ -42,10 +42,24 @@ __global__ void __launch_bounds__(128, 2)
     hcnt[s] = 0;
   }
   for (u32 s = t; s < K::STARS; s += K::T) M.stars[s] = 0;
+  if (t == 0) *M.queued = 0;
   if (t == 0) *slot = atomicAdd(h.d_work, (unsigned long long)K::T);
   if (!stage_tables(tab, gtab, L.words * 4, reinterpret_cast<uint64_t *>(smem + toff), h.d_err)) return;
-  uint32_t err = 0;
+  uint32_t err = 0, items = 0;
   unsigned long long failed = 0;
+  auto flush = [&] {  // the block's counts to the device table, by the thread that owns the slot
+    for (u32 s = t; s < K::HASH; s += K::T)
+      if (hcnt[s]) {
+        tc_global_add(out.gkeys, h.d_counts, h.slots, h.d_err, hkeys[s], hcnt[s]);
+        hcnt[s] = 0;
+      }
+    for (u32 R = t; R < K::STARS; R += K::T)
+      if (M.stars[R]) {
+        tc_global_add(out.gkeys, h.d_counts, h.slots, h.d_err, tc_sb_star_code(R), M.stars[R]);
+        M.stars[R] = 0;
+      }
+    __syncthreads();
+  };
   auto mask_of = [&](uint64_t i) -> u64 {  // of block i of the range, middle row zero
     const u64 u = hi0 + i;
     return ((flags & TS_ENUM_ORBITS) ? tc_orbit_high(u, flags) : u) << oshift;
@@ -80,9 +94,8 @@ __global__ void __launch_bounds__(128, 2)
       } else if (valid) {
         tc_sb_middle<K, K::NA>(M, t, hl, w, ishift, out, err, failed);
       }
-      __syncwarp();
+      tc_sb_flush_queue<K>(M, t, task + K::T >= K::T << lw, out, err, failed);
     }
-    __syncthreads();
     for (u32 hl = 0; hl < K::T; ++hl) {  // high parts the middle phase does not take
       const u32 hdr = M.rec[K::R_HDR * K::T + hl];
       if ((hdr >> 25) & 1u || hdr >> 31) continue;
@@ -95,17 +108,16 @@ __global__ void __launch_bounds__(128, 2)
         code = in ? code : 0ull;
         err |= in ? e : 0u;
         failed += in && code == 0;
-        tc_hist_add<K::HASH>(code, hkeys, hcnt, out.gkeys, h.d_counts, h.slots, h.d_err);
+        if (code) tc_sb_insert<K::HASH>(code, 1, hkeys, hcnt, out.gkeys, h.d_counts, h.slots, h.d_err);
         __syncthreads();
       }
     }
     __syncthreads();
+    // at most 2^10 patterns per high part: counts stay below 2^32 for 2^15 items
+    if ((++items & 63u) == 0) flush();
   }
   __syncthreads();
-  for (u32 s = t; s < K::HASH; s += K::T)
-    if (hkeys[s]) tc_global_add(out.gkeys, h.d_counts, h.slots, h.d_err, hkeys[s], hcnt[s]);
-  for (u32 R = t; R < K::STARS; R += K::T)
-    if (M.stars[R]) tc_global_add(out.gkeys, h.d_counts, h.slots, h.d_err, tc_sb_star_code(R), M.stars[R]);
+  flush();
   if (err) atomicOr(h.d_err, err);
   if (failed) atomicAdd(h.d_failed, failed);
 }

@@ -22,8 +22,12 @@
 //            pseudoline's two sides), where chi counts label starts minus join
 //            events.  Both are sums over nodes, kept modulo 2 as bit planes.
 //            Patterns whose regions all border the root (a star) are counted
-//            by their number of regions; the codes of the others are made one
-//            by one from their classes.
+//            by their number of regions.  Trees of depth two are told by that
+//            number and how many children of the root have 1, 2, ... children
+//            of their own: the regions' degrees are sums over classes too,
+//            three bit planes each, and one code is made for all patterns of a
+//            word with the same numbers.  Deeper trees are coded one by one
+//            from their classes.
 //
 // Every middle vertex has half-diamond neighbours of both signs: the triangle
 // over an edge of the x-axis has its apex at height 1, and the reflections
@@ -45,35 +49,47 @@ struct TcSbK : TcSlK<D_, 4> {
   // record of a high part (words, one column per thread)
   static constexpr u32 R_HDR = 0,          // comps | nodes << 8 | closed comps << 16 | star impossible << 24
                                            // | valid << 25 | corner edge signs << 26, 27
+                                           // | some closed comp is no leaf << 28
                        R_NODE = 1,         // nodes that must be in the root | chi parities << 16
                        R_ADJ = 2,          // per middle vertex: nodes next to it with sigma 0 | with sigma 1 << 16
                        R_TOG = R_ADJ + M,  // per middle vertex 4 bits: chi changes by an odd number; bit
                                            // sigma + 2 * (same sign as the vertex before)
                        R_NPAR = R_TOG + (4 * M + 31) / 32,  // parent of a node (byte): node, 254 closed, 255 none
                        R_NCOMP = R_NPAR + 4,                // comp of a node (byte)
-                       R_CPAR = R_NCOMP + 4,                // parent of a comp (byte)
+                       R_KIDS = R_NCOMP + 4,                // closed leaves at a node (byte)
+                       R_CPAR = R_KIDS + 4,                 // parent of a comp (byte)
                        R_CNODE = R_CPAR + 8,                // node of a comp (byte; 255: closed)
                        R_WORDS = R_CNODE + 8;
   static constexpr u32 T = Base::T;
-  // areas (words): the label area also holds the tree codes' children masks
-  // and parents (32 + 8 words per thread); scratch: M words per thread
-  static constexpr u32 LAB = Base::LABW > 40 * T ? Base::LABW : 40 * T;
+  // areas (words): the label area also holds, per thread, the degree planes
+  // (3 NB words) or a tree code's children masks and parents (32 + 8 words);
+  // scratch: M words per thread; the event chunks also hold the queue of deep
+  // trees
+  static constexpr u32 LAB = Base::LABW > 48 * T ? Base::LABW : 48 * T;
+  static constexpr u32 QUEUE = 512;  // deep trees in waiting (four words each)
+  static constexpr u32 HASH = D_ <= 7 ? 256 : 512;
   static constexpr u32 SW = (M > 16 ? M : 16) * T;
-  static constexpr u32 STARS = 48;  // star patterns by number of regions (64-bit counts)
+  static constexpr u32 STARS = 48;  // star patterns by number of regions
 };
 
 struct TcSbMem {
   TcSlMem s;     // tables, labels, events, sign planes
-  u32 *chi;      // K::NCB words per thread
   u32 *rec;      // K::R_WORDS words per thread
   u32 *scr;      // K::SW words
-  unsigned long long *stars;  // K::STARS counters
+  u32 *stars;    // K::STARS counters
+  u32 *queue;    // K::QUEUE deep trees: two words of node classes, high part | root node << 16, patterns
+  u32 *queued;   // their number
 };
 
 template <class K>
+__host__ __device__ constexpr u32 tc_sb_evwords(u32 chunks) {
+  return chunks * K::NG * TC_SL_GROUP > 4 * K::QUEUE ? chunks * K::NG * TC_SL_GROUP : 4 * K::QUEUE;
+}
+
+template <class K>
 __host__ __device__ constexpr u32 tc_sb_words(u32 chunks, u32 far) {
-  return K::LAB + chunks * K::NG * TC_SL_GROUP + tc_sl_xwords<typename K::Base>(far) + K::NCB * K::T +
-         K::R_WORDS * K::T + K::SW + 2 * K::STARS;
+  return K::LAB + tc_sb_evwords<K>(chunks) + tc_sl_xwords<typename K::Base>(far) +
+         K::R_WORDS * K::T + K::SW + K::STARS + 4;
 }
 
 template <class K>
@@ -82,11 +98,12 @@ __device__ __forceinline__ TcSbMem tc_sb_carve(const u32 *tab, u32 *area, u32 ch
   m.s.tab = tab;
   m.s.lab = area;
   m.s.ev = m.s.lab + K::LAB;
-  m.s.x = m.s.ev + chunks * K::NG * TC_SL_GROUP;
-  m.chi = m.s.x + tc_sl_xwords<typename K::Base>(far);
-  m.rec = m.chi + K::NCB * K::T;
+  m.queue = m.s.ev;
+  m.s.x = m.s.ev + tc_sb_evwords<K>(chunks);
+  m.rec = m.s.x + tc_sl_xwords<typename K::Base>(far);
   m.scr = m.rec + K::R_WORDS * K::T;
-  m.stars = reinterpret_cast<unsigned long long *>(m.scr + K::SW);
+  m.stars = m.scr + K::SW;
+  m.queued = m.stars + K::STARS;
   return m;
 }
 
@@ -111,34 +128,45 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
   for (u32 c = (HB + 31) / 32; c < K::NCB; ++c) I.set_event(c, 0);
   const u32 be = (I.event(K::NCB + nc1) | 1u) & ((1u << (2 * K::D - 1)) - 1u);
   I.set_event(K::NCB + nc1, be);
-  for (u32 c = 0; c < K::NCB; ++c) m.chi[c * K::T + t] = I.event(c);  // label starts, before joins drop some
+  u32 starts[K::NCB];
+#pragma unroll
+  for (u32 c = 0; c < K::NCB; ++c) starts[c] = I.event(c);
   tc_sl_joins<typename K::Base>(I, tab + tab[5], 0, nc1 + 1);
-  // chi of every comp modulo 2, at its root: label starts plus join events
-  auto toggle = [&](u32 r) { m.chi[(r >> 5) * K::T + t] ^= 1u << (r & 31u); };
-  {
-    u32 starts[K::NCB];  // (the starts that are roots keep their own bit)
+  u32 C = 0;  // comps, numbered by their roots
 #pragma unroll
-    for (u32 c = 0; c < K::NCB; ++c) {
-      starts[c] = m.chi[c * K::T + t] & ~I.event(c);
-      m.chi[c * K::T + t] = I.event(c);
-    }
-#pragma unroll
-    for (u32 c = 0; c < K::NCB; ++c)
-      for (u32 w = starts[c]; w; w &= w - 1u) toggle(I.root(32u * c + (u32)__ffs(w) - 1u));
-    const u32 *const site = tab + tab[5];
-    for (u32 c = 0; c <= nc1; ++c)
-      for (u32 w = I.event(K::NCB + c); w; w &= w - 1u)
-        toggle(I.root(site[32u * c + (u32)__ffs(w) - 1u] & 0xFFFFu));
-  }
-  u32 C = 0;  // comps, numbered by their roots; the join chunks are used up
-#pragma unroll
-  for (u32 c = 0; c < K::NCB; ++c) {
-    I.set_event(K::NCB + c, C);
-    C += (u32)__popc(I.event(c));
-  }
+  for (u32 c = 0; c < K::NCB; ++c) C += (u32)__popc(I.event(c));
   u32 *const rec = m.rec + t;
   rec[K::R_HDR * K::T] = 0;
   if (C > 32) return;  // not valid: the block's masks one by one
+  // every label start gets its comp (a parent is smaller, so it has its comp
+  // already), marked by the top three bits, which no vertex number has set
+  static_assert(K::LB == 1 && K::V < 224, "comps marked in label bytes");
+  u32 chis = 0;  // chi of every comp modulo 2: label starts plus join events
+  C = 0;
+#pragma unroll
+  for (u32 c = 0; c < K::NCB; ++c)
+    for (u32 w = starts[c]; w; w &= w - 1u) {
+      const u32 v = 32u * c + (u32)__ffs(w) - 1u, p = I.raw(v);
+      const u32 id = p == v ? C : I.raw(p) & 31u;
+      C += p == v ? 1u : 0u;
+      I.set(v, 224u | id);
+      chis ^= 1u << id;
+    }
+  auto comp_of = [&](u32 v) -> u32 {
+    const u32 x = I.raw(v);
+    return (x < 224u ? I.raw(x) : x) & 31u;
+  };
+  {
+    const u32 *const site = tab + tab[5];
+    u32 c = 0, w = 0;
+    for (;;) {
+      while (w == 0 && c <= nc1) w = I.event(K::NCB + c++);
+      if (w == 0) break;
+      const u32 s = site[32u * (c - 1u) + (u32)__ffs(w) - 1u];
+      w &= w - 1u;
+      chis ^= 1u << comp_of(s & 0xFFFFu);
+    }
+  }
   // the middle vertices' neighbours: comps next to them by sign, and whether
   // chi changes by an odd number when the vertex joins: 1 minus the runs of
   // its same-sign earlier neighbours, for either sign and with or without the
@@ -159,7 +187,7 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
         } else {
           // sigma of the middle vertex for which the two have one sign
           const u32 b = ((u32)(sig >> (e & 63u)) ^ (e >> 31) ^ 1u) & 1u;
-          const u32 c = 1u << I.region(I.root(u));
+          const u32 c = 1u << comp_of(u);
           m0 |= b ? 0u : c;
           m1 |= b ? c : 0u;
           bits |= b << n;
@@ -198,7 +226,9 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
   }
   // comps in order: parents, chi, what a star needs
   auto node_of = [&](u32 c) -> u32 { return (open >> c) & 1u ? (u32)__popc(open & ((1u << c) - 1u)) : 255u; };
-  u32 need = 0, chi = 0, nostar = 0;
+  u32 need = 0, chi = 0, nostar = 0, inner = 0;
+  u32 zkids = 0, zkid = 255u;  // comp 0's children, one of them
+  for (u32 k = 0; k < 4; ++k) rec[(K::R_KIDS + k) * K::T] = 0;
   const u32 *const vd = tab + tab[4];
   {
     u32 ch = 0, w = 0;
@@ -206,23 +236,42 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
       while (w == 0) w = I.event(ch++);
       const u32 v = 32u * (ch - 1u) + (u32)__ffs(w) - 1u;
       w &= w - 1u;
-      const u32 p = c ? I.region(I.root(vd[v] & 0x7FFFu)) : 255u, nc = node_of(c),
+      const u32 p = c ? comp_of(vd[v] & 0x7FFFu) : 255u, nc = node_of(c),
                 np = c ? node_of(p) : 255u;
       *tc_sb_byte<K>(m.rec, K::R_CPAR, c, t) = (u8)p;
       *tc_sb_byte<K>(m.rec, K::R_CNODE, c, t) = (u8)nc;
+      if (p == 0) {
+        ++zkids;
+        zkid = nc;
+      }
       if (nc != 255u) {
         *tc_sb_byte<K>(m.rec, K::R_NPAR, nc, t) = (u8)(c == 0 ? 255u : np == 255u ? 254u : np);
         *tc_sb_byte<K>(m.rec, K::R_NCOMP, nc, t) = (u8)c;
-        chi ^= ((m.chi[(v >> 5) * K::T + t] >> (v & 31u)) & 1u) << nc;
+        chi ^= ((chis >> c) & 1u) << nc;
         need |= c && np == 255u ? 1u << nc : 0u;
+        inner |= c && np == 255u && p != 0 ? 1u : 0u;
       } else if (c) {  // a closed comp: one more neighbour of its parent
         if (np == 255u) {
-          nostar = 1;
+          nostar = inner = 1;
         } else {
           chi ^= 1u << np;
           need |= 1u << np;
+          u8 *const k = tc_sb_byte<K>(m.rec, K::R_KIDS, np, t);
+          inner |= *k == 7u;
+          ++*k;
         }
       }
+    }
+  }
+  if (node_of(0) == 255u) {
+    if (zkids == 1u && zkid != 255u) {  // comp 0 is a closed leaf at its one child
+      *tc_sb_byte<K>(m.rec, K::R_NPAR, zkid, t) = 255u;
+      chi ^= 1u << zkid;
+      u8 *const k = tc_sb_byte<K>(m.rec, K::R_KIDS, zkid, t);
+      inner |= *k == 7u;
+      ++*k;
+    } else {
+      inner = 1;
     }
   }
   // sigma of each corner for which its half-diamond boundary edge is not
@@ -232,7 +281,8 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
   const u32 s0 = ((u32)(sig >> ((e0 >> 8) & 63u)) ^ (e0 >> 16)) & 1u;
   const u32 s1 = ((u32)(sig >> (e1 & 63u)) ^ (e1 >> 16)) & 1u;
   rec[K::R_NODE * K::T] = need | (chi << 16);
-  rec[K::R_HDR * K::T] = C | (N << 8) | ((C - N) << 16) | (nostar << 24) | (1u << 25) | (s0 << 26) | (s1 << 27);
+  rec[K::R_HDR * K::T] = C | (N << 8) | ((C - N) << 16) | (nostar << 24) | (1u << 25) | (s0 << 26) | (s1 << 27) |
+                         (inner << 28);
 }
 
 // ---- middle: 32 patterns per thread ----
@@ -250,10 +300,11 @@ __device__ __forceinline__ u32 tc_sb_plane(u32 j, u32 w) {
 }
 
 // Add cnt to key in the block's hash table, or in the device's if that is full.
+// The block's counts have 32 bits (a 64-bit add in shared memory is a
+// compare-and-swap loop) and are moved to the device every few work items.
 template <u32 HASH>
-__device__ __forceinline__ void tc_sb_insert(u64 key, unsigned long long cnt, u64 *hkeys,
-                                             unsigned long long *hcnt, u64 *gkeys, unsigned long long *gcnt,
-                                             u64 gslots, u32 *gerr) {
+__device__ __forceinline__ void tc_sb_insert(u64 key, u32 cnt, u64 *hkeys, u32 *hcnt, u64 *gkeys,
+                                             unsigned long long *gcnt, u64 gslots, u32 *gerr) {
   u32 s = tc_hash_slot(key, HASH - 1);
   for (u32 probe = 0; probe < HASH; ++probe) {
     unsigned long long *kp = reinterpret_cast<unsigned long long *>(hkeys + s);
@@ -277,12 +328,37 @@ __device__ __forceinline__ u64 tc_sb_star_code(u32 R) {
 // Where the codes of a sweep go.
 struct TcSbOut {
   u64 *hkeys;
-  unsigned long long *hcnt;
+  u32 *hcnt;
   u64 *gkeys;
   unsigned long long *gcnt;
   u64 gslots;
   u32 *gerr;
 };
+
+// Code and count cnt patterns of high part hl: low = the smallest node of every
+// node's class, 4 bits each, rootn a node of the root's class.
+template <class K>
+__device__ __noinline__ void tc_sb_deep(const TcSbMem &m, u32 t, u32 hl, u64 low, u32 rootn, u32 cnt,
+                                        const TcSbOut &out, u32 &err, unsigned long long &failed) {
+  u8 *const par = reinterpret_cast<u8 *>(m.s.lab + 32 * K::T + t);  // byte i: word i / 4 of the thread
+  const u32 C = m.rec[K::R_HDR * K::T + hl] & 255u;
+  auto comp = [&](u32 c) -> u32 {  // the region of comp c: its smallest comp
+    const u32 k = *tc_sb_byte<K>(m.rec, K::R_CNODE, c, hl);
+    return k == 255u ? c : (u32)*tc_sb_byte<K>(m.rec, K::R_NCOMP, (u32)(low >> (4 * k)) & 15u, hl);
+  };
+  u32 alive = 0;
+  for (u32 c = 0; c < C; ++c) {
+    if (comp(c) != c) continue;
+    alive |= 1u << c;
+    if (c) par[(c >> 2) * 4 * K::T + (c & 3u)] = (u8)comp(*tc_sb_byte<K>(m.rec, K::R_CPAR, c, hl));
+  }
+  const u32 root = *tc_sb_byte<K>(m.rec, K::R_NCOMP, rootn, hl);
+  const u64 key = tc_sl_tree_code<K::T, 4 * K::T, K::RMAX>(par, m.s.lab + t, alive, root, err);
+  if (key)
+    tc_sb_insert<K::HASH>(key, cnt, out.hkeys, out.hcnt, out.gkeys, out.gcnt, out.gslots, out.gerr);
+  else
+    failed += cnt;
+}
 
 // Word w of the patterns of high part hl (a column of the records), at most
 // NN nodes; ishift: the lowest middle-row bit that varies.
@@ -361,6 +437,7 @@ __device__ __forceinline__ void tc_sb_middle(const TcSbMem &m, u32 t, u32 hl, u3
     const u32 p = c < N ? (u32)*tc_sb_byte<K>(m.rec, K::R_NPAR, c, hl) : 255u;
     if (p != 255u) tg[c * K::T] ^= r;
     if (p < 254u) tg[p * K::T] ^= r;
+    first[c] = r;
     u32 carry = r;
 #pragma unroll
     for (u32 i = 0; i < 5; ++i) {
@@ -398,44 +475,181 @@ __device__ __forceinline__ void tc_sb_middle(const TcSbMem &m, u32 t, u32 hl, u3
     u32 x = star & any;
 #pragma unroll
     for (u32 i = 0; i < 5; ++i) x &= (k >> i) & 1u ? cnt[i] : ~cnt[i];
-    if (x) atomicAdd(m.stars + closed + k, (unsigned long long)__popc(x));
+    if (x) atomicAdd(m.stars + closed + k, (u32)__popc(x));
   }
   if (~any) {  // no root: counted as failed, not inserted
     failed += (u32)__popc(~any);
     err |= TC_ERR_INTERNAL;
   }
-  // the other patterns, one by one
-  u8 *const par = reinterpret_cast<u8 *>(m.s.lab + 32 * K::T + t);  // byte i: word i / 4 of the thread
-  for (u32 rest = any & ~star; rest; rest &= rest - 1u) {
-    const u32 i = (u32)__ffs(rest) - 1u, C = hdr & 255u;
+  u32 rest = any & ~star;
+  // Trees of depth two: every edge that does not touch the root has an end of
+  // degree one.  Degrees as three bit planes, by node (area: the label area,
+  // 3 NN + words per thread), then by class.
+  static_assert(3 * NN <= K::LAB / K::T, "degree planes");
+  {
+    if (rest && !((hdr >> 28) & 1u)) {
+      u32 *const A = m.s.lab + t;
+      u32 over = 0;  // patterns with a number too large for its planes
+      auto bump = [&](u32 c, u32 x) {
+#pragma unroll
+        for (u32 i = 0; i < 3; ++i) {
+          const u32 y = A[(3 * c + i) * K::T];
+          A[(3 * c + i) * K::T] = y ^ x;
+          x &= y;
+        }
+        over |= x;
+      };
+#pragma unroll
+      for (u32 c = 0; c < NN; ++c) {
+        const u32 k = c < N ? (u32)*tc_sb_byte<K>(m.rec, K::R_KIDS, c, hl) : 0u;
+#pragma unroll
+        for (u32 i = 0; i < 3; ++i) A[(3 * c + i) * K::T] = tc_bitmask(k, i);
+      }
+#pragma unroll
+      for (u32 c = 0; c < NN; ++c)
+        if (c < N) {
+          const u32 p = *tc_sb_byte<K>(m.rec, K::R_NPAR, c, hl);
+          if (p < 254u) {
+            bump(c, first[c]);
+            bump(p, first[c]);
+          }
+        }
+      u32 num[13];  // regions off the root with 1 (three planes), 2 .. 6 (two planes) children
+#pragma unroll
+      for (u32 i = 0; i < 13; ++i) num[i] = 0;
+#pragma unroll
+      for (u32 c = 0; c < NN; ++c) {
+        u32 d0 = A[(3 * c) * K::T], d1 = A[(3 * c + 1) * K::T], d2 = A[(3 * c + 2) * K::T], o = 0;
+#pragma unroll
+        for (u32 b = c + 1; b < NN; ++b) {
+          const u32 mk = conn[pair(c, b)];
+          const u32 x0 = A[(3 * b) * K::T] & mk, x1 = A[(3 * b + 1) * K::T] & mk, x2 = A[(3 * b + 2) * K::T] & mk;
+          const u32 c0 = d0 & x0, c1 = (d1 & x1) | (c0 & (d1 ^ x1)), c2 = (d2 & x2) | (c1 & (d2 ^ x2));
+          d0 ^= x0;
+          d1 ^= x1 ^ c0;
+          d2 ^= x2 ^ c1;
+          o |= c2;
+        }
+        over |= o & first[c];
+        n[c] = first[c] & d0 & ~d1 & ~d2;  // the class is a leaf (by its smallest node)
+        const u32 x = first[c] & ~T[c];
+        const u32 e2 = x & ~d0 & d1 & ~d2;
+        const u32 c0 = num[0] & e2, c1 = num[1] & c0;
+        num[0] ^= e2;
+        num[1] ^= c0;
+        over |= num[2] & c1;
+        num[2] ^= c1;
+#pragma unroll
+        for (u32 k = 3; k < 8; ++k) {
+          const u32 e = x & (k & 1u ? d0 : ~d0) & (k & 2u ? d1 : ~d1) & (k & 4u ? d2 : ~d2);
+          const u32 y = num[2 * k - 3] & e;
+          num[2 * k - 3] ^= e;
+          over |= num[2 * k - 2] & y;
+          num[2 * k - 2] ^= y;
+        }
+      }
+#pragma unroll
+      for (u32 c = 0; c < NN; ++c) {  // leaf planes of all nodes
+        u32 x = n[c];
+#pragma unroll
+        for (u32 a = 0; a < c; ++a) x |= conn[pair(a, c)] & n[a];
+        A[3 * c * K::T] = x;
+      }
+      u32 deep = over;
+#pragma unroll
+      for (u32 c = 0; c < NN; ++c)
+        if (c < N) {
+          const u32 p = *tc_sb_byte<K>(m.rec, K::R_NPAR, c, hl);
+          if (p < 254u) deep |= first[c] & ~(T[c] | tg[p * K::T] | A[3 * c * K::T] | A[3 * p * K::T]);
+        }
+      for (u32 f = rest & ~deep; f;) {  // patterns with the numbers of the first one
+        const u32 i = (u32)__ffs(f) - 1u;
+        u32 eq = f, R = closed, ovals = 0;
+        auto bit = [&](u32 x) -> u32 {
+          const u32 b = (x >> i) & 1u;
+          eq &= b ? x : ~x;
+          return b;
+        };
+#pragma unroll
+        for (u32 k = 0; k < 5; ++k) R += bit(cnt[k]) << k;
+        u32 q[8];
+        q[2] = bit(num[0]);
+        q[2] += bit(num[1]) << 1;
+        q[2] += bit(num[2]) << 2;
+#pragma unroll
+        for (u32 k = 3; k < 8; ++k) {
+          q[k] = bit(num[2 * k - 3]);
+          q[k] += bit(num[2 * k - 2]) << 1;
+        }
+        u64 key = 1;
+#pragma unroll
+        for (u32 k = 7; k >= 2; --k)  // a region with k - 1 leaves: 1 (10)^(k-1) 0
+          for (u32 j = 0; j < q[k]; ++j) {
+            key = (key << (2 * k)) | (1ull << (2 * k - 1)) | ((0xAAAAu & ((1u << (2 * k - 2)) - 1u)) << 1);
+            ovals += k;
+          }
+        const u32 leaves = R - 1u - ovals;
+        key = (key << (2 * leaves)) | (0xAAAAAAAAAAAAAAAAull & ((1ull << (2 * leaves)) - 1));
+        tc_sb_insert<K::HASH>(key, (u32)__popc(eq), out.hkeys, out.hcnt, out.gkeys, out.gcnt,
+                              out.gslots, out.gerr);
+        f &= ~eq;
+      }
+      rest &= deep;
+    }
+  }
+  // deeper trees, one by one (patterns of the word with the same classes and
+  // root together): queued for the whole block to code, so that its lanes have
+  // one each, or coded here when the queue is full
+  while (rest) {
+    const u32 i = (u32)__ffs(rest) - 1u;
     u64 low = 0;  // smallest node of every node's class, 4 bits each
-    u32 rootn = 0, have = 0;
+    u32 rootn = 0, have = 0, eq = rest;
 #pragma unroll
     for (u32 c = 0; c < NN; ++c) {
       u32 row = 1u << c;
 #pragma unroll
-      for (u32 a = 0; a < c; ++a) row |= ((conn[pair(a, c)] >> i) & 1u) << a;
-      low |= (u64)((u32)__ffs(row) - 1u) << (4 * c);
-      if (!have && ((T[c] >> i) & 1u)) {
-        have = 1;
-        rootn = c;
+      for (u32 a = 0; a < c; ++a) {
+        const u32 x = conn[pair(a, c)], b = (x >> i) & 1u;
+        row |= b << a;
+        eq &= x ^ (b - 1u);
       }
+      low |= (u64)((u32)__ffs(row) - 1u) << (4 * c);
+      const u32 g = (T[c] >> i) & 1u;
+      eq &= T[c] ^ (g - 1u);
+      rootn = g && !have ? c : rootn;
+      have |= g;
     }
-    auto comp = [&](u32 c) -> u32 {  // the region of comp c: its smallest comp
-      const u32 k = *tc_sb_byte<K>(m.rec, K::R_CNODE, c, hl);
-      return k == 255u ? c : (u32)*tc_sb_byte<K>(m.rec, K::R_NCOMP, (u32)(low >> (4 * k)) & 15u, hl);
-    };
-    u32 alive = 0;
-    for (u32 c = 0; c < C; ++c) {
-      if (comp(c) != c) continue;
-      alive |= 1u << c;
-      if (c) par[(c >> 2) * 4 * K::T + (c & 3u)] = (u8)comp(*tc_sb_byte<K>(m.rec, K::R_CPAR, c, hl));
+    rest &= ~eq;
+    const u32 at = atomicAdd(m.queued, 1u);
+    if (at < K::QUEUE) {
+      m.queue[4 * at] = (u32)low;
+      m.queue[4 * at + 1] = (u32)(low >> 32);
+      m.queue[4 * at + 2] = hl | (rootn << 16);
+      m.queue[4 * at + 3] = (u32)__popc(eq);
+    } else {
+      tc_sb_deep<K>(m, t, hl, low, rootn, (u32)__popc(eq), out, err, failed);
     }
-    const u32 root = *tc_sb_byte<K>(m.rec, K::R_NCOMP, rootn, hl);
-    const u64 key = tc_sl_tree_code<K::T, 4 * K::T, K::RMAX>(par, m.s.lab + t, alive, root, err);
-    if (key)
-      tc_sb_insert<K::HASH>(key, 1, out.hkeys, out.hcnt, out.gkeys, out.gcnt, out.gslots, out.gerr);
-    else
-      ++failed;
   }
 }
+
+#ifndef TC_SL_EMULATE
+// Barrier; then code the queued trees when there are enough of them for the
+// block's lanes, or (last) all of them.  All threads call it.  The choice is
+// one for the block: a thread that went on may already queue trees of its next
+// word, so it is thread 0's look before the barrier, not each thread's after it.
+template <class K>
+__device__ __forceinline__ void tc_sb_flush_queue(const TcSbMem &m, u32 t, bool last, const TcSbOut &out,
+                                                  u32 &err, unsigned long long &failed) {
+  volatile u32 *const queued = m.queued;
+  if (!__syncthreads_or(last || (t == 0 && *queued >= K::QUEUE / 2))) return;
+  u32 nq = *queued;
+  if (nq > K::QUEUE) nq = K::QUEUE;
+  for (u32 i = t; i < nq; i += K::T) {
+    const u32 *const q = m.queue + 4 * i;
+    tc_sb_deep<K>(m, t, q[2] & 0xFFFFu, ((u64)q[1] << 32) | q[0], q[2] >> 16, q[3], out, err, failed);
+  }
+  __syncthreads();
+  if (t == 0) *queued = 0;
+  __syncthreads();
+}
+#endif

@@ -7,6 +7,7 @@
 // the per-mask phases).
 #define TC_SL_NO_MAIN
 #include "run_sliced_sweep.cpp"
+static inline unsigned atomicAdd(unsigned *p, unsigned v) { auto o = *p; *p += v; return o; }
 #include "tc_block_sweep.cuh"
 #include <string>
 
@@ -72,16 +73,25 @@ int run_blocks(const char *edge_file, const std::string &mode, uint64_t seed) {
     if (!((M.rec[K::R_HDR * K::T + hl] >> 25) & 1u)) continue;
     ++valid;
     std::vector<u64> hk(K::HASH, 0), gk(16, 0);
-    std::vector<unsigned long long> hc(K::HASH, 0), gc(16, 0);
+    std::vector<u32> hc(K::HASH, 0);
+    std::vector<unsigned long long> gc(16, 0);
     u32 gerr = 0, err = 0;
     unsigned long long failed = 0;
     for (u32 i = 0; i < K::STARS; ++i) M.stars[i] = 0;
+    *M.queued = 0;
     const TcSbOut out{hk.data(), hc.data(), gk.data(), gc.data(), 16, &gerr};
     const u32 N = (M.rec[K::R_HDR * K::T + hl] >> 8) & 255u;
     for (u32 w = 0; w < (1u << ib) / 32; ++w) {
       const u32 th = (hl * 7 + w) % K::T;
       if (N <= K::NA && w % 2) tc_sb_middle<K, K::NA>(M, th, hl, w, ishift, out, err, failed);
       else tc_sb_middle<K, K::NB>(M, th, hl, w, ishift, out, err, failed);
+      if (w % 4 == 3 || w + 1 == (1u << ib) / 32) {  // the kernel's queue of deep trees
+        for (u32 i = 0; i < std::min(*M.queued, K::QUEUE); ++i) {
+          const u32 *const q = M.queue + 4 * i;
+          tc_sb_deep<K>(M, i % K::T, q[2] & 0xFFFFu, ((u64)q[1] << 32) | q[0], q[2] >> 16, q[3], out, err, failed);
+        }
+        *M.queued = 0;
+      }
     }
     std::map<u64, unsigned long long> got, want;
     for (u32 s = 0; s < K::HASH; ++s)
