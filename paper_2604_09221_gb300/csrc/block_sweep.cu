@@ -32,8 +32,8 @@ __global__ void __launch_bounds__(128, D <= 7 ? 3 : 2)
   u32 *const tab = reinterpret_cast<u32 *>(smem);
   u32 *const area = reinterpret_cast<u32 *>(smem + toff + 128);
   unsigned long long *const slot = reinterpret_cast<unsigned long long *>(smem + toff + 64);
-  const TcSbMem M = tc_sb_carve<K>(tab, area, L.chunks, L.far);
-  u64 *const hkeys = reinterpret_cast<u64 *>(area + tc_sb_words<K>(L.chunks, L.far));
+  const TcSbMem M = tc_sb_carve<K>(tab, area, L.chunks);
+  u64 *const hkeys = reinterpret_cast<u64 *>(area + tc_sb_words<K>(L.chunks));
   u32 *const hcnt = reinterpret_cast<u32 *>(hkeys + K::HASH);
   const TcSbOut out{hkeys, hcnt, reinterpret_cast<u64 *>(h.d_keys), h.d_counts, h.slots, h.d_err};
   const u32 t = threadIdx.x, mine = tc_sl_instance<B>(t), lw = ib - 5u;
@@ -74,8 +74,6 @@ __global__ void __launch_bounds__(128, D <= 7 ? 3 : 2)
     tc_sl_planes<B>(M.s, TcSig<1>{{base + t < n_hi ? mask_of(base + t) : 0ull}}, t);
     __syncthreads();
     tc_sl_logic<B>(M.s, t);
-    __syncthreads();
-    tc_sl_labels_halves<B>(M.s, t);
     __syncthreads();
     tc_sl_tiles<B>(M.s, t);
     tc_sl_events<B>(M.s, t);
@@ -131,7 +129,7 @@ cudaError_t launch_d(const ts_tri *t, uint64_t h0, uint64_t n, const Split &s, u
                      cudaStream_t st) {
   typedef TcSbK<D> K;
   const size_t smem = (t->slay.words * 4 + 127) / 128 * 128 + 128 +
-                      (size_t)tc_sb_words<K>(t->slay.chunks, t->slay.far) * 4 + (size_t)K::HASH * 16;
+                      (size_t)tc_sb_words<K>(t->slay.chunks) * 4 + (size_t)K::HASH * 16;
   cudaError_t e = cudaFuncSetAttribute(block_sweep_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kMaxBlockSmem);
   int per_sm = 0, sms = 0, dev = 0;

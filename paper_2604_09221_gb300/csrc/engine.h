@@ -51,7 +51,6 @@ struct WarpLayout {
 struct SlicedLayout {
   uint32_t words;   // padded to a multiple of 4
   uint32_t chunks;  // event chunks of 32: label starts, joins, boundary edges
-  uint32_t far;     // steps of four fan entries beyond a vertex's row of planes
 };
 // Device error word bits.
 enum : uint32_t {

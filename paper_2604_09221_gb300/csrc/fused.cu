@@ -243,7 +243,7 @@ int fused_tier(int d) {
 size_t fused_area_bytes(int d, const SlicedLayout &l) {
   switch (d) {
 #define TC_AREA(x) \
-  case x: return (size_t)tc_sl_words<TcSlK<x, (int)kFT / 32>>(l.chunks, l.far) * 4;
+  case x: return (size_t)tc_sl_words<TcSlK<x, (int)kFT / 32>>(l.chunks) * 4;
     TC_AREA(1) TC_AREA(2) TC_AREA(3) TC_AREA(4) TC_AREA(5) TC_AREA(6) TC_AREA(7) TC_AREA(8) TC_AREA(9)
     TC_AREA(10) TC_AREA(11) TC_AREA(12) TC_AREA(13) TC_AREA(14) TC_AREA(15) TC_AREA(16)
 #undef TC_AREA

@@ -343,20 +343,14 @@ bool pack_sliced_tables(const Diamond &D, std::vector<uint32_t> &tables, SlicedL
   const int V = D.V, d = D.d, H = d * d;  // [0, H) lower half, [H, 2H) upper half, then the middle row
   const uint32_t ncb = ((uint32_t)V + 31) / 32;
   std::vector<uint32_t> fan, vd(V), first(V), site0(V, 0), half_sites, mid_sites;
-  uint32_t half_steps[2] = {0, 0}, far = 0, half_far[2] = {0, 0};
-  // steps whose takes fit the vertex's row of label planes (TcSlK::TW / 4)
-  const size_t near = V <= 256 ? 2 : 4;
+  uint32_t half_steps[2] = {0, 0};
   auto can_join = [&](int v, size_t i) { return i >= 2 || (i == 1 && !D.link[v][1]); };
   for (int v = 0; v < V; ++v) {
-    if (v == H || v == 2 * H) {
-      half_steps[v / H - 1] = (uint32_t)fan.size() / 4;
-      half_far[v / H - 1] = far;
-    }
+    if (v == H || v == 2 * H) half_steps[v / H - 1] = (uint32_t)fan.size() / 4;
     const size_t len = D.fan[v].size(), padded = len ? (len + 3) / 4 * 4 : 4;
     if (len > 255 || fan.size() > 0xFFFF || D.k[v] > 255) return false;
     first[v] = (uint32_t)fan.size();
-    vd[v] = (len ? (uint32_t)D.fan[v][0] | 1u << 15 : 0u) | (far << 16);
-    if (padded / 4 > near) far += (uint32_t)(padded / 4 - near);
+    vd[v] = len ? (uint32_t)D.fan[v][0] | 1u << 15 : 0u;
     for (size_t i = 0; i < D.fan[v].size(); ++i) {
       const int u = D.fan[v][i];
       if (v < 2 * H && (u < H) != (v < H)) return false;  // no edge leaves a half-diamond
@@ -369,10 +363,9 @@ bool pack_sliced_tables(const Diamond &D, std::vector<uint32_t> &tables, SlicedL
     for (size_t i = len; i < padded; ++i) fan.push_back((uint32_t)D.k[v]);
   }
   // the half-diamonds are mirror images: as many steps each
-  if (half_steps[1] != 2 * half_steps[0] || half_far[1] != 2 * half_far[0] || far > 0xFFFF) return false;
+  if (half_steps[1] != 2 * half_steps[0]) return false;
   // chunks of joins: the half-diamonds', one of boundary pairs, the middle
-  // row's (with the corner pair of even d); at least as many as start chunks
-  if (d % 2 == 0) mid_sites.push_back(0);  // the corner pair, below
+  // row's; at least as many as start chunks
   uint32_t nc1 = ((uint32_t)half_sites.size() + 31) / 32;
   const uint32_t ncm = ((uint32_t)mid_sites.size() + 31) / 32;
   nc1 = std::max(nc1, ncb > ncm + 1 ? ncb - ncm - 1 : 0u);
@@ -398,12 +391,8 @@ bool pack_sliced_tables(const Diamond &D, std::vector<uint32_t> &tables, SlicedL
   for (int t = 0; t < 2 * d; ++t) {
     const int a = p[t], b = p[t + 1];            // edge t; if crossed, it joins
     const int x = p[t + 1], y = p[t + 1 + 2 * d];  // the pair behind it
-    uint32_t slot = 32 * (ncb + nc1) + (uint32_t)t;
-    uint32_t pair = (uint32_t)std::min(x, y) | ((uint32_t)std::max(x, y) << 16);
-    if (d % 2 == 0 && D.y[x] == 0) {  // the corner pair goes with the middle row, parity 1
-      slot = next_mid;
-      pair |= 1u << 31;
-    }
+    const uint32_t slot = 32 * (ncb + nc1) + (uint32_t)t;
+    const uint32_t pair = (uint32_t)std::min(x, y) | ((uint32_t)std::max(x, y) << 16);
     if (slot > 0x7FFF) return false;
     bx[t] = (uint32_t)D.k[a] | ((uint32_t)D.k[b] << 8) | ((uint32_t)(D.c[a] ^ D.c[b]) << 16) | (slot << 17);
     be[t] = (uint32_t)a | ((uint32_t)b << 16);
@@ -427,7 +416,6 @@ bool pack_sliced_tables(const Diamond &D, std::vector<uint32_t> &tables, SlicedL
   };
   tables[0] = half_steps[0];
   tables[8] = (uint32_t)fan.size() / 4;
-  tables[9] = half_far[0];
   tables[1] = nc1;
   tables[2] = ncb + nc1 + 1 + ncm;
   tables[3] = put(fan);
@@ -438,7 +426,6 @@ bool pack_sliced_tables(const Diamond &D, std::vector<uint32_t> &tables, SlicedL
   while (tables.size() % 4) tables.push_back(0);
   lay.words = (uint32_t)tables.size();
   lay.chunks = ncb + nc1 + 1 + ncm;
-  lay.far = far;
   return true;
 }
 }  // namespace tcurve

@@ -186,11 +186,15 @@ __global__ void __launch_bounds__(TableK<D, G>::THREADS)
 
 // ------------------------------------------------ bit-sliced kernels ----
 //
-// Blocks of 128 threads classify 128 sign vectors at a time (tc_sliced.cuh).
+// Blocks of 128 threads classify 128 sign vectors at a time (tc_sliced.cuh; 64
+// from d = 13).
 // smem: tables (toff bytes) | mbarrier, work slot (128 bytes) | the block's
 // areas | hash table (sweeps of one-word codes).
+// From d = 13 (130 to 210 KB for 128 sign vectors) blocks of 64:
+// what limits them is the blocks a multiprocessor's shared memory holds
+// (d = 13: three of 64, one of 128; 0.40 against 0.26e9 schemes/s).
 template <int D>
-using SlicedK = TcSlK<D, 4>;
+using SlicedK = TcSlK<D, D <= 12 ? 4 : 2>;
 
 template <class K>
 __global__ void __launch_bounds__(K::T)
@@ -230,7 +234,7 @@ __global__ void __launch_bounds__(K::T)
   u32 *const tab = reinterpret_cast<u32 *>(smem);
   u32 *const area = reinterpret_cast<u32 *>(smem + toff + 128);
   unsigned long long *const slot = reinterpret_cast<unsigned long long *>(smem + toff + 64);
-  u64 *const hkeys = reinterpret_cast<u64 *>(area + tc_sl_words<K>(L.chunks, L.far));
+  u64 *const hkeys = reinterpret_cast<u64 *>(area + tc_sl_words<K>(L.chunks));
   unsigned long long *const hcnt = reinterpret_cast<unsigned long long *>(hkeys + K::HASH);
   const u32 t = threadIdx.x, mine = tc_sl_instance<K>(t);
   for (u32 s = t; s < K::HASH; s += K::T) {
@@ -375,7 +379,7 @@ template <int D>
 cudaError_t real_schemes_sliced(const ts_tri *t, const uint64_t *signs, uint64_t n, uint64_t *codes,
                                 cudaStream_t st) {
   typedef SlicedK<D> K;
-  const size_t smem = sliced_table_bytes(t->slay.words) + 128 + (size_t)tc_sl_words<K>(t->slay.chunks, t->slay.far) * 4;
+  const size_t smem = sliced_table_bytes(t->slay.words) + 128 + (size_t)tc_sl_words<K>(t->slay.chunks) * 4;
   unsigned grid = 0;
   cudaError_t e = persistent_grid(sliced_real_schemes_kernel<K>, K::T, smem, (n + K::T - 1) / K::T, &grid);
   if (e != cudaSuccess) return e;
@@ -387,7 +391,7 @@ template <int D>
 cudaError_t enumerate_sliced(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *h,
                              cudaStream_t st) {
   typedef SlicedK<D> K;
-  const size_t smem = sliced_table_bytes(t->slay.words) + 128 + (size_t)tc_sl_words<K>(t->slay.chunks, t->slay.far) * 4 +
+  const size_t smem = sliced_table_bytes(t->slay.words) + 128 + (size_t)tc_sl_words<K>(t->slay.chunks) * 4 +
                       (size_t)K::HASH * 16;
   const uint64_t total = hi - lo;
   unsigned grid = 0;

@@ -87,20 +87,20 @@ __host__ __device__ constexpr u32 tc_sb_evwords(u32 chunks) {
 }
 
 template <class K>
-__host__ __device__ constexpr u32 tc_sb_words(u32 chunks, u32 far) {
-  return K::LAB + tc_sb_evwords<K>(chunks) + tc_sl_xwords<typename K::Base>(far) +
+__host__ __device__ constexpr u32 tc_sb_words(u32 chunks) {
+  return K::LAB + tc_sb_evwords<K>(chunks) + K::XW +
          K::R_WORDS * K::T + K::SW + K::STARS + 4;
 }
 
 template <class K>
-__device__ __forceinline__ TcSbMem tc_sb_carve(const u32 *tab, u32 *area, u32 chunks, u32 far) {
+__device__ __forceinline__ TcSbMem tc_sb_carve(const u32 *tab, u32 *area, u32 chunks) {
   TcSbMem m;
   m.s.tab = tab;
   m.s.lab = area;
   m.s.ev = m.s.lab + K::LAB;
   m.queue = m.s.ev;
   m.s.x = m.s.ev + tc_sb_evwords<K>(chunks);
-  m.rec = m.s.x + tc_sl_xwords<typename K::Base>(far);
+  m.rec = m.s.x + K::XW;
   m.scr = m.rec + K::R_WORDS * K::T;
   m.stars = m.scr + K::SW;
   m.queued = m.stars + K::STARS;
@@ -128,34 +128,27 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
   for (u32 c = (HB + 31) / 32; c < K::NCB; ++c) I.set_event(c, 0);
   const u32 be = (I.event(K::NCB + nc1) | 1u) & ((1u << (2 * K::D - 1)) - 1u);
   I.set_event(K::NCB + nc1, be);
-  u32 starts[K::NCB];
-#pragma unroll
-  for (u32 c = 0; c < K::NCB; ++c) starts[c] = I.event(c);
+  tc_sl_labels<typename K::Base>(I, 2 * K::H);
   tc_sl_joins<typename K::Base>(I, tab + tab[5], 0, nc1 + 1);
-  u32 C = 0;  // comps, numbered by their roots
-#pragma unroll
-  for (u32 c = 0; c < K::NCB; ++c) C += (u32)__popc(I.event(c));
   u32 *const rec = m.rec + t;
   rec[K::R_HDR * K::T] = 0;
-  if (C > 32) return;  // not valid: the block's masks one by one
-  // every label start gets its comp (a parent is smaller, so it has its comp
-  // already), marked by the top three bits, which no vertex number has set
-  static_assert(K::LB == 1 && K::V < 224, "comps marked in label bytes");
-  u32 chis = 0;  // chi of every comp modulo 2: label starts plus join events
-  C = 0;
+  // comps in the order of their smallest starts; chi of every comp modulo 2:
+  // label starts plus join events
+  static_assert(Inst::MARK + 32 <= 256, "32 comps in label bytes");
+  u32 C = 0;
+  {
+    u32 n = 0;  // roots, before they are numbered
 #pragma unroll
-  for (u32 c = 0; c < K::NCB; ++c)
-    for (u32 w = starts[c]; w; w &= w - 1u) {
-      const u32 v = 32u * c + (u32)__ffs(w) - 1u, p = I.raw(v);
-      const u32 id = p == v ? C : I.raw(p) & 31u;
-      C += p == v ? 1u : 0u;
-      I.set(v, 224u | id);
-      chis ^= 1u << id;
-    }
-  auto comp_of = [&](u32 v) -> u32 {
-    const u32 x = I.raw(v);
-    return (x < 224u ? I.raw(x) : x) & 31u;
-  };
+    for (u32 c = 0; c < K::NCB; ++c)
+      for (u32 w = I.event(c); w; w &= w - 1u) {
+        const u32 v = 32u * c + (u32)__ffs(w) - 1u;
+        n += I.raw(v) == v;
+      }
+    if (n > 32) return;  // not valid: the block's masks one by one
+  }
+  u32 chis = 0;
+  C = tc_sl_number<typename K::Base>(I, [&](u32 r) { chis ^= 1u << r; });
+  auto comp_of = [&](u32 v) -> u32 { return I.region(v); };
   {
     const u32 *const site = tab + tab[5];
     u32 c = 0, w = 0;

@@ -13,29 +13,30 @@
 //            bit transposes across the warp)
 //   logic    (vertex, group) per thread, vertices in order of fan length:
 //            for every fan entry the mask of the instances that take their
-//            label from it (first same-sign entry), per vertex the mask of
-//            the instances in which it starts a label, per entry that can
-//            start a second run the mask of the instances that have to join
-//   labels   the labels as bit planes, vertices in sweep order (the two
-//            half-diamonds side by side, then the middle row):
-//            L(v) = start(v) ? id(v) : OR over entries of take & L(u); a
-//            label's id is the vertex that starts it.  The takes of v lie
-//            where its planes will be (steps of longer fans: "far" steps, in
-//            the last area)
+//            label from it (first same-sign entry), hence the number of that
+//            neighbour (of the vertex itself if it starts a label) as bit
+//            planes; per vertex the mask of the instances in which it starts a
+//            label, per entry that can start a second run the mask of the
+//            instances that have to join
 //   tiles    planes -> one byte (d >= 11: half-word) per vertex and
 //            instance, in place; event masks -> one word per instance
+//   labels   one instance per thread: vertices in sweep order, every vertex
+//            gets the label of the neighbour its byte names (a label is the
+//            number of the vertex that starts it)
 //   trees    one instance per thread: joins in a union-find over the label
 //            bytes themselves (a vertex that starts a label points at itself),
-//            regions, region tree, root and code
+//            regions (whose numbers then replace the bytes of the starts),
+//            region tree, root and code
 //
 // Everything a block touches is in shared memory; nothing is allocated.
 //
-// Orientation parity (even d, Alg. 1 lines 6-7).  Before the middle row a set
-// of labels can mix the two half-diamonds only through antipodal pairs
-// (parity 1), so the parity between two labels is whether their halves
-// differ.  Links are stored relative to that: the half joins and the
-// antipodal joins need no parity at all, and only joins of the middle row
-// (and its corner pair) carry a "twist" bit.
+// Root of even degree (Alg. 1 lines 6-7), without orientation parities: a
+// region X that is a disk with holes has Euler number chi(X) = 2 - (its
+// neighbours in the region tree), the non-orientable region 1 less.  So the
+// root is the one region for which chi plus degree is odd; chi of a region
+// counts its label starts minus its join events (a vertex with k runs of
+// same-sign earlier neighbours adds 1 - k; identifying a run of boundary
+// vertices with its antipodes takes one away).
 //
 // Antipodal joins.  Consecutive boundary vertices of one sign are joined by
 // their boundary edge, and so are their antipodes; so a pair is joined only
@@ -50,7 +51,6 @@
 //   header   [0] steps of a half-diamond  [1] event chunks of half-diamond
 //            joins  [2] event chunks in all  [3] off_fan  [4] off_vd
 //            [5] off_site  [6] off_bx  [7] off_be  [8] steps in all
-//            [9] far steps of a half-diamond
 //   task[V]  two words per vertex, in order of fan length: k(v) (8 bits) |
 //            fan steps << 8 (8 bits) | first fan entry << 16, and
 //            v | first join site << 16
@@ -59,11 +59,9 @@
 //            u << 8 (16 bits) | "can start a second run" << 24 | "another step
 //            of this vertex follows" << 25 | link << 30 |
 //            (c(u) ^ c(v) ^ 1) << 31; padding: k(v), never of v's sign
-//   vd[V]    u of the first fan entry | "the fan is not empty" << 15 |
-//            first far step << 16
-//   site[]   32 per chunk of join events: v | u << 16 (| parity << 31 for the
-//            corner pair of even d): the half-diamonds' sites, one chunk of
-//            boundary pairs, the middle row's sites
+//   vd[V]    u of the first fan entry | "the fan is not empty" << 15
+//   site[]   32 per chunk of join events: v | u << 16: the half-diamonds'
+//            sites, one chunk of boundary pairs, the middle row's sites
 //   bx[2d]   k(a) | k(b) << 8 | (c(a) ^ c(b)) << 16 | event slot << 17 of the
 //            boundary edges of half the boundary, in cyclic order
 //   be[2d]   a | b << 16 of the same edges
@@ -80,16 +78,15 @@ struct TcSlK {
   static constexpr u32 LB = V <= 256 ? 1 : 2;     // bytes per label
   static constexpr u32 NPL = V <= 128 ? 7 : V <= 256 ? 8 : V <= 512 ? 9 : 10;  // label planes
   static constexpr u32 TW = 8 * LB;               // words of a vertex's tile per group
-  static constexpr u32 PP = NG >= 8 ? 4 : 2;      // planes per thread in the labels phase
-  static constexpr u32 PS = TW / PP;              // threads per group there
   static constexpr u32 NCB = (V + 31) / 32;       // birth chunks
   static constexpr bool EVEN = D % 2 == 0;
-  static constexpr bool TWTOP = LB == 2 || V <= 128;   // twist bit in the label's top bit
-  static constexpr u32 TWWORDS = EVEN && !TWTOP ? NCB : 0;  // else in words of their own
   static constexpr u32 LABW = V * TW * NG;        // words of the label area
   static constexpr u32 PAR_WORDS = (RMAX + 3) / 4 * T;  // region parents, a byte each
   static constexpr u32 PLANES = (NPOINTS * NG + 3) & ~3u;
-  static constexpr u32 BW = PAR_WORDS + TWWORDS * T;
+  // d = 10 (one-byte labels, more regions than spare byte values) keeps the
+  // roots' words apart from the starts' (NCB per thread)
+  static constexpr u32 ROOT_WORDS = LB == 1 && !(V < 224 && RMAX <= 32) ? NCB * T : 0;
+  static constexpr u32 XW = PLANES > PAR_WORDS + ROOT_WORDS ? PLANES : PAR_WORDS + ROOT_WORDS;
   // tree codes: the wide back end's scratch lies over the label area
   static constexpr u32 THREADS = T;
   static constexpr u32 WB = (RMAX + 3) / 4, WARENA = L.warena_words;
@@ -107,20 +104,14 @@ struct TcSlMem {
   const u32 *tab;  // staged tables
   u32 *lab;        // label planes, then label bytes (K::LABW words)
   u32 *ev;         // event chunks (chunks x NG x TC_SL_GROUP words)
-  u32 *x;          // sign planes and takes, then region parents and twists
+  u32 *x;          // sign planes, then region parents
 };
 
-// Words of the last area: sign planes and the takes of far steps (four per
-// step and group); in the trees phase region parents and twists.
+// Words of a block's areas behind the tables (chunks of events).  The last
+// area holds the sign planes, in the trees phase the region parents.
 template <class K>
-__host__ __device__ constexpr u32 tc_sl_xwords(u32 far) {
-  return ((K::PLANES + 4 * far * K::NG > K::BW ? K::PLANES + 4 * far * K::NG : K::BW) + 3) & ~3u;
-}
-
-// Words of a block's areas behind the tables (chunks of events, far steps).
-template <class K>
-__host__ __device__ constexpr u32 tc_sl_words(u32 chunks, u32 far) {
-  return K::LABW + chunks * K::NG * TC_SL_GROUP + tc_sl_xwords<K>(far);
+__host__ __device__ constexpr u32 tc_sl_words(u32 chunks) {
+  return K::LABW + chunks * K::NG * TC_SL_GROUP + K::XW;
 }
 
 template <class K>
@@ -219,34 +210,46 @@ __device__ __forceinline__ void tc_sl_logic(const TcSlMem &m, u32 t) {
     const u32 sv = P[(w.a & 255u) * K::NG], steps = (w.a >> 8) & 255u, v = w.b & 0xFFFFu;
     u32 site = w.b >> 16, any = 0, prev = 0;
     const TcQuad *f = reinterpret_cast<const TcQuad *>(fan + (w.a >> 16));
-    TcQuad *take = reinterpret_cast<TcQuad *>(m.lab + (v * K::NG + g) * K::TW);
+    u32 plane[K::NPL];  // of the number of the vertex the label comes from
+#pragma unroll
+    for (u32 i = 0; i < K::NPL; ++i) plane[i] = 0;
+    auto from = [&](u32 mask, u32 u) {
+#pragma unroll
+      for (u32 i = 0; i < K::NPL; ++i)
+        if (u & (1u << i)) plane[i] |= mask;
+    };
     for (u32 j = 0; j < steps; ++j, ++f) {
-      if (j >= K::TW / 4)  // a far step
-        take = reinterpret_cast<TcQuad *>(m.x + K::PLANES) +
-               ((m.tab[m.tab[4] + v] >> 16) + j - K::TW / 4) * K::NG + g;
       const TcQuad q = *f;
       // the four entries' masks "same sign as v"
       const u32 ea = P[(q.a & 255u) * K::NG] ^ sv ^ (u32)((int)q.a >> 31);
       const u32 eb = P[(q.b & 255u) * K::NG] ^ sv ^ (u32)((int)q.b >> 31);
       const u32 ec = P[(q.c & 255u) * K::NG] ^ sv ^ (u32)((int)q.c >> 31);
       const u32 ed = P[(q.d & 255u) * K::NG] ^ sv ^ (u32)((int)q.d >> 31);
-      TcQuad o;
-      auto entry = [&](u32 f, u32 e) -> u32 {
+      auto entry = [&](u32 f, u32 e) {
         if (f & (1u << 24)) {  // a run that may follow another one
           *tc_sl_event<K>(m, site, g) = e & any & ~(prev & tc_bitmask(f, 30));
           ++site;
         }
-        const u32 x = e & ~any;
+        from(e & ~any, f >> 8);
         any |= e;
         prev = e;
-        return x;
       };
-      o.a = entry(q.a, ea);
-      o.b = entry(q.b, eb);
-      o.c = entry(q.c, ec);
-      o.d = entry(q.d, ed);
-      *take = o;
-      ++take;
+      entry(q.a, ea);
+      entry(q.b, eb);
+      entry(q.c, ec);
+      entry(q.d, ed);
+    }
+    from(~any, v);
+    u32 *const out = m.lab + (v * K::NG + g) * K::TW;
+    if constexpr (K::LB == 1) {
+      TcQuad *const o = reinterpret_cast<TcQuad *>(out);
+      o[0] = TcQuad{plane[0], plane[1], plane[2], plane[3]};
+      o[1] = TcQuad{plane[4], plane[5], plane[6], K::NPL > 7 ? plane[K::NPL - 1] : 0u};
+    } else {
+      TcQuad *const o = reinterpret_cast<TcQuad *>(out);
+      o[0] = TcQuad{plane[0], plane[1], plane[2], plane[3]};
+      o[1] = TcQuad{plane[4], plane[5], plane[6], plane[7]};
+      o[2] = TcQuad{plane[8], K::NPL > 9 ? plane[K::NPL - 1] : 0u, 0u, 0u};
     }
     *tc_sl_event<K>(m, v, g) = ~any;  // v starts a label
   }
@@ -256,111 +259,6 @@ __device__ __forceinline__ void tc_sl_logic(const TcSlMem &m, u32 t) {
     const u32 w = bx[k];
     *tc_sl_event<K>(m, w >> 17, g) = P[(w & 255u) * K::NG] ^ P[((w >> 8) & 255u) * K::NG] ^ tc_bitmask(w, 16);
   }
-}
-
-// ---- labels: steps [s0, s1), vertices from v and far steps from `far` on,
-// K::PP planes per thread ----
-// A serial chain from vertex to vertex: the fan entries and takes of the next
-// step, which do not depend on it, are loaded a step ahead.  The threads of a
-// group are in one warp: they have all read a vertex's takes before one of
-// them writes its planes over them (mask: the warp's threads in this call).
-template <u32 PP>
-struct TcPlanes;
-template <>
-struct TcPlanes<2> {
-  typedef TcPair T;
-  static __device__ __forceinline__ void acc(u32 (&a)[2], u32 s, const T &p) {
-    a[0] |= s & p.a;
-    a[1] |= s & p.b;
-  }
-  static __device__ __forceinline__ T out(const u32 (&a)[2]) { return T{a[0], a[1]}; }
-};
-template <>
-struct TcPlanes<4> {
-  typedef TcQuad T;
-  static __device__ __forceinline__ void acc(u32 (&a)[4], u32 s, const T &p) {
-    a[0] |= s & p.a;
-    a[1] |= s & p.b;
-    a[2] |= s & p.c;
-    a[3] |= s & p.d;
-  }
-  static __device__ __forceinline__ T out(const u32 (&a)[4]) { return T{a[0], a[1], a[2], a[3]}; }
-};
-
-template <class K>
-__device__ __forceinline__ void tc_sl_label_run(const TcSlMem &m, u32 g, u32 part, u32 s0, u32 s1, u32 v,
-                                                u32 far, u32 mask) {
-  typedef TcPlanes<K::PP> PL;
-  typedef typename PL::T plane_t;
-  constexpr u32 ROW = K::TW * K::NG * 4;  // bytes per vertex
-  constexpr u32 NEAR = K::TW / 4;         // steps whose takes lie in the vertex's row
-  const TcQuad *fan = reinterpret_cast<const TcQuad *>(m.tab + m.tab[3]) + s0;
-  u8 *const L = reinterpret_cast<u8 *>(m.lab + g * K::TW + K::PP * part);
-  const TcQuad *ft = reinterpret_cast<const TcQuad *>(m.x + K::PLANES) + far * K::NG + g;
-  u32 row = v * ROW;
-  const u8 *const T = reinterpret_cast<const u8 *>(m.lab + g * K::TW);
-  auto planes = [&](u32 f) -> const plane_t & {
-    return *reinterpret_cast<const plane_t *>(L + ((f >> 8) & 0xFFFFu) * ROW);
-  };
-  TcQuad f = fan[0], s = *reinterpret_cast<const TcQuad *>(T + row);
-  u32 a[K::PP] = {}, any = 0, j = 0;
-  for (u32 n = s1 - s0; n; --n) {
-    const TcQuad sc = s;
-    const bool more = f.a & (1u << 25);  // another step of this vertex
-    const plane_t p0 = planes(f.a), p1 = planes(f.b), p2 = planes(f.c), p3 = planes(f.d);
-    const u32 here = row;
-    j = more ? j + 1 : 0;
-    row += more ? 0 : ROW;
-    // one step past the last one read here is still inside the areas (the
-    // tables' next part; the event chunks behind the labels)
-    f = *++fan;
-    if (j < NEAR) {
-      s = *reinterpret_cast<const TcQuad *>(T + row + 16 * j);
-    } else {
-      s = *ft;
-      ft += K::NG;
-    }
-    __syncwarp(mask);
-    PL::acc(a, sc.a, p0);
-    PL::acc(a, sc.b, p1);
-    PL::acc(a, sc.c, p2);
-    PL::acc(a, sc.d, p3);
-    any |= sc.a | sc.b | sc.c | sc.d;
-    if (!more) {
-#pragma unroll
-      for (u32 i = 0; i < K::PP; ++i) a[i] |= tc_bitmask(v, K::PP * part + i) & ~any;
-      *reinterpret_cast<plane_t *>(L + here) = PL::out(a);
-#pragma unroll
-      for (u32 i = 0; i < K::PP; ++i) a[i] = 0;
-      ++v;
-      any = 0;
-    }
-  }
-}
-
-// Thread t's planes, group and half-diamond (half > 1: none).
-template <class K>
-__device__ __forceinline__ void tc_sl_label_thread(u32 t, u32 &half, u32 &g, u32 &pair) {
-  pair = t % K::PS;
-  g = (t / K::PS) % K::NG;
-  half = t / (K::PS * K::NG);
-}
-__device__ __forceinline__ constexpr u32 tc_lanes(u32 n) { return n >= 32 ? 0xffffffffu : (1u << n) - 1u; }
-
-template <class K>
-__device__ __forceinline__ void tc_sl_labels_halves(const TcSlMem &m, u32 t) {
-  u32 half, g, pair;
-  tc_sl_label_thread<K>(t, half, g, pair);
-  if (half < 2)
-    tc_sl_label_run<K>(m, g, pair, half * m.tab[0], (half + 1) * m.tab[0], half * K::H, half * m.tab[9],
-                       tc_lanes(2 * K::PS * K::NG));
-}
-template <class K>
-__device__ __forceinline__ void tc_sl_labels_middle(const TcSlMem &m, u32 t) {
-  u32 half, g, pair;
-  tc_sl_label_thread<K>(t, half, g, pair);
-  if (half == 0)
-    tc_sl_label_run<K>(m, g, pair, 2 * m.tab[0], m.tab[8], 2 * K::H, 2 * m.tab[9], tc_lanes(K::PS * K::NG));
 }
 
 // ---- tiles ----
@@ -432,83 +330,55 @@ struct TcSlLab<2> {
 template <class K>
 struct TcSlInst {
   typedef typename TcSlLab<K::LB>::T lab_t;
-  static constexpr u32 TOP = K::LB == 1 ? 0x80u : 0x8000u;
-  static constexpr u32 LOW = K::EVEN && K::TWTOP ? TOP - 1u : 2u * TOP - 1u;
   static constexpr u32 ROW = K::T;  // labels per vertex
+  // A start's region number replaces its label byte, marked by bits that no
+  // vertex number has set; at d = 10 there are too few spare numbers, and a
+  // start is told by its event bit.
+  static constexpr u32 MARK = K::LB == 2 ? 0x8000u : K::V < 224 && K::RMAX <= 32 ? 224u : 0u;
   lab_t *l;
-  const u32 *ev;
+  u32 *ev;
   u8 *par;  // region r: byte r % 4 of word r / 4
-  u32 *tw;
   __device__ __forceinline__ TcSlInst(const TcSlMem &m, u32 t) {
     constexpr u32 WR = K::TW * K::NG;
     const u32 i = tc_sl_instance<K>(t);
     l = reinterpret_cast<lab_t *>(m.lab + t % WR) + t / WR;
     ev = m.ev + (i >> 5) * TC_SL_GROUP + (i & 31u);
     par = reinterpret_cast<u8 *>(m.x + t);
-    tw = m.x + K::PAR_WORDS + t;
+  }
+  // roots among the starts of chunk c: over the starts' word, but at d = 10
+  __device__ __forceinline__ u32 *root_word(u32 c) const {
+    return MARK ? ev + c * (K::NG * TC_SL_GROUP) : reinterpret_cast<u32 *>(par) + K::PAR_WORDS + c * K::T;
   }
   __device__ __forceinline__ u8 &parent(u32 r) const { return par[(r >> 2) * 4 * K::T + (r & 3u)]; }
-  __device__ __forceinline__ u32 *event_word(u32 v) const {
-    return const_cast<u32 *>(ev) + (v >> 5) * (K::NG * TC_SL_GROUP);
-  }
-  // label start x is no root any more
-  __device__ __forceinline__ void drop(u32 x) const { *event_word(x) &= ~(1u << (x & 31u)); }
-  // region of root x: the roots before it (rank kept per chunk in the first
-  // join chunks)
-  __device__ __forceinline__ u32 region(u32 x) const {
-    return event(K::NCB + (x >> 5)) + (u32)__popc(event(x >> 5) & ((1u << (x & 31u)) - 1u));
-  }
   __device__ __forceinline__ u32 raw(u32 v) const { return l[v * ROW]; }
   __device__ __forceinline__ void set(u32 v, u32 x) const { l[v * ROW] = (lab_t)x; }
-  __device__ __forceinline__ u32 lab(u32 v) const { return raw(v) & LOW; }
   __device__ __forceinline__ u32 event(u32 chunk) const { return ev[chunk * (K::NG * TC_SL_GROUP)]; }
-  __device__ __forceinline__ void set_event(u32 chunk, u32 w) const {
-    const_cast<u32 *>(ev)[chunk * (K::NG * TC_SL_GROUP)] = w;
-  }
-  __device__ __forceinline__ u32 root(u32 x) const {
-    u32 y = lab(x);
-    while (y != x) {
-      x = y;
-      y = lab(x);
-    }
-    return x;
-  }
-  // Whether vertex x's label started in the upper half-diamond; starts: the
-  // middle row's vertices that start a label themselves (their entries may be
-  // links by now).
-  __device__ __forceinline__ u32 upper(u32 x, u64 starts) const {
-    if (x >= 2 * K::H) x = (starts >> (x - 2 * K::H)) & 1ull ? x : lab(x);
-    return x - K::H < K::H ? 1u : 0u;
-  }
-  __device__ __forceinline__ u64 middle_starts() const {
-    constexpr u32 c = 2 * K::H / 32, sh = 2 * K::H % 32;
-    u64 b = event(c) >> sh;
-    if constexpr (c + 1 < K::NCB) b |= (u64)event(c + 1) << (32 - sh);
-    if constexpr (c + 2 < K::NCB) b |= sh ? (u64)event(c + 2) << (64 - sh) : 0ull;
-    return b;
-  }
-  // root of vertex x's set and the twist of the path to it
-  __device__ __forceinline__ u32 root_twist(u32 x, u32 &q) const {
-    for (;;) {
-      const u32 e = raw(x), y = e & LOW;
-      if (y == x) return x;
-      if constexpr (K::TWTOP)
-        q ^= (e & TOP) ? 1u : 0u;
-      else
-        q ^= (tw[(x >> 5) * K::T] >> (x & 31u)) & 1u;
-      x = y;
-    }
-  }
-  __device__ __forceinline__ void link(u32 hi, u32 lo, u32 q) const {
-    drop(hi);
-    if constexpr (K::TWTOP) {
-      set(hi, lo | (q ? TOP : 0u));
-    } else {
-      set(hi, lo);
-      if (q) tw[(hi >> 5) * K::T] |= 1u << (hi & 31u);
-    }
+  __device__ __forceinline__ void set_event(u32 chunk, u32 w) const { ev[chunk * (K::NG * TC_SL_GROUP)] = w; }
+  // region of vertex v, once the starts up to it (or its label) have theirs
+  __device__ __forceinline__ u32 region(u32 v) const {
+    const u32 x = raw(v);
+    if constexpr (MARK != 0)
+      return (x < MARK ? raw(x) : x) - MARK;
+    else
+      return (event(v >> 5) >> (v & 31u)) & 1u ? x : raw(x);
   }
 };
+
+// ---- labels: vertices [0, n) in sweep order ----
+// A vertex's neighbour comes before it, so that one's entry is its label
+// already.  Four vertices' entries are loaded ahead of their labels.
+template <class K>
+__device__ __forceinline__ void tc_sl_labels(const TcSlInst<K> &I, u32 n) {
+  u32 v = 0;
+  for (; v + 4 <= n; v += 4) {
+    u32 p[4];
+#pragma unroll
+    for (u32 i = 0; i < 4; ++i) p[i] = I.raw(v + i);
+#pragma unroll
+    for (u32 i = 0; i < 4; ++i) I.set(v + i, I.raw(p[i]));
+  }
+  for (; v < n; ++v) I.set(v, I.raw(I.raw(v)));
+}
 
 // Joins of the event chunks [c0, c1) without parity.  The next event and its
 // two labels are loaded before the present join's roots are known (a label
@@ -537,123 +407,134 @@ __device__ __forceinline__ void tc_sl_joins(const TcSlInst<K> &I, const u32 *sit
       a = I.raw(pa);
       b = I.raw(pb);
     } while (a != pa || b != pb);
-    if (a != b) {
-      const u32 hi = a < b ? b : a;
-      I.set(hi, a < b ? a : b);
-      I.drop(hi);
-    }
+    if (a != b) I.set(a < b ? b : a, a < b ? a : b);
     if (!more) return;
   }
 }
 
-// The middle row's joins of even degree, with parity: odd1 / odd2 receive
-// labels of the first and last set found to hold an odd antipodal cycle.
-template <class K>
-__device__ __forceinline__ void tc_sl_joins_twisted(const TcSlInst<K> &I, const u32 *site, u32 c0, u32 c1,
-                                                    u32 &odd1, u32 &odd2) {
-  const u64 starts = I.middle_starts();
-  u32 c = c0, w = 0;
-  for (;;) {
+// Region numbers in the order of the regions' smallest labels: every start
+// gets its region (a parent is smaller, so it has its region already), and
+// the roots' words the starts that are roots.  on_start(r): called for every
+// start with its region.  Returns the number of regions.
+template <class K, class F>
+__device__ __forceinline__ u32 tc_sl_number(const TcSlInst<K> &I, F on_start) {
+  constexpr u32 MARK = TcSlInst<K>::MARK;
+  u32 R = 0, left = 0;
+#pragma unroll
+  for (u32 c = 0; c < K::NCB; ++c) left += (u32)__popc(I.event(c));
+  u32 c = 0, w = 0, roots = 0;
+  for (; left; --left) {
     while (w == 0) {
-      if (c == c1) return;
-      w = I.event(K::NCB + c++);
+      if (c) *I.root_word(c - 1u) = roots;
+      roots = 0;
+      w = I.event(c++);
     }
-    const u32 s = site[32u * (c - 1u) + (u32)__ffs(w) - 1u];
+    const u32 bit = (u32)__ffs(w) - 1u, v = 32u * (c - 1u) + bit;
     w &= w - 1u;
-    const u32 v = s & 0xFFFFu, u = (s >> 16) & 0x7FFFu;
-    // parity asked for, relative to the halves of the two labels
-    u32 q = (s >> 31) ^ I.upper(v, starts) ^ I.upper(u, starts);
-    const u32 ra = I.root_twist(v, q), rb = I.root_twist(u, q);
-    if (ra != rb) {
-      I.link(ra < rb ? rb : ra, ra < rb ? ra : rb, q);
-    } else if (q) {
-      if (odd1 == ~0u) odd1 = ra;
-      odd2 = ra;
-    }
+    const u32 p = I.raw(v);
+    const bool is_root = p == v;
+    const u32 x = is_root ? MARK + R : I.raw(p);
+    I.set(v, x);
+    on_start(x - MARK);
+    roots |= is_root ? 1u << bit : 0u;
+    R += is_root;
   }
+  *I.root_word(c - 1u) = roots;
+  return R;
 }
 
 // Joins, regions and the region tree of one instance.  Returns the number of
-// regions R (0: failed, err set) with their parents in I.par (par[r] < r,
-// r >= 1) and the region the tree is rooted at; star: every oval is
-// outermost.
+// regions R (0: failed, err set) with their parents in I.parent(r) (< r, r >=
+// 1) and the region the tree is rooted at; star (narrow back end): every oval
+// is outermost.
 template <class K>
 __device__ __forceinline__ u32 tc_sl_regions(const TcSlMem &m, const TcSlInst<K> &I, u32 &root, bool &star,
                                              u32 &err) {
   const u32 *const tab = m.tab;
   const u32 *const site = tab + tab[5];
   const u32 nc1 = tab[1], nc = tab[2] - K::NCB;
-  u32 rv = ~0u;  // a label of the root's set
-  if constexpr (K::EVEN) {
-#pragma unroll
-    for (u32 w = 0; w < K::TWWORDS; ++w) I.tw[w * K::T] = 0;
-    tc_sl_joins<K>(I, site, 0, nc1 + 1);
-    u32 odd2 = ~0u;
-    tc_sl_joins_twisted<K>(I, site, nc1 + 1, nc, rv, odd2);
-    if (rv == ~0u || I.root(rv) != I.root(odd2)) {  // exactly one odd set
-      err |= TC_ERR_INTERNAL;
-      return 0;
+  tc_sl_joins<K>(I, site, 0, nc);
+  // chi + degree of the regions modulo 2, a bit each (even d)
+  u64 odd = 0, odd1 = 0;
+  auto toggle = [&](u32 r) {
+    if constexpr (K::RMAX <= 32) {
+      odd ^= 1u << (r & 31u);
+    } else if constexpr (K::RMAX <= 64) {
+      odd ^= 1ull << (r & 63u);
+    } else {
+      const u64 b = 1ull << (r & 63u);
+      odd ^= r < 64u ? b : 0ull;
+      odd1 ^= r < 64u ? 0ull : b;
     }
-    rv = I.root(rv);
+  };
+  u32 R;
+  if constexpr (K::EVEN) {
+    R = tc_sl_number<K>(I, toggle);
+    u32 c = 0, w = 0;
+    for (;;) {
+      while (w == 0 && c < nc) w = I.event(K::NCB + c++);
+      if (w == 0) break;
+      const u32 s = site[32u * (c - 1u) + (u32)__ffs(w) - 1u];
+      w &= w - 1u;
+      toggle(I.region(s & 0xFFFFu));
+    }
   } else {
-    tc_sl_joins<K>(I, site, 0, nc);
+    R = tc_sl_number<K>(I, [](u32) {});
     // the pseudoline's region: both ends of a crossed boundary edge in one
     // region; the near end of a crossed edge is in the region of the far end
     // of the one before
     const u32 *const be = tab + tab[7];
-    u32 prev = I.root(be[0] & 0xFFFFu);
+    u32 prev = I.region(be[0] & 0xFFFFu), rv = ~0u;
     bool two = false;
     for (u32 w = I.event(K::NCB + nc1); w; w &= w - 1u) {
-      const u32 a = I.root(be[(u32)__ffs(w) - 1u] >> 16);
-      if (a == prev) {
-        two |= rv != ~0u && rv != a;
-        rv = a;
-      }
+      const u32 a = I.region(be[(u32)__ffs(w) - 1u] >> 16);
+      two |= a == prev && rv != ~0u && rv != a;
+      rv = a == prev ? a : rv;
       prev = a;
     }
-    if (two) {
+    if (two || rv == ~0u) {
       err |= TC_ERR_INTERNAL;
       return 0;
     }
-    if (rv == ~0u) {
-      err |= TC_ERR_INTERNAL;
-      return 0;
-    }
-  }
-  // regions in the order of their smallest label: the starts that are still
-  // roots, counted chunk by chunk (the join chunks are used up)
-  u32 R = 0;
-#pragma unroll
-  for (u32 c = 0; c < K::NCB; ++c) {
-    I.set_event(K::NCB + c, R);
-    R += (u32)__popc(I.event(c));
+    root = rv;
   }
   if (R > K::RMAX) {
     err |= TC_ERR_OVERFLOW;
     return 0;
   }
-  root = I.region(rv);
   // the tree hanging from region 0: the parent of region r is the region of
   // the first earlier neighbour of its smallest label's vertex
   const u32 *const vd = tab + tab[4];
-  star = true;
   bool bad = false;
-  u32 c = 0, w = 0;
+  u32 internal = 0, kids0 = 0, c = 0, w = 0;
   for (u32 r = 0; r < R; ++r) {
-    while (w == 0) w = I.event(c++);
+    while (w == 0) w = *I.root_word(c++);
     const u32 v = 32u * (c - 1u) + (u32)__ffs(w) - 1u;
     w &= w - 1u;
     if (r) {
-      const u32 d = vd[v], p = I.region(I.root(d & 0x7FFFu));
+      const u32 d = vd[v], p = I.region(d & 0x7FFFu);
       bad |= !(d & 0x8000u) || p >= r;  // no earlier neighbour, or not a tree
       I.parent(r) = (u8)p;
-      star &= p == (r == root ? 0u : root);
+      if constexpr (K::EVEN) {
+        toggle(r);
+        toggle(p);
+      }
+      if constexpr (!K::WIDE) {
+        internal |= 1u << (p & 31u);
+        kids0 |= p == 0 ? 1u << r : 0u;
+      }
     }
+  }
+  if constexpr (K::EVEN) {
+    bad |= __popcll(odd) + __popcll(odd1) != 1;
+    root = odd ? (u32)__ffsll(odd) - 1u : 63u + (u32)__ffsll(odd1);
   }
   if (bad) {
     err |= TC_ERR_INTERNAL;
     return 0;
   }
+  if constexpr (!K::WIDE)
+    star = !(internal & ~(1u | (1u << root))) && (root == 0 || kids0 == 1u << root);
   return R;
 }
 
@@ -773,15 +654,11 @@ __device__ __forceinline__ void tc_sl_classify(const TcSlMem &m, const TcSig<K::
   __syncthreads();
   tc_sl_logic<K>(m, t);
   __syncthreads();
-  tc_sl_labels_halves<K>(m, t);
-  if constexpr (2 * K::PS * K::NG <= 32) __syncwarp();  // one warp holds both halves
-  else __syncthreads();
-  tc_sl_labels_middle<K>(m, t);
-  __syncthreads();
   tc_sl_tiles<K>(m, t);
   tc_sl_events<K>(m, t);
   __syncthreads();
   const TcSlInst<K> I(m, t);
+  tc_sl_labels<K>(I, K::V);
   u32 root = 0;
   bool star = false;
   const u32 R = tc_sl_regions<K>(m, I, root, star, err);

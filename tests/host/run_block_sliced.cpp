@@ -45,11 +45,11 @@ int run_blocks(const char *edge_file, const std::string &mode, uint64_t seed) {
   const int np = (D + 1) * (D + 2) / 2;
   const uint64_t hmax = 1ull << (np - oshift - (oflags ? 2 : 0));
   const u32 *tab = t.host_stables.data();
-  const u32 words = tc_sb_words<K>(t.slay.chunks, t.slay.far);
+  const u32 words = tc_sb_words<K>(t.slay.chunks);
   std::vector<TcQuad> area(words / 4 + 2, TcQuad{0xA5A5A5A5u, 0xA5A5A5A5u, 0xA5A5A5A5u, 0xA5A5A5A5u});
   u32 *const base = reinterpret_cast<u32 *>(area.data());
   for (u32 i = words; i < 4 * area.size(); ++i) base[i] = 0xC3C3C3C3u;
-  const TcSbMem M = tc_sb_carve<K>(tab, base, t.slay.chunks, t.slay.far);
+  const TcSbMem M = tc_sb_carve<K>(tab, base, t.slay.chunks);
   const TcSlMem &m = M.s;
   std::vector<uint64_t> mask(K::T);
   for (u32 i = 0; i < K::T; ++i) {
@@ -63,7 +63,7 @@ int run_blocks(const char *edge_file, const std::string &mode, uint64_t seed) {
       for (u32 i = 0; i < 32; ++i) x |= (u32)((mask[32 * g + i] >> k) & 1) << i;
       m.x[k * B::NG + g] = x;
     }
-  emulate_labels<B>(m, false);
+  for (u32 i = 0; i < K::T; ++i) tc_sl_logic<B>(m, i);
   for (u32 i = 0; i < K::T; ++i) tc_sl_tiles<B>(m, i);
   emulate_events<B>(m, t.slay.chunks);
   for (u32 i = 0; i < K::T; ++i) tc_sb_record<K>(M, i, mask[tc_sl_instance<B>(i)]);

@@ -9,7 +9,6 @@
 #include "run_table_sweep.cpp"
 #undef main
 #define TC_SL_EMULATE
-static inline void __syncwarp(unsigned) {}
 #include "tc_sliced.cuh"
 
 static uint64_t special(int d, int which, u32 w) {
@@ -22,34 +21,6 @@ static uint64_t special(int d, int which, u32 w) {
       if (b[which] && (u32)(k >> 6) == w) x |= 1ull << (k & 63);
     }
   return x;
-}
-
-// The logic and labels phases (middle: the middle row too).
-template <class K>
-static void emulate_labels(const TcSlMem &m, bool middle) {
-  for (u32 i = 0; i < K::T; ++i) tc_sl_logic<K>(m, i);
-  // the threads of a group share a vertex's takes before they write its
-  // planes over them: each runs on the takes as they were, and its planes
-  // are collected
-  std::vector<u32> takes(m.lab, m.lab + K::LABW), planes(K::LABW, 0);
-  for (int part = 0; part < (middle ? 2 : 1); ++part) {
-    for (u32 i = 0; i < K::T; ++i) {
-      u32 half, g, pair;
-      tc_sl_label_thread<K>(i, half, g, pair);
-      if (half > 1 || (part && half)) continue;
-      std::copy(takes.begin(), takes.end(), m.lab);
-      if (part) std::copy(planes.begin(), planes.begin() + 2 * K::H * K::TW * K::NG, m.lab);
-      if (part) tc_sl_labels_middle<K>(m, i);
-      else tc_sl_labels_halves<K>(m, i);
-      const u32 v0 = part ? 2 * K::H : half * K::H, v1 = part ? K::V : (half + 1) * K::H;
-      for (u32 v = v0; v < v1; ++v)
-        for (u32 w = 0; w < K::PP; ++w) {
-          const u32 at = (v * K::NG + g) * K::TW + K::PP * pair + w;
-          planes[at] = m.lab[at];
-        }
-    }
-  }
-  std::copy(planes.begin(), planes.begin() + (middle ? K::V : 2 * K::H) * K::TW * K::NG, m.lab);
 }
 
 template <class K>
@@ -82,7 +53,7 @@ int run_sliced(const char *edge_file, int blocks) {
   std::vector<int32_t> otri(6 * D * D);
   if (orc_triangles_from_edges(D, ne, e.data(), otri.data(), D * D) != D * D) return 2;
   const u32 *tab = t.host_stables.data();
-  const u32 nch = t.slay.chunks, words = tc_sl_words<K>(nch, t.slay.far);
+  const u32 nch = t.slay.chunks, words = tc_sl_words<K>(nch);
   std::vector<TcQuad> area(words / 4 + 2, TcQuad{0xA5A5A5A5u, 0xA5A5A5A5u, 0xA5A5A5A5u, 0xA5A5A5A5u});
   u32 *const base = reinterpret_cast<u32 *>(area.data());
   for (u32 i = words; i < 4 * area.size(); ++i) base[i] = 0xC3C3C3C3u;  // behind the areas: not to be written
@@ -104,7 +75,7 @@ int run_sliced(const char *edge_file, int blocks) {
         for (u32 i = 0; i < 32; ++i) x |= sig[32 * g + i].bit(k) << i;
         m.x[k * K::NG + g] = x;
       }
-    emulate_labels<K>(m, true);
+    for (u32 i = 0; i < K::T; ++i) tc_sl_logic<K>(m, i);
     for (u32 i = 0; i < K::T; ++i) tc_sl_tiles<K>(m, i);
     emulate_events<K>(m, nch);
     std::vector<u64> code((size_t)K::T * K::CW, 0);
@@ -113,6 +84,7 @@ int run_sliced(const char *edge_file, int blocks) {
     for (u32 i = 0; i < K::T; ++i) {
       const TcSlInst<K> I(m, i);
       bool st = false;
+      tc_sl_labels<K>(I, K::V);
       R[i] = tc_sl_regions<K>(m, I, root[i], st, err[i]);
       star[i] = st;
     }
