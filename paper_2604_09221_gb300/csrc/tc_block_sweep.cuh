@@ -346,7 +346,7 @@ __device__ __noinline__ void tc_sb_deep(const TcSbMem &m, u32 t, u32 hl, u64 low
     if (c) par[(c >> 2) * 4 * K::T + (c & 3u)] = (u8)comp(*tc_sb_byte<K>(m.rec, K::R_CPAR, c, hl));
   }
   const u32 root = *tc_sb_byte<K>(m.rec, K::R_NCOMP, rootn, hl);
-  const u64 key = tc_sl_tree_code<K::T, 4 * K::T, K::RMAX>(par, m.s.lab + t, alive, root, err);
+  const u64 key = tc_sl_tree_code<1, K::T, 4 * K::T, K::RMAX>(par, m.s.lab + t, alive, root, err);
   if (key)
     tc_sb_insert<K::HASH>(key, cnt, out.hkeys, out.hcnt, out.gkeys, out.gcnt, out.gslots, out.gerr);
   else

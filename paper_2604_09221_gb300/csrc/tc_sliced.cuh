@@ -93,6 +93,13 @@ struct TcSlK {
   static constexpr u32 OFF_WPAR = 0, OFF_WFC = WB, OFF_WNS = 2 * WB, OFF_WENT = 3 * WB,
                        OFF_WARENA = 3 * WB + (RMAX / 2 + 2 + 1) / 2,
                        OFF_WTEMP = OFF_WARENA + WARENA, WIDE_WORDS = OFF_WTEMP + WARENA;
+  // up to 57 regions (d <= 12): tree codes in two words, children sets of two
+  // words each over the label area and the event chunks (AREA words of them).
+  // Against the byte-tree back end (tc_backend_wide's code): 2^18 queries at
+  // d = 12 562 -> 437 us, 2^21 sampled vectors at d = 10 1914 -> 1546 us.
+  static constexpr bool TREE2 = WIDE && RMAX <= 58;
+  static constexpr u32 AREA = TREE2 && 2 * RMAX * T > LABW ? 2 * RMAX * T - LABW : 0;
+  static_assert(!TREE2 || CW == 2, "tree codes of two words");
   static_assert(WIDE || RMAX * T <= LABW, "the narrow tree code's children masks fit the label area");
   static_assert(!WIDE || WIDE_WORDS * T <= LABW, "the wide back end's scratch fits the label area");
   // unused members TcScratch names
@@ -110,8 +117,12 @@ struct TcSlMem {
 // Words of a block's areas behind the tables (chunks of events).  The last
 // area holds the sign planes, in the trees phase the region parents.
 template <class K>
+__host__ __device__ constexpr u32 tc_sl_evwords(u32 chunks) {
+  return chunks * K::NG * TC_SL_GROUP > K::AREA ? chunks * K::NG * TC_SL_GROUP : K::AREA;
+}
+template <class K>
 __host__ __device__ constexpr u32 tc_sl_words(u32 chunks) {
-  return K::LABW + chunks * K::NG * TC_SL_GROUP + K::XW;
+  return K::LABW + tc_sl_evwords<K>(chunks) + K::XW;
 }
 
 template <class K>
@@ -120,7 +131,7 @@ __device__ __forceinline__ TcSlMem tc_sl_carve(const u32 *tab, u32 *area, u32 ch
   m.tab = tab;
   m.lab = area;
   m.ev = m.lab + K::LABW;
-  m.x = m.ev + chunks * K::NG * TC_SL_GROUP;
+  m.x = m.ev + tc_sl_evwords<K>(chunks);
   return m;
 }
 
@@ -538,83 +549,128 @@ __device__ __forceinline__ u32 tc_sl_regions(const TcSlMem &m, const TcSlInst<K>
   return R;
 }
 
-// Canonical code of a region tree of at most 29 regions that is no star (28
-// ovals).  alive: the regions' numbers (below 32, region 0 the smallest);
-// parent of region r: byte r % 4 of par's group r / 4 (PW bytes apart), for
-// r > 0, smaller than r; adj: children masks, word r at adj[r * AW], written
-// here.  The tree is re-rooted by reversing the path from the root to region
-// 0; AHU codes follow for the regions with children, those off the path by
-// falling number (children have larger ones), then along the path.  A code is
-// left-aligned in 64 bits with its length in the low byte (at most 56 bits);
-// a leaf's code '10' is the smallest.
-template <u32 AW, u32 PW, u32 RMAX>
-__device__ __forceinline__ u64 tc_sl_tree_code(u8 *par, u32 *adj, u32 alive, u32 root, u32 &err) {
-  static_assert(2 * RMAX <= 58, "narrow tree codes");
-  auto up_of = [&](u32 r) -> u8 & { return par[(r >> 2) * PW + (r & 3u)]; };
-  const u32 first = (u32)__ffs(alive) - 1u;
-  for (u32 a = alive; a; a &= a - 1u) adj[((u32)__ffs(a) - 1u) * AW] = 0;
-  u32 internal = 0, path = 0;
-  for (u32 a = alive & (alive - 1u); a; a &= a - 1u) {
-    const u32 r = (u32)__ffs(a) - 1u, p = up_of(r);
-    adj[p * AW] |= 1u << r;
-    internal |= 1u << p;
+// Sets of regions and codes of the tree codes below: up to 32 regions with
+// codes of up to 56 bits, or up to 64 with codes of up to 112 bits.
+template <u32 WORDS>
+struct TcTreeSet;
+template <>
+struct TcTreeSet<1> {
+  typedef u32 set_t;
+  typedef u64 code_t;
+  static __device__ __forceinline__ u32 low(set_t x) { return (u32)__ffs(x) - 1u; }
+  static __device__ __forceinline__ u32 high(set_t x) { return 31u - (u32)__clz(x); }
+  static __device__ __forceinline__ u32 size(set_t x) { return (u32)__popc(x); }
+};
+template <>
+struct TcTreeSet<2> {
+  typedef u64 set_t;
+  typedef unsigned __int128 code_t;
+  static __device__ __forceinline__ u32 low(set_t x) { return (u32)__ffsll(x) - 1u; }
+  static __device__ __forceinline__ u32 high(set_t x) {
+    return x >> 32 ? 63u - (u32)__clz((u32)(x >> 32)) : 31u - (u32)__clz((u32)x);
   }
-  for (u32 x = root, prev = 32;;) {  // reverse the path root -> region 0
-    const u32 up = x == first ? 32u : (u32)up_of(x);
-    u32 kids = adj[x * AW];
-    if (prev < 32) kids &= ~(1u << prev);
-    if (x != first) kids |= 1u << up;
-    adj[x * AW] = kids;
-    internal = kids ? internal | (1u << x) : internal & ~(1u << x);
-    path |= 1u << x;
+  static __device__ __forceinline__ u32 size(set_t x) { return (u32)__popcll(x); }
+};
+
+// Canonical code of a region tree that is no star.  alive: the regions'
+// numbers (region 0 or the smallest one first); parent of region r: byte r % 4
+// of par's group r / 4 (PW bytes apart), smaller than r; adj: children sets,
+// word w of region r's at adj[(WORDS r + w) AW], written here.  The tree is
+// re-rooted by reversing the path from the root to the first region; AHU codes
+// follow for the regions with children, those off the path by falling number
+// (children have larger ones), then along the path.  A code is left-aligned
+// with its length in the low byte; a leaf's code '10' is the smallest.  The
+// halves of a region's code take the place of its children set and of one
+// child's (whose code is used by then), that child's number the place of its
+// parent: no local memory.
+// Returns (1 << bits) | bits, zero with err set on failure.
+template <u32 WORDS, u32 AW, u32 PW, u32 RMAX>
+__device__ __forceinline__ typename TcTreeSet<WORDS>::code_t tc_sl_tree_code(
+    u8 *par, u32 *adj, typename TcTreeSet<WORDS>::set_t alive, u32 root, u32 &err) {
+  typedef TcTreeSet<WORDS> TS;
+  typedef typename TS::set_t set_t;
+  typedef typename TS::code_t code_t;
+  constexpr u32 BITS = 64 * WORDS, NONE = 255;
+  static_assert(2 * RMAX <= BITS - 6 && RMAX <= 32 * WORDS, "tree codes");
+  auto up_of = [&](u32 r) -> u8 & { return par[(r >> 2) * PW + (r & 3u)]; };
+  auto kids_of = [&](u32 r) -> set_t {
+    if constexpr (WORDS == 1) return adj[r * AW];
+    else return (set_t)adj[2 * r * AW] | ((set_t)adj[(2 * r + 1) * AW] << 32);
+  };
+  auto set_kids = [&](u32 r, set_t x) {
+    adj[WORDS * r * AW] = (u32)x;
+    if constexpr (WORDS == 2) adj[(2 * r + 1) * AW] = (u32)(x >> 32);
+  };
+  const set_t one = 1;
+  const u32 first = TS::low(alive);
+  for (set_t a = alive; a; a &= a - 1u) set_kids(TS::low(a), 0);
+  set_t internal = 0, path = 0;
+  for (set_t a = alive & (alive - 1u); a; a &= a - 1u) {
+    const u32 r = TS::low(a), p = up_of(r);
+    adj[(WORDS * p + (r >> 5)) * AW] |= 1u << (r & 31u);
+    internal |= one << p;
+  }
+  for (u32 x = root, prev = NONE;;) {  // reverse the path root -> first region
+    const u32 up = x == first ? NONE : (u32)up_of(x);
+    set_t kids = kids_of(x);
+    if (prev != NONE) kids &= ~(one << prev);
+    if (x != first) kids |= one << up;
+    set_kids(x, kids);
+    internal = kids ? internal | (one << x) : internal & ~(one << x);
+    path |= one << x;
     up_of(x) = (u8)prev;
     if (x == first) break;
     prev = x;
     x = up;
   }
-  const u32 nb2 = 2u * ((u32)__popc(alive) - 1u);
-  u64 node[(RMAX + 1) / 2];  // codes of the regions with children, by rank among them
-  auto rank = [&](u32 x) -> u32 { return (u32)__popc(internal & ((1u << x) - 1u)); };
-  for (u32 off = internal & ~path, x = 0;;) {
+  const u32 nb2 = 2u * (TS::size(alive) - 1u);
+  if (nb2 == 0) return 1;  // no ovals (the pseudoline alone)
+  code_t tens = 0xAAAAAAAAAAAAAAAAull;
+  if constexpr (WORDS == 2) tens |= tens << 64;
+  set_t off = internal & ~path;
+  u32 x = 0, next = first;
+  for (;;) {
     if (off) {
-      x = 31u - (u32)__clz(off);
-      off &= ~(1u << x);
-    } else if (path) {  // from region 0 towards the root
-      x = (path >> first) & 1u ? first : (u32)up_of(x);
-      path &= ~(1u << x);
+      x = TS::high(off);
+      off &= ~(one << x);
+    } else if (path) {  // from the first region towards the root
+      x = next;
+      next = up_of(x);
+      path &= ~(one << x);
       if (!((internal >> x) & 1u)) continue;
     } else {
       break;
     }
-    const u32 kids = adj[x * AW];
-    u64 v = 0;
+    const set_t kids = kids_of(x);
+    code_t v = 0;
     u32 len = 0;
-    for (u32 big = kids & internal; big;) {  // larger codes first
+    for (set_t big = kids & internal; big;) {  // larger codes first
       u32 best = 0;
-      u64 bv = 0;
-      for (u32 y = big; y; y &= y - 1u) {
-        const u32 k = (u32)__ffs(y) - 1u;
-        const u64 cv = node[rank(k)];
+      code_t bv = 0;
+      for (set_t y = big; y; y &= y - 1u) {
+        const u32 k = TS::low(y);
+        const code_t cv = ((code_t)kids_of(k) << (BITS / 2)) | (code_t)kids_of(up_of(k));
         if (cv > bv) {
           bv = cv;
           best = k;
         }
       }
-      v |= (bv & ~255ull) >> len;
+      v |= (bv & ~(code_t)255) >> len;
       len += (u32)bv & 255u;
-      big &= ~(1u << best);
+      big &= ~(one << best);
     }
-    const u32 nl = 2u * (u32)__popc(kids & ~internal);
-    if (nl) v |= (0xAAAAAAAAAAAAAAAAull & ~(~0ull >> nl)) >> len;
+    const u32 nl = 2u * TS::size(kids & ~internal);
+    if (nl) v |= (tens & ~(~(code_t)0 >> nl)) >> len;
     len += nl;
     if (x == root) {
-      if (len != nb2) {
-        err |= TC_ERR_INTERNAL;
-        return 0;
-      }
-      return (1ull << len) | (v >> (64u - len));
+      if (len != nb2) break;
+      return ((code_t)1 << len) | (v >> (BITS - len));
     }
-    node[rank(x)] = (1ull << 63) | (v >> 1) | (u64)(len + 2u);
+    const u32 slot = TS::low(kids);
+    const code_t c = ((code_t)1 << (BITS - 1)) | (v >> 1) | (code_t)(len + 2u);
+    set_kids(x, (set_t)(c >> (BITS / 2)));
+    set_kids(slot, (set_t)c);
+    up_of(x) = (u8)slot;
   }
   err |= TC_ERR_INTERNAL;
   return 0;
@@ -626,19 +682,26 @@ __device__ __forceinline__ u64 tc_sl_tree_code(u8 *par, u32 *adj, u32 alive, u32
 template <class K>
 __device__ __forceinline__ void tc_sl_finish(const TcSlMem &m, const TcSlInst<K> &I, u32 t, u32 R, u32 root,
                                              bool star, u32 &err, u64 *code) {
-  if constexpr (K::WIDE) {
+  if constexpr (!K::WIDE) {
+    const u32 q = 2 * (R - 1);
+    code[0] = R == 0 ? 0ull
+              : star ? (1ull << q) | (0xAAAAAAAAAAAAAAAAull & ((1ull << q) - 1))
+                     : tc_sl_tree_code<1, K::T, 4 * K::T, K::RMAX>(I.par, m.lab + t,
+                                                                   R >= 32 ? ~0u : (1u << R) - 1u, root, err);
+  } else if constexpr (K::TREE2) {
+    code[0] = code[1] = 0;
+    if (R == 0) return;
+    const unsigned __int128 c = tc_sl_tree_code<2, K::T, 4 * K::T, K::RMAX>(
+        I.par, m.lab + t, R >= 64 ? ~0ull : (1ull << R) - 1ull, root, err);
+    code[0] = (u64)c;
+    code[1] = (u64)(c >> 64);
+  } else {
 #pragma unroll
     for (u32 w = 0; w < K::CW; ++w) code[w] = 0;
     if (R == 0) return;
     const TcScratch<K> S{m.lab + t};
     for (u32 r = 1; r < R; ++r) *S.byte(K::OFF_WPAR, r) = I.parent(r);
     tc_wide_tree_code(S, R, (int)root, err, code);
-  } else {
-    const u32 q = 2 * (R - 1);
-    code[0] = R == 0 ? 0ull
-              : star ? (1ull << q) | (0xAAAAAAAAAAAAAAAAull & ((1ull << q) - 1))
-                     : tc_sl_tree_code<K::T, 4 * K::T, K::RMAX>(I.par, m.lab + t, R >= 32 ? ~0u : (1u << R) - 1u,
-                                                                root, err);
   }
 }
 
