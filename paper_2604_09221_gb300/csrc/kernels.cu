@@ -1,25 +1,28 @@
 // kernels.cu -- table-driven sm_103a kernels of the T-curve real-scheme
-// engine (TS_KERNEL_TABLE): one kernel per degree (1..16), any triangulation
-// of that degree, no compilation at load time.
+// engine (TS_KERNEL_TABLE and TS_KERNEL_AUTO): one kernel per degree (1..16),
+// any triangulation of that degree, no compilation at load time.
 //
-// One thread classifies one sign vector with Algorithm 1 (Sec. 2):
-//   (a) the triangulation tables (host.cpp; format in tc_runtime.cuh) are
-//       copied global -> shared once per block with cp.async.bulk completing
-//       on an mbarrier (plain bulk copy, no multicast; bounded wait);
-//   (b) the sign of a diamond vertex is bit k(v) of sigma xor the Eq. 2
+// Blocks classify 32 sign vectors per instruction where the work is boolean
+// (Algorithm 1, Sec. 2, in the phases of tc_sliced.cuh): the tables
+// (host.cpp) are copied global -> shared once per block with cp.async.bulk
+// completing on an mbarrier (plain bulk copy, no multicast; bounded wait), and
+// everything else stays in shared memory.  Sweeps add codes to a block-private
+// shared-memory hash table that is merged into the device hash table at the
+// end (multi-word codes: straight into the device table); ranges of whole
+// blocks of middle-row patterns go to block_sweep.cu.
+//
+// TS_KERNEL_TABLE with TS_SCRATCH_GLOBAL: one thread per sign vector.
+//   (a) the sign of a diamond vertex is bit k(v) of sigma xor the Eq. 2
 //       parity constant c(v);
-//   (c) an edge is crossed iff its end points' signs differ;
-//   (d) Alg. 1 lines 3-4: tc_sweep_table gives every vertex the label of its
+//   (b) an edge is crossed iff its end points' signs differ;
+//   (c) Alg. 1 lines 3-4: tc_sweep_table gives every vertex the label of its
 //       first same-sign earlier neighbour (or a fresh label); joins between
 //       labels (several same-sign runs in a vertex's fan, antipodal pairs)
 //       are appended without branching and applied on a static schedule;
-//   (e)-(f) Alg. 1 lines 5-11: tc_backend / tc_backend_wide (regions, region
-//       tree from the regions' smallest labels, root, AHU code).  Sweeps add
-//       codes to a block-private shared-memory hash table (warp-aggregated)
-//       that is merged into the device hash table at the end (multi-word
-//       codes: straight into the device table).
-// Per-thread scratch (tc_layout.h) is interleaved by 32-bit word across the
-// block, in shared memory or, from d = 7 by default, in global memory.
+//   (d) Alg. 1 lines 5-11: tc_backend / tc_backend_wide (regions, region
+//       tree from the regions' smallest labels, root, AHU code).
+// Its per-thread scratch (tc_layout.h) is interleaved by 32-bit word across
+// the block, in global memory.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -34,12 +37,10 @@
 namespace tcurve {
 namespace {
 
-// Scratch placement: shared memory (block size from the layout: the
-// largest of which two blocks fit an SM), or global memory, L1/L2-resident,
-// with 128-thread blocks (more warps per SM for the large degrees, whose
-// per-thread scratch leaves room for one or two warps in shared memory).
-template <int D, bool G>
-using TableK = TcTableK<D, G ? 128 : 256, G>;
+// Thread-per-instance kernels: 128 threads, scratch in global memory
+// (L1/L2-resident).
+template <int D>
+using TableK = TcTableK<D, 128, true>;
 
 // With global scratch the label slots of the sweep (one load per fan
 // entry) stay in shared memory: ceil(nslots / labels per word) words per
@@ -49,11 +50,10 @@ __host__ __device__ constexpr uint32_t slot_words(uint32_t nslots) {
   return (nslots + TcScratch<K>::EPW - 1) / TcScratch<K>::EPW;
 }
 
-template <class K, bool G>
+template <class K>
 constexpr size_t smem_bytes(uint32_t table_words, uint32_t nslots, bool with_hash) {
   return ((size_t)table_words * 4 + 127) / 128 * 128 + 128 +
-         (G ? (size_t)slot_words<K>(nslots) * 4 * K::THREADS : (size_t)K::WORDS * 4 * K::THREADS) +
-         (with_hash ? (size_t)K::HASH * 16 : 0);
+         (size_t)slot_words<K>(nslots) * 4 * K::THREADS + (with_hash ? (size_t)K::HASH * 16 : 0);
 }
 
 struct SmemLayout {
@@ -61,12 +61,12 @@ struct SmemLayout {
   uint64_t *bar;
   unsigned long long *chunk;  // work-chunk broadcast slot (inside the barrier line)
   u32 *scratch;
-  u32 *slots;  // label slots in shared memory (global scratch), else null
+  u32 *slots;  // label slots
   u64 *hkeys;
   unsigned long long *hcnt;
 };
 
-template <class K, bool G>
+template <class K>
 __device__ SmemLayout carve(uint8_t *smem, uint32_t table_words, uint32_t nslots, u32 *gscratch) {
   SmemLayout s;
   size_t off = 0;
@@ -75,15 +75,9 @@ __device__ SmemLayout carve(uint8_t *smem, uint32_t table_words, uint32_t nslots
   s.bar = reinterpret_cast<uint64_t *>(smem + off);
   s.chunk = reinterpret_cast<unsigned long long *>(smem + off + 64);
   off += 128;
-  if (G) {
-    s.scratch = gscratch + (size_t)blockIdx.x * K::WORDS * K::THREADS;
-    s.slots = reinterpret_cast<u32 *>(smem + off);
-    off += (size_t)slot_words<K>(nslots) * 4 * K::THREADS;
-  } else {
-    s.scratch = reinterpret_cast<u32 *>(smem + off);
-    s.slots = nullptr;
-    off += (size_t)K::WORDS * 4 * K::THREADS;
-  }
+  s.scratch = gscratch + (size_t)blockIdx.x * K::WORDS * K::THREADS;
+  s.slots = reinterpret_cast<u32 *>(smem + off);
+  off += (size_t)slot_words<K>(nslots) * 4 * K::THREADS;
   s.hkeys = reinterpret_cast<u64 *>(smem + off);
   s.hcnt = reinterpret_cast<unsigned long long *>(smem + off + K::HASH * 8);
   return s;
@@ -106,24 +100,24 @@ __host__ __device__ constexpr uint32_t sliced_table_bytes(uint32_t words) {
 
 // ----------------------------------------------------- query kernel ----
 
-template <int D, bool G>
-__global__ void __launch_bounds__(TableK<D, G>::THREADS)
+template <int D>
+__global__ void __launch_bounds__(TableK<D>::THREADS)
     real_schemes_kernel(TableLayout L, const uint32_t *__restrict__ gtab,
                         const uint64_t *__restrict__ signs, uint64_t n, uint64_t *codes,
                         uint32_t *err_word, u32 *gscratch) {
-  typedef TableK<D, G> K;
+  typedef TableK<D> K;
   extern __shared__ __align__(128) uint8_t smem[];
-  SmemLayout M = carve<K, G>(smem, L.words, L.nslots, gscratch);
+  SmemLayout M = carve<K>(smem, L.words, L.nslots, gscratch);
   if (!stage_tables(M.tab, gtab, L.words * 4, M.bar, err_word)) return;
   const TcScratch<K> S{M.scratch + threadIdx.x};
-  u32 *const ls = G ? M.slots + threadIdx.x : nullptr;
-  if (G) fan_offsets<K>(M.tab, L);
+  u32 *const ls = M.slots + threadIdx.x;
+  fan_offsets<K>(M.tab, L);
   const u64 *sg = reinterpret_cast<const u64 *>(signs);
   uint32_t err = 0;
   for (uint64_t i = (uint64_t)blockIdx.x * K::THREADS + threadIdx.x; i < n;
        i += (uint64_t)gridDim.x * K::THREADS) {
     const TcCodeOut<K> c =
-        tc_table_classify<K, G>(tc_load_sig<K>(sg, i), M.tab, L.off_fan, L.off_vext, S, err, ls);
+        tc_table_classify<K, true>(tc_load_sig<K>(sg, i), M.tab, L.off_fan, L.off_vext, S, err, ls);
 #pragma unroll
     for (u32 w = 0; w < K::CW; ++w) codes[i * K::CW + w] = c.w[w];
   }
@@ -132,22 +126,22 @@ __global__ void __launch_bounds__(TableK<D, G>::THREADS)
 
 // ----------------------------------------------- enumeration kernel ----
 
-template <int D, bool G>
-__global__ void __launch_bounds__(TableK<D, G>::THREADS)
+template <int D>
+__global__ void __launch_bounds__(TableK<D>::THREADS)
     enumerate_kernel(TableLayout L, const uint32_t *__restrict__ gtab, uint64_t lo, uint64_t total,
                      uint32_t flags, ts_hist h, u32 *gscratch) {
-  typedef TableK<D, G> K;
+  typedef TableK<D> K;
   constexpr uint32_t kChunk = K::THREADS * 16;
   extern __shared__ __align__(128) uint8_t smem[];
-  SmemLayout M = carve<K, G>(smem, L.words, L.nslots, gscratch);
+  SmemLayout M = carve<K>(smem, L.words, L.nslots, gscratch);
   for (int s = threadIdx.x; s < (int)K::HASH; s += K::THREADS) {
     M.hkeys[s] = 0;
     M.hcnt[s] = 0;
   }
   if (!stage_tables(M.tab, gtab, L.words * 4, M.bar, h.d_err)) return;
   const TcScratch<K> S{M.scratch + threadIdx.x};
-  u32 *const ls = G ? M.slots + threadIdx.x : nullptr;
-  if (G) fan_offsets<K>(M.tab, L);
+  u32 *const ls = M.slots + threadIdx.x;
+  fan_offsets<K>(M.tab, L);
   uint32_t err = 0;
   unsigned long long failed = 0;
   for (;;) {
@@ -160,7 +154,7 @@ __global__ void __launch_bounds__(TableK<D, G>::THREADS)
       const uint64_t idx = base + j + threadIdx.x;
       TcCodeOut<K> key{};
       if (idx < total) {
-        key = tc_table_classify<K, G>(tc_enum_sig<K::W>(lo + idx, flags, D), M.tab, L.off_fan,
+        key = tc_table_classify<K, true>(tc_enum_sig<K::W>(lo + idx, flags, D), M.tab, L.off_fan,
                                       L.off_vext, S, err, ls);
         u64 any = 0;
 #pragma unroll
@@ -403,56 +397,59 @@ cudaError_t enumerate_sliced(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t
   return cudaGetLastError();
 }
 
-template <int D, bool G>
+template <int D>
 cudaError_t real_schemes_dg(const ts_tri *t, const uint64_t *signs, uint64_t n, uint64_t *codes,
                             cudaStream_t st) {
-  typedef TableK<D, G> K;
-  const size_t smem = smem_bytes<K, G>(t->lay.words, t->lay.nslots, false);
+  typedef TableK<D> K;
+  const size_t smem = smem_bytes<K>(t->lay.words, t->lay.nslots, false);
   unsigned grid = 0;
-  cudaError_t e = persistent_grid(real_schemes_kernel<D, G>, K::THREADS, smem,
+  cudaError_t e = persistent_grid(real_schemes_kernel<D>, K::THREADS, smem,
                                   (n + K::THREADS - 1) / K::THREADS, &grid);
   if (e != cudaSuccess) return e;
   GlobalScratch gs(st);
-  if (G && (e = gs.alloc((size_t)grid * K::WORDS * K::THREADS * 4)) != cudaSuccess) return e;
-  real_schemes_kernel<D, G><<<grid, K::THREADS, smem, st>>>(t->lay, t->d_tables, signs, n, codes,
+  if ((e = gs.alloc((size_t)grid * K::WORDS * K::THREADS * 4)) != cudaSuccess) return e;
+  real_schemes_kernel<D><<<grid, K::THREADS, smem, st>>>(t->lay, t->d_tables, signs, n, codes,
                                                             t->d_err, gs.p);
   return cudaGetLastError();
 }
 
-template <int D, bool G>
+template <int D>
 cudaError_t enumerate_dg(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *h,
                          cudaStream_t st) {
-  typedef TableK<D, G> K;
-  const size_t smem = smem_bytes<K, G>(t->lay.words, t->lay.nslots, true);
+  typedef TableK<D> K;
+  const size_t smem = smem_bytes<K>(t->lay.words, t->lay.nslots, true);
   const uint64_t total = hi - lo;
   const uint64_t chunk = (uint64_t)K::THREADS * 16;
   unsigned grid = 0;
-  cudaError_t e = persistent_grid(enumerate_kernel<D, G>, K::THREADS, smem, (total + chunk - 1) / chunk,
+  cudaError_t e = persistent_grid(enumerate_kernel<D>, K::THREADS, smem, (total + chunk - 1) / chunk,
                                   &grid);
   if (e != cudaSuccess) return e;
   GlobalScratch gs(st);
-  if (G && (e = gs.alloc((size_t)grid * K::WORDS * K::THREADS * 4)) != cudaSuccess) return e;
+  if ((e = gs.alloc((size_t)grid * K::WORDS * K::THREADS * 4)) != cudaSuccess) return e;
   e = cudaMemsetAsync(h->d_work, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  enumerate_kernel<D, G><<<grid, K::THREADS, smem, st>>>(t->lay, t->d_tables, lo, total, flags, *h,
+  enumerate_kernel<D><<<grid, K::THREADS, smem, st>>>(t->lay, t->d_tables, lo, total, flags, *h,
                                                          gs.p);
   return cudaGetLastError();
 }
 
-// One thread per sign vector, scratch in global memory, only when asked for.
-bool global_scratch(const ts_tri *t) { return t->scratch == TS_SCRATCH_GLOBAL; }
+// One thread per sign vector, scratch in global memory: only when both are
+// asked for (d = 7: 0.6e9/s against the bit-sliced kernel's 4.5e9).
+bool global_scratch(const ts_tri *t) {
+  return t->kernel == TS_KERNEL_TABLE && t->scratch == TS_SCRATCH_GLOBAL;
+}
 
 template <int D>
 cudaError_t real_schemes_d(const ts_tri *t, const uint64_t *signs, uint64_t n, uint64_t *codes,
                            cudaStream_t st) {
-  return global_scratch(t) ? real_schemes_dg<D, true>(t, signs, n, codes, st)
+  return global_scratch(t) ? real_schemes_dg<D>(t, signs, n, codes, st)
                            : real_schemes_sliced<D>(t, signs, n, codes, st);
 }
 
 template <int D>
 cudaError_t enumerate_d(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *h,
                         cudaStream_t st, bool allow_global) {
-  if (allow_global && global_scratch(t)) return enumerate_dg<D, true>(t, lo, hi, flags, h, st);
+  if (allow_global && global_scratch(t)) return enumerate_dg<D>(t, lo, hi, flags, h, st);
   // whole blocks of middle-row patterns by the block sweep, the ragged ends
   // (or everything, if there are few blocks) mask by mask
   uint64_t a = hi, b = hi;
