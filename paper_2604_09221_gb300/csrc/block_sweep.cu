@@ -2,9 +2,10 @@
 // (tc_block_sweep.cuh): the kernel, and the split of a range into whole
 // blocks, for 4 <= d <= 9.
 //
-// A persistent block takes 128 high parts at a time.  What bounds it is
-// integer issue: at d = 7 the middle phase is about 75 instructions per mask
-// and the halves about 25 per mask (6 000 per high part over 256 masks).
+// A persistent block takes 128 high parts at a time, or for short ranges one
+// of 2^lparts equal parts of their patterns.  What bounds it is integer issue:
+// at d = 7 the halves and their records take about as long as two words (64
+// patterns) of the middle phase.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -19,12 +20,14 @@ namespace {
 
 // Masks (h << oshift) | (t << ishift) for h = hi0 .. hi0 + n_hi - 1 (with
 // TS_ENUM_ORBITS in flags, h = the block's high part, tc_orbit_high) and
-// t < 2^ib.  smem: tables (toff bytes) | mbarrier, work slot (128 bytes) |
+// t < 2^ib, in work items of 128 high parts and 2^(ib - lparts) patterns.
+// smem: tables (toff bytes) | mbarrier, work slot (128 bytes) |
 // the areas | hash table.
 template <int D>
 __global__ void __launch_bounds__(128, D <= 7 ? 3 : 2)
     block_sweep_kernel(SlicedLayout L, const uint32_t *__restrict__ gtab, uint64_t hi0, uint64_t n_hi,
-                       uint32_t oshift, uint32_t ishift, uint32_t ib, uint32_t flags, ts_hist h) {
+                       uint32_t oshift, uint32_t ishift, uint32_t ib, uint32_t lparts, uint32_t flags,
+                       ts_hist h) {
   typedef TcSbK<D> K;
   typedef typename K::Base B;
   extern __shared__ __align__(128) uint8_t smem[];
@@ -36,14 +39,14 @@ __global__ void __launch_bounds__(128, D <= 7 ? 3 : 2)
   u64 *const hkeys = reinterpret_cast<u64 *>(area + tc_sb_words<K>(L.chunks));
   u32 *const hcnt = reinterpret_cast<u32 *>(hkeys + K::HASH);
   const TcSbOut out{hkeys, hcnt, reinterpret_cast<u64 *>(h.d_keys), h.d_counts, h.slots, h.d_err};
-  const u32 t = threadIdx.x, mine = tc_sl_instance<B>(t), lw = ib - 5u;
+  const u32 t = threadIdx.x, mine = tc_sl_instance<B>(t), lw = ib - 5u - lparts;
   for (u32 s = t; s < K::HASH; s += K::T) {
     hkeys[s] = 0;
     hcnt[s] = 0;
   }
   for (u32 s = t; s < K::STARS; s += K::T) M.stars[s] = 0;
   if (t == 0) *M.queued = 0;
-  if (t == 0) *slot = atomicAdd(h.d_work, (unsigned long long)K::T);
+  if (t == 0) *slot = atomicAdd(h.d_work, 1ull);
   if (!stage_tables(tab, gtab, L.words * 4, reinterpret_cast<uint64_t *>(smem + toff), h.d_err)) return;
   uint32_t err = 0, items = 0;
   unsigned long long failed = 0;
@@ -65,11 +68,12 @@ __global__ void __launch_bounds__(128, D <= 7 ? 3 : 2)
     return ((flags & TS_ENUM_ORBITS) ? tc_orbit_high(u, flags) : u) << oshift;
   };
   for (;;) {
-    const uint64_t base = *slot;
+    const uint64_t item = *slot, base = (item >> lparts) * K::T;
+    const u32 part = (u32)item & ((1u << lparts) - 1u);
     if (base >= n_hi) break;
     __syncthreads();
     // the next work item is fetched while this one runs
-    if (t == 0) *slot = atomicAdd(h.d_work, (unsigned long long)K::T);
+    if (t == 0) *slot = atomicAdd(h.d_work, 1ull);
     tc_sl_clear<B>(M.s, t);
     tc_sl_planes<B>(M.s, TcSig<1>{{base + t < n_hi ? mask_of(base + t) : 0ull}}, t);
     __syncthreads();
@@ -84,7 +88,7 @@ __global__ void __launch_bounds__(128, D <= 7 ? 3 : 2)
     if (!live) M.rec[K::R_HDR * K::T + t] = 1u << 31;  // behind the range
     __syncthreads();
     for (u32 task = t; task < K::T << lw; task += K::T) {
-      const u32 hl = task >> lw, w = task & ((1u << lw) - 1u), hdr = M.rec[K::R_HDR * K::T + hl];
+      const u32 hl = task >> lw, w = part << lw | (task & ((1u << lw) - 1u)), hdr = M.rec[K::R_HDR * K::T + hl];
       const bool valid = (hdr >> 25) & 1u;
       // the larger size when a lane of the warp needs it
       if (__any_sync(0xffffffffu, valid && ((hdr >> 8) & 255u) > K::NA)) {
@@ -98,11 +102,12 @@ __global__ void __launch_bounds__(128, D <= 7 ? 3 : 2)
       const u32 hdr = M.rec[K::R_HDR * K::T + hl];
       if ((hdr >> 25) & 1u || hdr >> 31) continue;
       const u64 hm = mask_of(base + tc_sl_instance<B>(hl));
-      for (u32 p = 0; p < 1u << ib; p += K::T) {
+      const u32 pend = (part + 1u) << (lw + 5u);
+      for (u32 p = part << (lw + 5u); p < pend; p += K::T) {
         u32 e = 0;
         u64 code = 0;
-        tc_sl_classify<B>(M.s, TcSig<1>{{hm | ((u64)(p + t) << ishift)}}, t, e, &code);
-        const bool in = p + mine < 1u << ib;
+        tc_sl_classify<B>(M.s, TcSig<1>{{hm | ((u64)(p + t < pend ? p + t : p) << ishift)}}, t, e, &code);
+        const bool in = p + mine < pend;
         code = in ? code : 0ull;
         err |= in ? e : 0u;
         failed += in && code == 0;
@@ -141,9 +146,24 @@ cudaError_t launch_d(const ts_tri *t, uint64_t h0, uint64_t n, const Split &s, u
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   e = cudaMemsetAsync(h->d_work, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)std::min<uint64_t>((n + 127) / 128, (uint64_t)per_sm * sms);
-  block_sweep_kernel<D><<<grid, 128, smem, st>>>(t->slay, t->d_stables, h0, n, s.oshift, s.ishift, s.ib, flags,
-                                                 *h);
+  // Parts: the fewest that make the waves times a part's time smallest, in
+  // words of the middle phase, the halves counted as two (0.28, 0.45, 0.57 of
+  // 6.6, 4.4, 2.5 ms at d = 9, 8, 7).  2^19 masks in one
+  // part took 736, 306, 114 us (few of the blocks the device holds at work),
+  // in parts 100, 80, 64; a flip sweep of 2^26 at d = 9 4.55 -> 3.25 ms.
+  const uint64_t groups = (n + 127) / 128, held = (uint64_t)per_sm * sms;
+  uint32_t lparts = 0;
+  uint64_t best = ~0ull;
+  for (uint32_t l = 0; l <= s.ib - 5; ++l) {
+    const uint64_t time = (((groups << l) + held - 1) / held) * (2 + (1ull << (s.ib - 5 - l)));
+    if (time < best) {
+      best = time;
+      lparts = l;
+    }
+  }
+  const unsigned grid = (unsigned)std::min<uint64_t>(groups << lparts, held);
+  block_sweep_kernel<D><<<grid, 128, smem, st>>>(t->slay, t->d_stables, h0, n, s.oshift, s.ishift, s.ib, lparts,
+                                                 flags, *h);
   return cudaGetLastError();
 }
 
