@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <memory>
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <utility>
@@ -111,6 +112,9 @@ struct ts_tri {
   tcurve::Diamond dia;
   int kernel = 0;                // TS_KERNEL_*
   int scratch = 0;               // TS_SCRATCH_* (both kernel families)
+  // blocks the device holds of the bit-sliced query and sweep kernels (0: not
+  // asked yet); they depend on the degree and the tables alone
+  mutable std::atomic<uint32_t> resident[2] = {};
   int occupancy = 0;             // target blocks per SM of the specialised kernels (0: default)
   std::mutex jit_mu;
   std::shared_ptr<tcurve::JitModule> jit;

@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "engine.h"
@@ -358,6 +359,25 @@ cudaError_t persistent_grid(F fn, int threads, size_t smem, uint64_t want, unsig
   return cudaSuccess;
 }
 
+// The same for kernel `which` of tri (ts_tri::resident), whose resident blocks
+// are asked for once: 2^15 queries at d = 4, one call after
+// another, 15.0 -> 13.5 us a call.
+template <class F>
+cudaError_t persistent_grid(const ts_tri *t, int which, F fn, int threads, size_t smem, uint64_t want,
+                            unsigned *grid) {
+  int dev = -1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev != t->device) return persistent_grid(fn, threads, smem, want, grid);
+  unsigned cap = t->resident[which].load(std::memory_order_acquire);
+  if (!cap) {
+    if ((e = persistent_grid(fn, threads, smem, ~0ull, &cap)) != cudaSuccess) return e;
+    t->resident[which].store(cap, std::memory_order_release);
+  }
+  *grid = (unsigned)std::min<uint64_t>(want ? want : 1, cap);
+  return cudaSuccess;
+}
+
 // Global scratch of a launch: stream-ordered allocation, freed after it.
 struct GlobalScratch {
   u32 *p = nullptr;
@@ -375,7 +395,7 @@ cudaError_t real_schemes_sliced(const ts_tri *t, const uint64_t *signs, uint64_t
   typedef SlicedK<D> K;
   const size_t smem = sliced_table_bytes(t->slay.words) + 128 + (size_t)tc_sl_words<K>(t->slay.chunks) * 4;
   unsigned grid = 0;
-  cudaError_t e = persistent_grid(sliced_real_schemes_kernel<K>, K::T, smem, (n + K::T - 1) / K::T, &grid);
+  cudaError_t e = persistent_grid(t, 0, sliced_real_schemes_kernel<K>, K::T, smem, (n + K::T - 1) / K::T, &grid);
   if (e != cudaSuccess) return e;
   sliced_real_schemes_kernel<K><<<grid, K::T, smem, st>>>(t->slay, t->d_stables, signs, n, codes, t->d_err);
   return cudaGetLastError();
@@ -389,7 +409,7 @@ cudaError_t enumerate_sliced(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t
                       (size_t)K::HASH * 16;
   const uint64_t total = hi - lo;
   unsigned grid = 0;
-  cudaError_t e = persistent_grid(sliced_enumerate_kernel<K>, K::T, smem, (total + K::T - 1) / K::T, &grid);
+  cudaError_t e = persistent_grid(t, 1, sliced_enumerate_kernel<K>, K::T, smem, (total + K::T - 1) / K::T, &grid);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(h->d_work, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
