@@ -25,6 +25,7 @@
 #include <cstring>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -230,6 +231,42 @@ ts_status cuda_st(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? TS_ENOMEM : TS_ECUDA;
 }
 
+// Packed histogram of one job: entries found, failed instances, error word, 0;
+// then per entry its code words and its count.
+constexpr uint64_t kPackHeader = 4;
+constexpr uint64_t kPackMax = 1 << 14;   // entries there is room for
+constexpr uint64_t kPackFirst = 1 << 10;  // entries read along with the header
+
+// The occupied slots (a nonzero key word) of a job's table, in any order, at
+// most cap of them stored: one atomic per warp, lanes ranked by a ballot.
+// Bound by the table's bytes (512 KB of 2^15 slots: 3 us).
+__global__ void batch_pack_kernel(const uint64_t *__restrict__ keys, const unsigned long long *__restrict__ counts,
+                                  uint64_t slots, int cw, uint64_t cap, const uint32_t *err,
+                                  const unsigned long long *failed, unsigned long long *out) {
+  const uint32_t lane = threadIdx.x & 31u;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    out[1] = *failed;
+    out[2] = *err;
+  }
+  for (uint64_t base = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ull; base < slots;
+       base += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t s = base + lane;
+    bool nz = false;
+    if (s < slots)
+      for (int w = 0; w < cw; ++w) nz |= keys[s * cw + w] != 0;
+    const unsigned ball = __ballot_sync(0xffffffffu, nz);
+    unsigned long long first = 0;
+    if (lane == 0 && ball) first = atomicAdd(out, (unsigned long long)__popc(ball));
+    first = __shfl_sync(0xffffffffu, first, 0);
+    const uint64_t o = first + __popc(ball & ((1u << lane) - 1u));
+    if (nz && o < cap) {
+      unsigned long long *e = out + kPackHeader + o * (cw + 1);
+      for (int w = 0; w < cw; ++w) e[w] = keys[s * cw + w];
+      e[cw] = counts[s] & kCountMask;
+    }
+  }
+}
+
 }  // namespace
 }  // namespace tcurve
 
@@ -271,6 +308,9 @@ struct ts_batch {
   unsigned long long *d_counts = nullptr;
   uint32_t *d_err = nullptr;
   unsigned long long *d_failed = nullptr;
+  std::mutex read_mu;               // of the packed entries (ts_batch_read)
+  unsigned long long *d_pack = nullptr;  // kPackHeader words, then pack_cap entries
+  uint64_t pack_cap = 0;
   cudaEvent_t fork = nullptr;
   cudaGraphExec_t exec = nullptr;
   int device = 0;
@@ -603,6 +643,13 @@ ts_status ts_batch_create(int njobs, ts_tri *const *tris, const uint64_t *counts
   if (e == cudaSuccess) e = cudaMalloc(&b->d_counts, b->count_words * 8);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_err, 4);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_failed, 8);
+  uint64_t pack_words = 0;
+  for (int j = 0; j < njobs; ++j) {
+    b->pack_cap = std::max(b->pack_cap, std::min(b->jslots[j], kPackMax));
+    pack_words = std::max<uint64_t>(pack_words, b->cws[j] + 1);
+  }
+  pack_words = pack_words * b->pack_cap + kPackHeader;
+  if (e == cudaSuccess) e = cudaMalloc(&b->d_pack, pack_words * 8);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
   std::map<int, int> gi;
   for (int j = 0; j < njobs && e == cudaSuccess; ++j) {
@@ -686,6 +733,7 @@ void ts_batch_free(ts_batch *b) {
   if (b->d_counts) cudaFree(b->d_counts);
   if (b->d_err) cudaFree(b->d_err);
   if (b->d_failed) cudaFree(b->d_failed);
+  if (b->d_pack) cudaFree(b->d_pack);
   delete b;
 }
 
@@ -899,37 +947,70 @@ ts_status ts_batch_read(ts_batch *b, int job, uint64_t *codes, uint64_t *counts,
                         uint64_t *n_out, uint64_t *n_failed, void *stream) {
   if (!b || !n_out || job < 0 || job >= (int)b->jobs.size() || (cap && (!codes || !counts)))
     return TS_EINVAL;
-  cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
+  // The occupied slots are packed on the device and cross with the header in
+  // one copy (the first kPackFirst of them; the rest in a second one).  A
+  // table is at most half full and usually nearly empty: a batch of 5.1e6 sign
+  // vectors with 12 reads of 2^15 slots took 3.77 ms with whole tables copied,
+  // 2.96 ms now.  More schemes than kPackMax: the whole table.
   const int cw = b->cws[job];
   const uint64_t hs = b->jslots[job];
-  std::vector<uint64_t> k(hs * cw);
-  std::vector<unsigned long long> c(hs);
-  uint32_t err = 0;
-  unsigned long long failed = 0;
-  if (e == cudaSuccess)
-    e = cudaMemcpy(k.data(), b->d_keys + b->kofs[job], k.size() * 8, cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess)
-    e = cudaMemcpy(c.data(), b->d_counts + b->cofs[job], hs * 8,
-                   cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) e = cudaMemcpy(&err, b->d_err, 4, cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) e = cudaMemcpy(&failed, b->d_failed, 8, cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_st(e);
-  std::vector<uint64_t> idx;
-  for (uint64_t s = 0; s < hs; ++s) {
-    bool nz = false;
-    for (int w = 0; w < cw; ++w) nz |= k[s * cw + w] != 0;
-    if (nz) idx.push_back(s);
+  const uint64_t ew = cw + 1;
+  std::vector<unsigned long long> buf;
+  std::lock_guard<std::mutex> lock(b->read_mu);
+  cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
+  int device = b->device;  // the caller's: the pack kernel runs on the batch's
+  if (e == cudaSuccess) e = cudaGetDevice(&device);
+  if (e == cudaSuccess && device != b->device) e = cudaSetDevice(b->device);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_pack, 0, 8, cudaStreamLegacy);
+  if (e == cudaSuccess) {
+    const uint64_t blocks = std::min<uint64_t>((hs + 255) / 256, 1024);
+    batch_pack_kernel<<<(unsigned)blocks, 256, 0, cudaStreamLegacy>>>(
+        b->d_keys + b->kofs[job], b->d_counts + b->cofs[job], hs, cw, b->pack_cap, b->d_err, b->d_failed,
+        b->d_pack);
+    e = cudaGetLastError();
   }
+  if (device != b->device) cudaSetDevice(device);
+  const uint64_t first = std::min(b->pack_cap, kPackFirst);
+  buf.resize(kPackHeader + first * ew);
+  if (e == cudaSuccess) e = cudaMemcpy(buf.data(), b->d_pack, buf.size() * 8, cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return cuda_st(e);
+  const uint64_t n = buf[0];
+  const unsigned long long failed = buf[1];
+  const uint32_t err = (uint32_t)buf[2];
+  std::vector<unsigned long long> ent;  // n entries
+  if (n <= b->pack_cap) {
+    ent.assign(buf.begin() + kPackHeader, buf.begin() + kPackHeader + std::min(n, first) * ew);
+    ent.resize(n * ew);
+    if (n > first)
+      e = cudaMemcpy(ent.data() + first * ew, b->d_pack + kPackHeader + first * ew, (n - first) * ew * 8,
+                     cudaMemcpyDeviceToHost);
+  } else {
+    std::vector<uint64_t> k(hs * cw);
+    std::vector<unsigned long long> c(hs);
+    e = cudaMemcpy(k.data(), b->d_keys + b->kofs[job], k.size() * 8, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess)
+      e = cudaMemcpy(c.data(), b->d_counts + b->cofs[job], hs * 8, cudaMemcpyDeviceToHost);
+    for (uint64_t s = 0; s < hs; ++s) {
+      bool nz = false;
+      for (int w = 0; w < cw; ++w) nz |= k[s * cw + w] != 0;
+      if (!nz) continue;
+      ent.insert(ent.end(), k.begin() + s * cw, k.begin() + (s + 1) * cw);
+      ent.push_back(c[s] & kCountMask);
+    }
+  }
+  if (e != cudaSuccess) return cuda_st(e);
+  std::vector<uint64_t> idx(ent.size() / ew);
+  for (uint64_t i = 0; i < idx.size(); ++i) idx[i] = i;
   std::sort(idx.begin(), idx.end(), [&](uint64_t a, uint64_t x) {
     for (int w = cw - 1; w >= 0; --w)
-      if (k[a * cw + w] != k[x * cw + w]) return k[a * cw + w] < k[x * cw + w];
+      if (ent[a * ew + w] != ent[x * ew + w]) return ent[a * ew + w] < ent[x * ew + w];
     return false;
   });
   *n_out = idx.size();
   if (n_failed) *n_failed = failed;
   for (uint64_t i = 0; i < idx.size() && i < cap; ++i) {
-    for (int w = 0; w < cw; ++w) codes[i * cw + w] = k[idx[i] * cw + w];
-    counts[i] = c[idx[i]] & kCountMask;
+    for (int w = 0; w < cw; ++w) codes[i * cw + w] = ent[idx[i] * ew + w];
+    counts[i] = ent[idx[i] * ew + cw];
   }
   if (idx.size() > cap) return TS_EOVERFLOW;
   if (err & kErrTimeout) return TS_ETIMEOUT;
