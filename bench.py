@@ -247,7 +247,6 @@ def main():
         hist.clear(stream)
         eng.enumerate_schemes(tri, lo, lo + SLICE, hist, stream=stream)
 
-    tri.prepare()  # build the specialised kernels before anything is timed
     int_peak = measure_int_peak(eng, args.trips)
 
     for _ in range(max(args.warmup, 0)):
@@ -320,13 +319,15 @@ def main():
     peak_tops = int_peak["peak"] / 1e12
     kms = sum(ktimes) / len(ktimes)
     achieved_tops = ALG_OPS_PER_INSTANCE * SLICE / (kms / 1e3) / 1e12
-    roofline = {"bound": "alu", "kernel": "tc_enumerate_blocks (specialised to the triangulation)",
+    roofline = {"bound": "alu", "kernel": "block_sweep_kernel (bit-sliced: 32 masks per instruction)",
                 "kernel_ms": kms,
                 "achieved": achieved_tops, "peak": peak_tops, "unit": "Tops/s",
                 "frac": achieved_tops / peak_tops, "traffic": None,
-                "traffic_note": "no input is read; DRAM carries only scratch write-backs from L2 "
-                                "(55.6 MB per 2^26-mask launch by ncu), which do not scale with the "
-                                "masks swept, so no per-launch figure is given for 2^32",
+                "traffic_note": "no input is read and all scratch is in shared memory; DRAM carries "
+                                "the tables and the histogram only",
+                "frac_note": "achieved counts the method's operations for one sign vector at a time; "
+                             "the kernel does a boolean operation of 32 of them in one instruction and "
+                             "shares the half-diamonds of a block, so frac may exceed 1",
                 "peak_source": "measured: ts_int_issue_peak, the best of its instruction kinds "
                                f"({int_peak['best']}) on this GPU in this run",
                 "int_peak_tops": {k: v / 1e12 for k, v in int_peak["kinds"].items()},
@@ -506,7 +507,7 @@ def profile_case(args):
     tri.set_scratch({"auto": eng.TS_SCRATCH_AUTO, "shared": eng.TS_SCRATCH_SHARED,
                      "global": eng.TS_SCRATCH_GLOBAL}[args.scratch])
     tri.set_occupancy(args.occupancy)
-    if args.kernel in ("auto", "specialized") and d <= 9:
+    if args.kernel == "specialized" and d <= 9:
         tri.prepare()
     n = 1 << args.log2n
     if args.batch:  # a one-degree batch of 8 triangulations, n sign vectors in all
@@ -603,7 +604,7 @@ def plain_kernel(eng, tri, ti, stream):
     hbm_peak = measured_peaks().get("hbm_gbs")
     gbs = nbytes / (ms / 1e3) / 1e9
     return {"value": n / (ms / 1e3), "unit": "schemes/s",
-            "kernel": "tc_real_schemes (specialised, one launch over materialised masks)",
+            "kernel": "sliced_real_schemes_kernel (bit-sliced, one launch over materialised masks)",
             "n": n, "ms": ms, "hbm_bytes": nbytes, "hbm_gbs": gbs,
             "hbm_frac": gbs / hbm_peak if hbm_peak else None,
             "hbm_peak_gbs": hbm_peak}
@@ -688,7 +689,7 @@ def serving_run(seconds, degrees=tuple(range(6, 17)), per_degree=4, slots=8, see
             "mean_queue_ms": 1e3 * sum(r.queued for r in res) / len(res),
             "schemes_per_s": inst / wall, "slots": slots, "degrees": list(degrees),
             "sign_vectors_per_job": "sample 2^U(8,22), query 2^U(8,18), enum 2^U(8,22)",
-            "kernel": "table-driven (resident, uncompiled; global scratch from d = 7)",
+            "kernel": "table-driven, bit-sliced (resident, uncompiled)",
             "resident_mb": srv.resident / 2 ** 20, "requeued": len(srv.requeued),
             "peak_running": srv.peak_running, "seconds": wall}
 
@@ -723,7 +724,7 @@ def alg_ops(d: int) -> float:
 def mixed_run(steps, warmup, degrees=(5, 6, 7, 8, 9, 10), per_degree=32, seed=31):
     """The mixed-degree batch: 32 seeded triangulations per d in 5..10,
     2^U(10,24) splitmix64 sign vectors each, one CUDA-graph launch per step
-    (one fused persistent kernel for all degrees, or one per degree: the
+    (a fused persistent kernel per tier of degrees, or one per degree: the
     faster plan), tiles from the autotuner; every job's histogram is checked
     to count all its sign vectors."""
     import numpy as np
@@ -760,7 +761,7 @@ def mixed_run(steps, warmup, degrees=(5, 6, 7, 8, 9, 10), per_degree=32, seed=31
         return out
     # three launch plans, each measured on two runs; the fastest is the one
     # timed: the degree groups concurrently (forked streams), one after the
-    # other, or every job of every degree in one fused persistent launch
+    # other, or every job of every degree in the fused plan
     # (fused tiles from the autotuner)
     ftiles = autotune.autotune_fused(tris, counts, bases, reps=1)
     autotune.apply_fused(batch, ftiles)
@@ -782,6 +783,9 @@ def mixed_run(steps, warmup, degrees=(5, 6, 7, 8, 9, 10), per_degree=32, seed=31
     total = sum(counts)
     ops = sum(n * alg_ops(t.d) for t, n in zip(tris, counts))
     fam = {d: batch.info(d) for d in degrees}
+    # the fused plan's tiers: degrees up to 6, 8, 10, 16, and the warp tiles
+    fused_launches = len({("warp",) if ftiles.get(d, (1, 0))[0] == 3 else
+                          min(b for b in (6, 8, 10, 16) if d <= b) for d in degrees})
     return {"value": total / (ms / 1e3), "unit": "schemes/s", "ms": ms, "steps": steps,
             "workload": "mixed_degree_batch", "degrees": list(degrees),
             "triangulations_per_degree": per_degree, "jobs": len(tris), "sign_vectors": total,
@@ -791,11 +795,12 @@ def mixed_run(steps, warmup, degrees=(5, 6, 7, 8, 9, 10), per_degree=32, seed=31
             "build_s": build_s, "alg_tops": ops / (ms / 1e3) / 1e12,
             "launch": {"concurrent": "one persistent kernel per degree, concurrent streams",
                        "serial": "one persistent kernel per degree, one after the other",
-                       "fused": "one fused persistent kernel for all degrees"}[plan],
+                       "fused": "one persistent kernel per tier of degrees (up to 6, 8, 10, 16; "
+                                "warp tiles), concurrent streams"}[plan],
             "plan_ms": order,
             "fused_tiles": {str(d): [{1: "thread", 3: "warp"}.get(k, k), c]
                             for d, (k, c) in sorted(ftiles.items())},
-            "gpu_launches_per_step": 1 if plan == "fused" else len(degrees)}
+            "gpu_launches_per_step": fused_launches if plan == "fused" else len(degrees)}
 
 
 def mixed_families(reps=3, degrees=(5, 6, 7, 8, 9, 10), per_degree=32, seed=31, occupancies=(0,)):

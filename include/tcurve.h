@@ -120,7 +120,9 @@ ts_status ts_real_schemes(const ts_tri *tri, const uint64_t *signs, uint64_t n,
  *   TS_KERNEL_TABLE: one generic kernel per degree; the triangulation's
  *     tables are staged into shared memory by a bulk copy in every block.
  *     Blocks classify 64 or 128 sign vectors together, bit-sliced (with
- *     TS_SCRATCH_GLOBAL: one thread per sign vector).
+ *     TS_SCRATCH_GLOBAL: one thread per sign vector).  Sweeps of at least 2^19
+ *     masks that differ in the middle row block by block (4 <= d <= 9, not
+ *     TS_ENUM_SPLITMIX) share the half-diamonds of each block.
  *   TS_KERNEL_SPECIALIZED: a kernel generated for this triangulation (its
  *     structure compiled into the instruction stream) with NVRTC on first use;
  *     d <= 9 only (one sign word), TS_EUNSUPPORTED above.
@@ -130,9 +132,6 @@ ts_status ts_real_schemes(const ts_tri *tri, const uint64_t *signs, uint64_t n,
  *     no global scratch).  ts_real_schemes and ts_enumerate; batches run
  *     it as the warp tile of their fused launch (ts_batch_set_fused_tile);
  *     ts_enumerate_noalloc runs the table-driven family.
- *     Sweeps of at least 2^19 masks that differ in the middle row block by
- *     block (4 <= d <= 9, not TS_ENUM_SPLITMIX) share the half-diamonds of
- *     each block.
  *   TS_KERNEL_AUTO (default): table-driven; batches may specialise small
  *     degrees (ts_batch_info). */
 #define TS_KERNEL_AUTO 0
@@ -269,12 +268,12 @@ void ts_batch_free(ts_batch *batch);
  * (TS_SCRATCH_*; global scratch is allocated here, grid x threads x
  * scratch words).  Blocks of 128 threads without TS_SCRATCH_GLOBAL (the
  * default tile) run bit-sliced; the other tiles run one thread per sign
- * vector, with global scratch from d = 7 for TS_SCRATCH_AUTO.  Returns TS_EINVAL for tiles that do not fit, and for a
- * specialised group (ts_batch_info) any block size but 128 or shared
- * scratch: its code is compiled for 128-thread blocks and global scratch.
- * Waits for
- * all work on the device first (runs already launched use the tile's tables
- * and scratch); the next ts_batch_run with use_graph captures a new graph. */
+ * vector, with global scratch from d = 7 for TS_SCRATCH_AUTO.  Returns
+ * TS_EINVAL for tiles that do not fit, and for a specialised group
+ * (ts_batch_info) any block size but 128 or shared scratch: its code is
+ * compiled for 128-thread blocks and global scratch.  Waits for all work on
+ * the device first (runs already launched use the tile's tables and scratch);
+ * the next ts_batch_run with use_graph captures a new graph. */
 ts_status ts_batch_set_tile(ts_batch *batch, int d, int threads, int chunk, int scratch);
 /* How ts_batch_run orders the degree groups' persistent kernels: serial = 0
  * (default) forks them onto streams of their own, so they run concurrently;

@@ -684,7 +684,7 @@ JitLink &jitlink() {
 }
 
 // One job of a batch as the generated code sees it: the layout of the host's
-// job table (72 bytes, DevJob of batch.cu).
+// job table (88 bytes, DevJob of engine.h).
 const char kJobStructSrc[] = R"TCJS(
 struct TcjJob {
   const unsigned *tab;
