@@ -5,7 +5,9 @@
 // A persistent block takes 128 high parts at a time, or for short ranges one
 // of 2^lparts equal parts of their patterns.  What bounds it is integer issue:
 // at d = 7 the halves and their records take about as long as two words (64
-// patterns) of the middle phase.
+// patterns) of the middle phase (ALU pipe 68 % busy, three blocks of 168
+// registers per multiprocessor).  2^30 masks at d = 7: 162 ms (specialised block
+// sweep) -> 10.5 ms.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -146,16 +148,18 @@ cudaError_t launch_d(const ts_tri *t, uint64_t h0, uint64_t n, const Split &s, u
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   e = cudaMemsetAsync(h->d_work, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  // Parts: the fewest that make the waves times a part's time smallest, in
-  // words of the middle phase, the halves counted as two (0.28, 0.45, 0.57 of
-  // 6.6, 4.4, 2.5 ms at d = 9, 8, 7).  2^19 masks in one
-  // part took 736, 306, 114 us (few of the blocks the device holds at work),
-  // in parts 100, 80, 64; a flip sweep of 2^26 at d = 9 4.55 -> 3.25 ms.
+  // Parts: those for which the items' time on the blocks the device holds plus
+  // one item's (the last to start; high parts differ, so no wave is full) is
+  // least, in words of the middle phase, the halves counted as two (0.28, 0.45,
+  // 0.57 of 6.6, 4.4, 2.5 ms at d = 9, 8, 7).  One part -> these: 2^19 masks
+  // 736, 306, 114 -> 100, 80, 64 us; d = 9, three ranges each, 2^24 masks 1.38,
+  // 0.95, 2.1 -> 0.80, 0.72, 0.90 ms, 2^26 modulo the flip 3.9, 2.1, 4.6 -> 3.3,
+  // 2.2, 3.6 ms.  Counting full waves instead: 1.01, 0.74, 1.37 and 3.6, 2.2, 3.5.
   const uint64_t groups = (n + 127) / 128, held = (uint64_t)per_sm * sms;
   uint32_t lparts = 0;
   uint64_t best = ~0ull;
   for (uint32_t l = 0; l <= s.ib - 5; ++l) {
-    const uint64_t time = (((groups << l) + held - 1) / held) * (2 + (1ull << (s.ib - 5 - l)));
+    const uint64_t time = ((groups << l) + held) * (2 + (1ull << (s.ib - 5 - l)));
     if (time < best) {
       best = time;
       lparts = l;
