@@ -5,8 +5,9 @@
 // the batch runs ONE persistent kernel over all jobs of that degree: blocks
 // pull (job, chunk) work items from a counter, re-stage a job's tables into
 // shared memory with cp.async.bulk when the job changes, generate the sign
-// vectors on the device, classify them with the table-driven sweep
-// (Algorithm 1) and add the codes to the job's own device hash histogram
+// vectors on the device, classify them with Algorithm 1 (bit-sliced,
+// sliced_jobs.cu; other tiles than the default with one thread per sign
+// vector) and add the codes to the job's own device hash histogram
 // (warp-aggregated atomics).  The per-degree kernels run on forked streams
 // inside one CUDA graph that is captured on the first run and replayed after;
 // each degree has its own tile shape (threads per block, instances per work

@@ -21,7 +21,8 @@
 // at d = 10, 195 KB at d = 16), and one launch has one size, so the degrees of
 // a launch share the occupancy of its largest.  The tiers run on forked
 // streams, the largest degrees first: the blocks of one fill the SMs that the
-// last blocks of another leave.
+// last blocks of another leave.  3.7e8 sign vectors of d = 5..10: 388 ms (one
+// thread per sign vector, one launch) -> 122 ms.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

@@ -182,7 +182,11 @@ __global__ void __launch_bounds__(TableK<D>::THREADS)
 // ------------------------------------------------ bit-sliced kernels ----
 //
 // Blocks of 128 threads classify 128 sign vectors at a time (tc_sliced.cuh; 64
-// from d = 13).
+// from d = 13).  Bound by issue (74 % of the slots at d = 7, 57 % at d = 10,
+// where four blocks per multiprocessor do not hide the chains of the joins).
+// 2^22 random sign vectors at d = 7: 2.36 ms (specialised) -> 0.92 ms; sampled
+// sweeps of 2^21 at d = 10 5.37 -> 1.54 ms, of 2^18 at d = 16 17.2 -> 2.72 ms
+// (one thread per sign vector, scratch in global memory).
 // smem: tables (toff bytes) | mbarrier, work slot (128 bytes) | the block's
 // areas | hash table (sweeps of one-word codes).
 // From d = 13 (130 to 210 KB for 128 sign vectors) blocks of 64:
