@@ -360,7 +360,7 @@ bool pack_sliced_tables(const Diamond &D, std::vector<uint32_t> &tables, SlicedL
       if (can_join(v, i))
         (v < 2 * H ? half_sites : mid_sites).push_back((uint32_t)v | ((uint32_t)u << 16));
     }
-    for (size_t i = len; i < padded; ++i) fan.push_back((uint32_t)D.k[v]);
+    for (size_t i = len; i < padded; ++i) fan.push_back((uint32_t)D.k[v] | 1u << 26);
   }
   // the half-diamonds are mirror images: as many steps each
   if (half_steps[1] != 2 * half_steps[0]) return false;

@@ -173,7 +173,7 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
 #pragma unroll
       for (u32 i = 0; i < 4; ++i) {
         const u32 e = i == 0 ? q.a : i == 1 ? q.b : i == 2 ? q.c : q.d, u = (e >> 8) & 0xFFFFu;
-        if (u == 0) continue;  // padding: vertex 0 is never next to the middle row
+        if (e & (1u << 26)) continue;  // padding
         links |= ((e >> 30) & 1u) << n;
         if (u >= 2 * K::H) {
           left = 1u << n;

@@ -58,7 +58,7 @@
 //            last step padded (one step for an empty fan): k(u) (8 bits) |
 //            u << 8 (16 bits) | "can start a second run" << 24 | "another step
 //            of this vertex follows" << 25 | link << 30 |
-//            (c(u) ^ c(v) ^ 1) << 31; padding: k(v), never of v's sign
+//            (c(u) ^ c(v) ^ 1) << 31; padding: k(v) (never of v's sign) | 1 << 26
 //   vd[V]    u of the first fan entry | "the fan is not empty" << 15
 //   site[]   32 per chunk of join events: v | u << 16: the half-diamonds'
 //            sites, one chunk of boundary pairs, the middle row's sites

@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 import tcurve_inputs as ti
+from triangulations import apex_triangulation
 
 pytestmark = pytest.mark.gpu
 
@@ -75,3 +76,28 @@ def test_block_sweep_matches_the_specialised_kernels(eng, d, flag, name):
             assert failed == 0 and int(counts.sum()) == hi - lo
             got.append(dict(zip(codes[:, 0].tolist(), counts.tolist())))
         assert got[0] == got[1], (lo, hi)
+
+
+def _triangulation(d, name):
+    kind, k = name.split("-")
+    return {"apex": apex_triangulation}[kind](d, int(k))
+
+
+@pytest.mark.parametrize("d,flag,name", [
+    (5, 0, "apex-2"), (6, 2, "apex-1"), (7, 1, "apex-3"), (8, 8, "apex-3"), (9, 0, "apex-2")])
+def test_block_sweep_on_irregular_triangulations(eng, d, flag, name):
+    """Whole blocks and ragged ends under AUTO and TABLE against the
+    specialised kernels."""
+    tri = eng.Triangulation(d, _triangulation(d, name))
+    bits = tri.num_points - {0: 0, 1: 1, 2: 3, 8: 3}[flag]
+    lo = (1 << (bits - 1)) - 5
+    hi = min(lo + (1 << 20) + 77, 1 << bits)
+    got = []
+    for kind in (eng.TS_KERNEL_SPECIALIZED, eng.TS_KERNEL_AUTO, eng.TS_KERNEL_TABLE):
+        tri.set_kernel(kind)
+        h = eng.Histogram(4096, 1)
+        eng.enumerate_schemes(tri, lo, hi, h, flag)
+        codes, counts, failed = h.read()
+        assert failed == 0 and int(counts.sum()) == hi - lo
+        got.append(dict(zip(codes[:, 0].tolist(), counts.tolist())))
+    assert got[1] == got[0] and got[2] == got[0]

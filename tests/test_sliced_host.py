@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 
 import tcurve_inputs as ti
+from triangulations import apex_triangulation
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -78,3 +79,29 @@ def test_block_sweep_on_the_host(sliced_exe, tmp_path, d):
             assert out.returncode == 0, (name, mode, out.stdout + out.stderr)
             taken = int(out.stdout.split("middle phase=")[1].split()[0])
             assert taken == (0 if (name, d) == ("fan", 9) else 128), out.stdout
+
+
+def _block_sweep(exe, tmp_path, d, edges, mode, seed=1):
+    """Run the block sweep's host emulation; it agrees with the oracle.
+    Returns how many of the 128 high parts the middle phase took."""
+    np.savetxt(tmp_path / "tri.txt", edges, fmt="%d")
+    out = subprocess.run([str(exe), str(d), str(tmp_path / "tri.txt"), mode, str(seed)],
+                         capture_output=True, text=True)
+    assert out.returncode == 0, (mode, out.stdout + out.stderr)
+    return int(out.stdout.split("middle phase=")[1].split()[0])
+
+
+MAPS = {"plain": 1, "flip": 0, "reduced": -1, "orbits": 1}  # middle-row bits less d
+
+
+def _maps(d, every):
+    return [m for m, b in MAPS.items() if d + b >= 5 and (every or m == "plain")]
+
+
+@pytest.mark.parametrize("d,k", [(d, k) for d in range(4, 10) for k in range(1, d) if np.gcd(d, k) == 1])
+def test_block_sweep_keeps_vertex_0_beside_the_middle_row(sliced_exe, tmp_path, d, k):
+    """An edge (0, d)-(k, 0): the first vertex of the sweep is a neighbour of
+    the middle row."""
+    for mode in _maps(d, every=k == {5: 2, 6: 1, 7: 3, 8: 3, 9: 2}.get(d)):
+        taken = _block_sweep(sliced_exe["blocks"], tmp_path, d, apex_triangulation(d, k), mode)
+        assert taken == (0 if d >= 8 and k in (1, d - 1) else 128)
