@@ -166,7 +166,11 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
   // vertex before it
   u32 open = 0, tog = 0, vi = 0;
   {
-    u32 m0 = 0, m1 = 0, bits = 0, links = 0, left = 0, n = 0;
+    // The four choices of the vertex at once, a bit each (choice k: sigma = k &
+    // 1, of one sign with the vertex before if k & 2): the ones for which the
+    // last entry had the vertex's sign, and 1 minus the runs modulo 2.  A fan
+    // may have any length.
+    u32 m0 = 0, m1 = 0, same = 0, runs = 15;
     const TcQuad *f = reinterpret_cast<const TcQuad *>(tab + tab[3]) + 2 * tab[0];
     for (u32 s = 2 * tab[0]; s < tab[8]; ++s, ++f) {
       const TcQuad q = *f;
@@ -174,26 +178,20 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
       for (u32 i = 0; i < 4; ++i) {
         const u32 e = i == 0 ? q.a : i == 1 ? q.b : i == 2 ? q.c : q.d, u = (e >> 8) & 0xFFFFu;
         if (e & (1u << 26)) continue;  // padding
-        links |= ((e >> 30) & 1u) << n;
-        if (u >= 2 * K::H) {
-          left = 1u << n;
-        } else {
+        u32 now = 12;
+        if (u < 2 * K::H) {
           // sigma of the middle vertex for which the two have one sign
           const u32 b = ((u32)(sig >> (e & 63u)) ^ (e >> 31) ^ 1u) & 1u;
           const u32 c = 1u << comp_of(u);
           m0 |= b ? 0u : c;
           m1 |= b ? c : 0u;
-          bits |= b << n;
+          now = 5u << b;
         }
-        ++n;
+        runs ^= now & ~(same & tc_bitmask(e, 30));
+        same = now;
       }
       if (q.a & (1u << 25)) continue;  // another step of this vertex
-      const u32 all = ((1u << n) - 1u) & ~left;
-#pragma unroll
-      for (u32 k = 0; k < 4; ++k) {
-        const u32 e = ((k & 1u) ? bits : ~bits & all) | ((k & 2u) ? left : 0u);
-        tog |= ((1u + (u32)__popc(e & ~((e << 1) & links))) & 1u) << ((4u * vi + k) & 31u);
-      }
+      tog |= runs << ((4u * vi) & 31u);
       rec[(K::R_ADJ + vi) * K::T] = m0;
       m.scr[vi * K::T + t] = m1;
       open |= m0 | m1;
@@ -202,7 +200,8 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
         tog = 0;
       }
       ++vi;
-      m0 = m1 = bits = links = left = n = 0;
+      m0 = m1 = same = 0;
+      runs = 15;
     }
   }
   const u32 N = (u32)__popc(open);

@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 import tcurve_inputs as ti
-from triangulations import apex_triangulation
+from triangulations import apex_triangulation, greedy_triangulation, hub_triangulation
 
 pytestmark = pytest.mark.gpu
 
@@ -80,11 +80,12 @@ def test_block_sweep_matches_the_specialised_kernels(eng, d, flag, name):
 
 def _triangulation(d, name):
     kind, k = name.split("-")
-    return {"apex": apex_triangulation}[kind](d, int(k))
+    return {"apex": apex_triangulation, "hub": hub_triangulation, "greedy": greedy_triangulation}[kind](d, int(k))
 
 
 @pytest.mark.parametrize("d,flag,name", [
-    (5, 0, "apex-2"), (6, 2, "apex-1"), (7, 1, "apex-3"), (8, 8, "apex-3"), (9, 0, "apex-2")])
+    (5, 0, "apex-2"), (6, 2, "apex-1"), (7, 1, "apex-3"), (8, 8, "apex-3"), (9, 0, "apex-2"),
+    (6, 0, "hub-8"), (7, 8, "hub-8"), (8, 2, "hub-9"), (9, 1, "hub-9"), (8, 0, "greedy-19")])
 def test_block_sweep_on_irregular_triangulations(eng, d, flag, name):
     """Whole blocks and ragged ends under AUTO and TABLE against the
     specialised kernels."""

@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 
 import tcurve_inputs as ti
-from triangulations import apex_triangulation
+from triangulations import apex_triangulation, greedy_triangulation, hub_triangulation
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -105,3 +105,19 @@ def test_block_sweep_keeps_vertex_0_beside_the_middle_row(sliced_exe, tmp_path, 
     for mode in _maps(d, every=k == {5: 2, 6: 1, 7: 3, 8: 3, 9: 2}.get(d)):
         taken = _block_sweep(sliced_exe["blocks"], tmp_path, d, apex_triangulation(d, k), mode)
         assert taken == (0 if d >= 8 and k in (1, d - 1) else 128)
+
+
+@pytest.mark.parametrize("d,n", [(6, 7), (6, 8), (7, 8), (8, 8), (8, 9), (9, 8), (9, 9)])
+def test_block_sweep_takes_fans_of_any_length(sliced_exe, tmp_path, d, n):
+    """The origin has 31, 35 or 39 earlier neighbours and the middle phase
+    takes every high part."""
+    for mode in _maps(d, every=n == 8):
+        assert _block_sweep(sliced_exe["blocks"], tmp_path, d, hub_triangulation(d, n), mode) == 128
+
+
+@pytest.mark.parametrize("d", [5, 6, 7, 8, 9])
+def test_block_sweep_on_random_triangulations(sliced_exe, tmp_path, d):
+    """Twenty triangulations with edges of any length, each in one mask map."""
+    maps = _maps(d, every=True)
+    for seed in range(20):
+        _block_sweep(sliced_exe["blocks"], tmp_path, d, greedy_triangulation(d, seed), maps[seed % len(maps)])

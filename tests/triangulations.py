@@ -43,3 +43,12 @@ def apex_triangulation(d: int, k: int, seed: int = 0) -> np.ndarray:
     """With the edge (0, d)-(k, 0), gcd(d, k) = 1: vertex (0, -d) of the
     reflected triangulation is next to the middle row."""
     return greedy_triangulation(d, seed, first=[(0, d, k, 0)], short=True)
+
+
+def hub_triangulation(d: int, n: int, seed: int = 0) -> np.ndarray:
+    """With the origin joined to n interior points (and (1, 0), (0, 1)): 4n + 3
+    neighbours of the middle vertex (0, 0) come before it in the sweep."""
+    inner = sorted((i + j, i, j) for i in range(1, d) for j in range(1, d - i) if gcd(i, j) == 1)
+    if len(inner) < n:
+        raise ValueError(f"degree {d} has {len(inner)} primitive interior points")
+    return greedy_triangulation(d, seed, first=[(0, 0, i, j) for _, i, j in inner[:n]], short=True)
