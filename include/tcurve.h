@@ -133,7 +133,10 @@ ts_status ts_real_schemes(const ts_tri *tri, const uint64_t *signs, uint64_t n,
  *     it as the warp tile of their fused launch (ts_batch_set_fused_tile);
  *     ts_enumerate_noalloc runs the table-driven family.
  *   TS_KERNEL_AUTO (default): table-driven; batches may specialise small
- *     degrees (ts_batch_info). */
+ *     degrees (ts_batch_info), and sweeps of at least 2^22 masks at d = 9 take
+ *     the specialised kernels for triangulations whose long edges at the x-axis
+ *     keep the block sweep from them (unless they are captured before the
+ *     kernels are built, ts_prepare). */
 #define TS_KERNEL_AUTO 0
 #define TS_KERNEL_TABLE 1
 #define TS_KERNEL_SPECIALIZED 2
@@ -166,8 +169,9 @@ ts_status ts_set_scratch(ts_tri *tri, int where);
 ts_status ts_set_occupancy(ts_tri *tri, int blocks_per_sm);
 
 /* Build the specialised kernels now (NVRTC compile and module load on the
- * current device; about a second), for TS_KERNEL_SPECIALIZED.  Call it before
- * capturing launches of such a triangulation in a CUDA graph, since the first
+ * current device; about a second), for TS_KERNEL_SPECIALIZED and the sweeps
+ * that TS_KERNEL_AUTO gives to them.  Call it before capturing launches of a
+ * TS_KERNEL_SPECIALIZED triangulation in a CUDA graph, since the first
  * specialised launch otherwise compiles.  Returns TS_ECUDA if compilation or loading fails
  * (ts_specialized_log then holds the compiler log), TS_EUNSUPPORTED for
  * d > 9. */

@@ -192,6 +192,11 @@ cudaError_t launch(const ts_tri *t, uint64_t h0, uint64_t n, const Split &s, uin
 // the pivots zero, tc_orbit_high).
 bool block_range(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, uint64_t *a, uint64_t *b) {
   if (t->d < 4 || t->d > 9 || (flags & TS_ENUM_SPLITMIX)) return false;
+  // More open components than the middle phase holds: the sliced kernel's own
+  // sweep, with more blocks per multiprocessor and no halves in vain (2^22 masks
+  // of three triangulations each, in this kernel -> there: d = 6 4.0 -> 0.73 ms,
+  // d = 8 6.2 -> 1.5, d = 9 6.7 -> 2.0; specialised 1.3, 1.8 and 1.7).
+  if (t->open > tc_block_nodes(t->d)) return false;
   const uint32_t ib = t->d + 1 - ((flags & TS_ENUM_FLIP) ? 1 : 0) - ((flags & TS_ENUM_REDUCED) ? 2 : 0);
   if (ib < 5) return false;  // fewer patterns than a word has bits
   const uint64_t first = (lo >> ib) + ((lo & ((1ull << ib) - 1)) != 0), last = hi >> ib;

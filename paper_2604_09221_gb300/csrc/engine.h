@@ -81,6 +81,14 @@ bool pack_diamond_tables(const Diamond &D, std::vector<uint32_t> &tables, TableL
 bool pack_warp_tables(const Diamond &D, std::vector<uint32_t> &tables, WarpLayout &lay);
 // Tables of the bit-sliced kernels (host.cpp; format in tc_sliced.cuh).
 bool pack_sliced_tables(const Diamond &D, std::vector<uint32_t> &tables, SlicedLayout &lay);
+// Components of the half-diamonds (antipodal boundary points identified) that
+// are next to the middle row, under the sign vector `mask` (one word; d <= 9).
+// Their number is the triangulation's: off the neighbourhood of a line the
+// projective plane is a disk, which m arcs of the curve cut into m + 1 such
+// components; the path of edges around the middle row, whose crossed edges the
+// arcs end at, holds every edge of one quadrant with its three mirror images,
+// and of these four two are crossed (Eq. 2; an edge's ends differ modulo 2).
+int open_components(const Diamond &D, uint64_t mask);
 // Label slot of every vertex in the table-driven sweep (a slot is reused once
 // its vertex has no later reader) and, in *nslots, how many slots are used.
 std::vector<int> lab_slots(const Diamond &D, int *nslots);
@@ -109,6 +117,7 @@ struct ts_tri {
   std::vector<uint32_t> host_stables;
   uint32_t *d_stables = nullptr;  // slay.words words (bit-sliced kernels)
   uint32_t *d_err = nullptr;     // device error word (scratch, owned here)
+  int open = 0;                  // components next to the middle row (d <= 9)
   tcurve::Diamond dia;
   int kernel = 0;                // TS_KERNEL_*
   int scratch = 0;               // TS_SCRATCH_* (both kernel families)

@@ -428,6 +428,27 @@ bool pack_sliced_tables(const Diamond &D, std::vector<uint32_t> &tables, SlicedL
   lay.chunks = ncb + nc1 + 1 + ncm;
   return true;
 }
+
+int open_components(const Diamond &D, uint64_t mask) {
+  const int n = 2 * D.d * D.d;  // vertices off the middle row
+  std::vector<int> up(n);
+  for (int v = 0; v < n; ++v) up[v] = v;
+  auto find = [&](int v) {
+    while (up[v] != v) v = up[v] = up[up[v]];
+    return v;
+  };
+  auto sign = [&](int v) { return (int)(mask >> D.k[v] & 1) ^ D.c[v]; };
+  for (int v = 0; v < n; ++v)
+    for (int u : D.fan[v])
+      if (sign(u) == sign(v)) up[find(u)] = find(v);
+  for (auto &p : D.anti)
+    if (p.second < n) up[find(p.first)] = find(p.second);
+  std::vector<char> open(n, 0);
+  for (int v = n; v < D.V; ++v)
+    for (int u : D.fan[v])
+      if (u < n) open[find(u)] = 1;
+  return (int)std::count(open.begin(), open.end(), 1);
+}
 }  // namespace tcurve
 
 namespace {
@@ -436,6 +457,7 @@ bool pack_tables(const Diamond &D, ts_tri *t) {
   if (!pack_diamond_tables(D, t->host_tables, t->lay)) return false;
   if (!pack_sliced_tables(D, t->host_stables, t->slay)) return false;
   if (!pack_warp_tables(D, t->host_wtables, t->wlay)) return false;
+  t->open = D.d <= kMaxSpecialized ? open_components(D, 0) : 0;
   t->V = D.V;
   return true;
 }
@@ -553,12 +575,32 @@ int ts_sign_words(const ts_tri *t) { return t ? t->sw : 0; }
 int ts_code_words(const ts_tri *t) { return t ? t->cw : 0; }
 
 namespace {
-// Kernel choice: the specialised kernels only when asked for.  AUTO takes the
-// table-driven (bit-sliced) kernels: on random sign vectors at d = 7 they
-// classify 4.6e9/s against the specialised query kernel's 1.8e9, and sweeps of
-// 2^14 masks and more are faster at every degree (2^19 masks: d = 7 172 ->
-// 64 us, d = 9 488 -> 100; 2^30 at d = 7 166 -> 10.4 ms).
+// Kernel choice: AUTO takes the table-driven (bit-sliced) kernels: on random
+// sign vectors at d = 7 they classify 4.6e9/s against the specialised query
+// kernel's 1.8e9, and sweeps of 2^14 masks and more are faster (2^19 masks: d =
+// 7 172 -> 64 us, d = 9 488 -> 100; 2^30 at d = 7 166 -> 10.4 ms), with one
+// exception below.
 bool want_specialised(const ts_tri *t) { return t->kernel == TS_KERNEL_SPECIALIZED; }
+
+// Triangulations with more components next to the middle row than the block
+// sweep holds are swept mask by mask.  Against the specialised block sweep that
+// takes 0.13 to 1.0 times as long at d = 5..8 (16 of them, 2^14 to 2^28 masks)
+// and at d = 9 up to 2^21 masks or with TS_ENUM_REDUCED (0.5 to 1.05); at d = 9
+// from 2^22 masks 1.13 to 1.5 times with 16 components, 1.0 to 1.4 with 18, 0.9
+// to 1.1 with 22 and 0.6 to 0.97 with 23 to 29.
+bool want_specialised_sweep(ts_tri *t, uint64_t n, uint32_t flags, cudaStream_t st) {
+  if (want_specialised(t)) return true;
+  if (t->kernel != TS_KERNEL_AUTO || t->d != 9 || t->open <= tc_block_nodes(9) || t->open > 22 ||
+      n < (1ull << 22) || (flags & (TS_ENUM_REDUCED | TS_ENUM_SPLITMIX)))
+    return false;
+  {
+    std::lock_guard<std::mutex> g(t->jit_mu);
+    if (t->jit) return true;
+  }
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;  // nothing is compiled in a capture
+  if (cudaStreamIsCapturing(st, &c) != cudaSuccess || c != cudaStreamCaptureStatusNone) return false;
+  return jit_prepare(t) == cudaSuccess;
+}
 }  // namespace
 
 ts_status ts_real_schemes(const ts_tri *tc, const uint64_t *signs, uint64_t n, uint64_t *codes,
@@ -768,7 +810,7 @@ ts_status ts_enumerate(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags
   ts_tri *tm = const_cast<ts_tri *>(t);
   if (tm->kernel == TS_KERNEL_WARP)
     return cuda_status(launch_enumerate_warp(tm, lo, hi, flags, h, (cudaStream_t)stream));
-  if (want_specialised(tm))
+  if (want_specialised_sweep(tm, hi - lo, flags, (cudaStream_t)stream))
     return cuda_status(launch_enumerate_jit(tm, lo, hi, flags, h, (cudaStream_t)stream));
   return cuda_status(launch_enumerate(t, lo, hi, flags, h, (cudaStream_t)stream));
 }

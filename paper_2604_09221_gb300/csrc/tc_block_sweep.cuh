@@ -34,8 +34,12 @@
 // (x, 1) and (x, -1) have opposite signs (Eq. 2).  So no region lies in the
 // middle row alone, and every run has a node.
 //
-// High parts with more than K::NB open comps or more than 32 comps (none on
-// the seeded regular triangulations) take the per-mask phases of tc_sliced.cuh.
+// The open comps are as many under every high part (open_components, engine.h):
+// d + 1 or fewer on the seeded regular triangulations up to d = 8, more the
+// more points the edges of the triangulation join to the x-axis.  Above K::NB
+// of them the block sweep is not launched (block_range).  High parts with more
+// than 32 comps (none seen below K::NB open ones) take the per-mask phases of
+// tc_sliced.cuh.
 #pragma once
 
 #include "tc_sliced.cuh"
@@ -45,7 +49,7 @@ template <int D_>
 struct TcSbK : TcSlK<D_, 4> {
   typedef TcSlK<D_, 4> Base;
   static constexpr u32 D = D_, M = 2 * D_ + 1;  // middle vertices
-  static constexpr u32 NA = D_ <= 8 ? D_ + 1 : 13, NB = D_ + 6 < 16 ? D_ + 6 : 16;
+  static constexpr u32 NA = D_ <= 8 ? D_ + 1 : 13, NB = tc_block_nodes(D_);
   // record of a high part (words, one column per thread)
   static constexpr u32 R_HDR = 0,          // comps | nodes << 8 | closed comps << 16 | star impossible << 24
                                            // | valid << 25 | corner edge signs << 26, 27
@@ -134,7 +138,7 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
   rec[K::R_HDR * K::T] = 0;
   // comps in the order of their smallest starts; chi of every comp modulo 2:
   // label starts plus join events
-  static_assert(Inst::MARK + 32 <= 256, "32 comps in label bytes");
+  static_assert(kBlockComps == 32 && Inst::MARK + 32 <= 256, "comps in label bytes, sets of them in words");
   u32 C = 0;
   {
     u32 n = 0;  // roots, before they are numbered
@@ -144,7 +148,7 @@ __device__ __forceinline__ void tc_sb_record(const TcSbMem &m, u32 t, u64 sig) {
         const u32 v = 32u * c + (u32)__ffs(w) - 1u;
         n += I.raw(v) == v;
       }
-    if (n > 32) return;  // not valid: the block's masks one by one
+    if (n > kBlockComps) return;  // not valid: the block's masks one by one
   }
   u32 chis = 0;
   C = tc_sl_number<typename K::Base>(I, [&](u32 r) { chis ^= 1u << r; });

@@ -95,6 +95,12 @@ constexpr TcLayout tc_layout(int d, bool vertex_labels, int max_threads) {
   return L;
 }
 
+// What the middle phase of the block sweep holds of a high part
+// (tc_block_sweep.cuh): components in all, and components next to the middle
+// row.
+constexpr int kBlockComps = 32;
+constexpr int tc_block_nodes(int d) { return d + 6 < 16 ? d + 6 : 16; }
+
 // Pivots of the orbit sweep (TS_ENUM_ORBITS, Sec. 3 symmetry).  The four
 // elements of (Z/2)^3 that keep sigma(0, 1) (sigma -> sigma + a + b i + c j
 // with a + c = 0 mod 2) change the high part of a mask (bits d+2 .. |A|-1:

@@ -85,7 +85,8 @@ def _triangulation(d, name):
 
 @pytest.mark.parametrize("d,flag,name", [
     (5, 0, "apex-2"), (6, 2, "apex-1"), (7, 1, "apex-3"), (8, 8, "apex-3"), (9, 0, "apex-2"),
-    (6, 0, "hub-8"), (7, 8, "hub-8"), (8, 2, "hub-9"), (9, 1, "hub-9"), (8, 0, "greedy-19")])
+    (6, 0, "hub-8"), (7, 8, "hub-8"), (8, 2, "hub-9"), (9, 1, "hub-9"), (8, 0, "greedy-19"),
+    (6, 2, "greedy-3"), (7, 8, "greedy-7"), (8, 1, "greedy-0"), (9, 0, "greedy-3")])
 def test_block_sweep_on_irregular_triangulations(eng, d, flag, name):
     """Whole blocks and ragged ends under AUTO and TABLE against the
     specialised kernels."""
@@ -102,3 +103,56 @@ def test_block_sweep_on_irregular_triangulations(eng, d, flag, name):
         assert failed == 0 and int(counts.sum()) == hi - lo
         got.append(dict(zip(codes[:, 0].tolist(), counts.tolist())))
     assert got[1] == got[0] and got[2] == got[0]
+
+
+@pytest.mark.parametrize("d,name", [(6, "greedy-3"), (7, "greedy-7"), (8, "greedy-0"), (9, "greedy-3")])
+def test_sweeps_the_block_sweep_cannot_hold_are_no_slower(eng, d, name):
+    """More components next to the middle row than the middle phase holds: the
+    default takes another way, at most 1.3 times the specialised kernels'
+    time (1.0 at most where both were timed; mask by mask inside the block
+    sweep it took 1.8 to 3.2 times as long)."""
+    import torch
+    tri = eng.Triangulation(d, _triangulation(d, name))
+    n = 1 << 22
+    lo = (1 << (tri.num_points - 2)) + 12345
+    h = eng.Histogram(4096, 1)
+    best = {}
+    for kind in (eng.TS_KERNEL_SPECIALIZED, eng.TS_KERNEL_AUTO):
+        tri.set_kernel(kind)
+        times = []
+        for _ in range(6):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            eng.enumerate_schemes(tri, lo, lo + n, h)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        best[kind] = min(times[1:])
+    assert best[eng.TS_KERNEL_AUTO] < 1.3 * best[eng.TS_KERNEL_SPECIALIZED], best
+
+
+@pytest.mark.parametrize("d,name,prepare", [(8, "apex-3", False), (9, "greedy-3", False), (9, "greedy-3", True)])
+def test_a_captured_sweep(eng, d, name, prepare):
+    """A first sweep in a CUDA graph: nothing is compiled in the capture, and
+    each replay adds the range's histogram."""
+    import torch
+    tri = eng.Triangulation(d, _triangulation(d, name))
+    if prepare:
+        tri.prepare()
+    n = 1 << 22
+    lo = (1 << (tri.num_points - 2)) + 12345
+    h = eng.Histogram(4096, 1)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        eng.enumerate_schemes(tri, lo, lo + n, h)
+    graph.replay()
+    graph.replay()
+    codes, counts, failed = h.read()
+    assert failed == 0 and int(counts.sum()) == 2 * n
+    tri.set_kernel(eng.TS_KERNEL_TABLE)
+    want = eng.Histogram(4096, 1)
+    eng.enumerate_schemes(tri, lo, lo + n, want)
+    wcodes, wcounts, _ = want.read()
+    np.testing.assert_array_equal(codes, wcodes)
+    np.testing.assert_array_equal(counts, 2 * wcounts)

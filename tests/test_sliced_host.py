@@ -121,3 +121,34 @@ def test_block_sweep_on_random_triangulations(sliced_exe, tmp_path, d):
     maps = _maps(d, every=True)
     for seed in range(20):
         _block_sweep(sliced_exe["blocks"], tmp_path, d, greedy_triangulation(d, seed), maps[seed % len(maps)])
+
+
+@pytest.fixture(scope="module")
+def open_exe(sliced_exe, tmp_path_factory):
+    csrc = os.path.join(ROOT, "paper_2604_09221_gb300", "csrc")
+    exe = tmp_path_factory.mktemp("open") / "run"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-w", f"-I{csrc}", f"-I{os.path.join(ROOT, 'oracle')}",
+                    f"-I{CUDA}/include", "-o", str(exe), os.path.join(HERE, "host", "run_open_components.cpp"),
+                    "-x", "c", os.path.join(ROOT, "oracle", "tcurve_oracle.c"), "-x", "none",
+                    f"-L{CUDA}/lib64", f"-Wl,-rpath,{CUDA}/lib64", "-lcudart", "-lpthread"],
+                   check=True, capture_output=True)
+    return exe
+
+
+@pytest.mark.parametrize("d", [5, 6, 7, 8, 9])
+def test_the_host_knows_what_the_middle_phase_holds(open_exe, sliced_exe, tmp_path, d):
+    """A triangulation's components next to the middle row, counted when it is
+    loaded: the same for every sign vector, and within the middle phase's limit
+    exactly if it takes the high parts."""
+    held = set()
+    for edges in ([ti.standard_triangulation(d), ti.fan_triangulation(d), apex_triangulation(d, 1)]
+                  + [greedy_triangulation(d, seed) for seed in range(8)]):
+        np.savetxt(tmp_path / "tri.txt", edges, fmt="%d")
+        out = subprocess.run([str(open_exe), str(d), str(tmp_path / "tri.txt"), "300"],
+                             capture_output=True, text=True)
+        assert out.returncode == 0, out.stderr
+        n, most = map(int, out.stdout.split())
+        mode = "reduced" if d > 5 else "plain"
+        assert (_block_sweep(sliced_exe["blocks"], tmp_path, d, edges, mode) == 128) == (n <= most)
+        held.add(n <= most)
+    assert held == {True, False}
