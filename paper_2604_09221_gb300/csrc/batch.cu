@@ -232,6 +232,23 @@ ts_status cuda_st(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? TS_ENOMEM : TS_ECUDA;
 }
 
+// Makes a device current for a scope (its calls are ordered by that device's
+// legacy stream), then the caller's again.
+struct DeviceScope {
+  cudaError_t status = cudaSuccess;
+  int device = -1;  // the caller's, if it is another
+  explicit DeviceScope(int wanted) {
+    int now = wanted;
+    status = cudaGetDevice(&now);
+    if (status != cudaSuccess || now == wanted) return;
+    status = cudaSetDevice(wanted);
+    if (status == cudaSuccess) device = now;
+  }
+  ~DeviceScope() {
+    if (device >= 0) cudaSetDevice(device);
+  }
+};
+
 // Packed histogram of one job: entries found, failed instances, error word, 0;
 // then per entry its code words and its count.
 constexpr uint64_t kPackHeader = 4;
@@ -957,11 +974,10 @@ ts_status ts_batch_read(ts_batch *b, int job, uint64_t *codes, uint64_t *counts,
   const uint64_t hs = b->jslots[job];
   const uint64_t ew = cw + 1;
   std::vector<unsigned long long> buf;
-  std::lock_guard<std::mutex> lock(b->read_mu);
   cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
-  int device = b->device;  // the caller's: the pack kernel runs on the batch's
-  if (e == cudaSuccess) e = cudaGetDevice(&device);
-  if (e == cudaSuccess && device != b->device) e = cudaSetDevice(b->device);
+  std::lock_guard<std::mutex> lock(b->read_mu);  // of d_pack, up to the last copy
+  const DeviceScope scope(b->device);
+  if (e == cudaSuccess) e = scope.status;
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_pack, 0, 8, cudaStreamLegacy);
   if (e == cudaSuccess) {
     const uint64_t blocks = std::min<uint64_t>((hs + 255) / 256, 1024);
@@ -970,7 +986,6 @@ ts_status ts_batch_read(ts_batch *b, int job, uint64_t *codes, uint64_t *counts,
         b->d_pack);
     e = cudaGetLastError();
   }
-  if (device != b->device) cudaSetDevice(device);
   const uint64_t first = std::min(b->pack_cap, kPackFirst);
   buf.resize(kPackHeader + first * ew);
   if (e == cudaSuccess) e = cudaMemcpy(buf.data(), b->d_pack, buf.size() * 8, cudaMemcpyDeviceToHost);
