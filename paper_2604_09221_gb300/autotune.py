@@ -2,17 +2,19 @@
 
 For every degree in a batch the persistent kernel has three knobs: threads
 per block, sign vectors per work item, and where the per-thread scratch
-lives (shared memory, or global memory for the large degrees whose scratch
-leaves few warps per SM).  A degree group that runs specialised code
+lives: blocks of 128 threads with shared memory classify 128 sign vectors
+together (bit-sliced), the others one sign vector per thread.  A degree group that runs specialised code
 (ts_batch_info: compiled per triangulation, 128-thread blocks and global
 scratch fixed at compile time) has one knob, the sign vectors per work item.
 The tuner times candidate tiles on the batch's own jobs of that degree (a
 sub-batch, so degrees are tuned independently), keeps the fastest, and can
 store the choice in a JSON cache keyed by GPU name, degree and kernel family
-(path from the argument or the TCURVE_TILE_CACHE environment variable).
+(path from the argument or the TCURVE_TILE_CACHE environment variable).  An
+entry holds the generation of the kernels it was timed with (GENERATION);
+entries of another one are timed again.
 
-In the fused launch (ts_batch_set_fused: one kernel for all degrees) a
-degree's tile is the kind (one thread or, from d = 7, one warp per sign
+In the fused launch (ts_batch_set_fused: one kernel per tier of degrees) a
+degree's tile is the kind (bit-sliced or, from d = 7, one warp per sign
 vector) and the sign vectors per work item; autotune_fused times those the
 same way, on fused sub-batches of one degree.
 """
@@ -22,6 +24,7 @@ import json
 import os
 from typing import Dict, Iterable, Optional, Tuple
 
+GENERATION = 2                   # raised when a tile stands for another kernel than before
 THREADS = (64, 96, 128, 192, 256)
 CHUNK_PER_THREAD = (4, 16, 64)
 SHARED, GLOBAL = 1, 2            # TS_SCRATCH_SHARED, TS_SCRATCH_GLOBAL
@@ -30,6 +33,13 @@ SHARED, GLOBAL = 1, 2            # TS_SCRATCH_SHARED, TS_SCRATCH_GLOBAL
 def scratch_choices(d: int):
     """Scratch placements worth timing: shared below d = 8, both above."""
     return (SHARED,) if d < 8 else (SHARED, GLOBAL)
+
+
+def _cached(store: dict, key: str, fields: int):
+    """The first `fields` of a cache entry, if it was timed with these kernels:
+    [*tile, ms, GENERATION]."""
+    entry = store.get(key, [])
+    return tuple(entry[:fields]) if entry[fields + 1:] == [GENERATION] else None
 
 
 def _gpu_name() -> str:
@@ -107,12 +117,13 @@ def autotune(tris, counts, bases, cache: Optional[str] = None, reps: int = 3,
         sel = ([tris[i] for i in idx], [counts[i] for i in idx], [bases[i] for i in idx])
         sub = Batch(*sel)   # its kernel family decides the tile space
         key = f"{gpu}|d={d}|{sub.info(d)['kernel']}|tile3"
-        if key in store:
-            tiles[d] = tuple(store[key][:3])
+        tile = _cached(store, key, 3)
+        if tile:
+            tiles[d] = tile
         else:
             t, c, s, ms = tune_degree(*sel, threads, chunk_per_thread, reps, sub=sub)
             tiles[d] = (t, c, s)
-            store[key] = [t, c, s, ms]
+            store[key] = [t, c, s, ms, GENERATION]
         sub.close()
     if cache:
         tmp = cache + ".tmp"
@@ -128,7 +139,7 @@ def apply(batch, tiles: Dict[int, Tuple[int, ...]]):
             batch.set_tile(d, *tile)
 
 
-# fused launch: work items of 128 x c sign vectors; warp tiles from d = 7
+# fused plan: work items of 128 x c sign vectors; warp tiles from d = 7
 FUSED_THREAD_CHUNKS = (4, 8, 16, 64)
 FUSED_WARP_CHUNKS = (2, 8)
 FUSED_WARP_FROM = 7
@@ -181,14 +192,15 @@ def autotune_fused(tris, counts, bases, cache: Optional[str] = None, reps: int =
     for d in sorted({t.d for t in tris}):
         idx = [i for i, t in enumerate(tris) if t.d == d]
         key = f"{gpu}|d={d}|fused|tile2"
-        if key in store:
-            tiles[d] = tuple(store[key][:2])
+        tile = _cached(store, key, 2)
+        if tile:
+            tiles[d] = tile
         else:
             kind, chunk, ms = tune_fused_degree([tris[i] for i in idx], [counts[i] for i in idx],
                                                 [bases[i] for i in idx], reps, thread_chunks,
                                                 warp_chunks)
             tiles[d] = (kind, chunk)
-            store[key] = [kind, chunk, ms]
+            store[key] = [kind, chunk, ms, GENERATION]
     if cache:
         tmp = cache + ".tmp"
         with open(tmp, "w") as f:

@@ -185,3 +185,21 @@ def test_fused_tiles_per_degree_with_cache(monkeypatch, tmp_path):
     applied = FakeFusedBatch(tris, [1, 1, 1], [0, 0, 0])
     autotune.apply_fused(applied, tiles)
     assert applied.tiles == tiles
+
+
+def test_tiles_timed_with_other_kernels_are_timed_again(monkeypatch, fakes, tmp_path):
+    """Cache entries without the present generation (older files have none) are
+    replaced, plain and fused; the others are kept."""
+    cache = str(tmp_path / "tiles.json")
+    json.dump({"FakeGPU|d=5|table|tile3": [64, 256, 2, 0.1], "FakeGPU|d=13|fused|tile2": [3, 256, 0.1],
+               "FakeGPU|d=5|fused|tile2": [1, 512, 0.1, autotune.GENERATION],
+               "FakeGPU|d=10|table|tile3": [64, 256, 1, 0.1, autotune.GENERATION - 1]}, open(cache, "w"))
+    tiles = autotune.autotune([FakeTri(5), FakeTri(10)], [1, 2], [0, 0], cache=cache)
+    assert tiles == {5: (96, 96 * 64, autotune.SHARED), 10: (128, 128 * 16, autotune.GLOBAL)}
+    assert fakes
+    monkeypatch.setattr(eng, "Batch", FakeFusedBatch)
+    monkeypatch.setattr(autotune, "_time_batch", lambda batch, reps: 1.0 + (batch.tile != (1, 1024)))
+    tiles = autotune.autotune_fused([FakeTri(5), FakeTri(13)], [1, 2], [0, 0], cache=cache)
+    assert tiles == {5: (1, 512), 13: (1, 1024)}
+    store = json.load(open(cache))
+    assert all(e[-1] == autotune.GENERATION for e in store.values())
