@@ -181,20 +181,14 @@ __global__ void __launch_bounds__(TableK<D>::THREADS)
 
 // ------------------------------------------------ bit-sliced kernels ----
 //
-// Blocks of 128 threads classify 128 sign vectors at a time (tc_sliced.cuh; 64
-// from d = 13).  Bound by issue (74 % of the slots at d = 7, 57 % at d = 10,
+// Blocks of 128 threads classify 128 sign vectors at a time (64 or 192 from d =
+// 13, tc_sl_wide).  Bound by issue (74 % of the slots at d = 7, 57 % at d = 10,
 // where four blocks per multiprocessor do not hide the chains of the joins).
 // 2^22 random sign vectors at d = 7: 2.36 ms (specialised) -> 0.92 ms; sampled
 // sweeps of 2^21 at d = 10 5.37 -> 1.54 ms, of 2^18 at d = 16 17.2 -> 2.72 ms
 // (one thread per sign vector, scratch in global memory).
 // smem: tables (toff bytes) | mbarrier, work slot (128 bytes) | the block's
 // areas | hash table (sweeps of one-word codes).
-// From d = 13 (130 to 210 KB for 128 sign vectors) blocks of 64:
-// what limits them is the blocks a multiprocessor's shared memory holds
-// (d = 13: three of 64, one of 128; 0.40 against 0.26e9 schemes/s).
-template <int D>
-using SlicedK = TcSlK<D, D <= 12 ? 4 : 2>;
-
 template <class K>
 __global__ void __launch_bounds__(K::T)
     sliced_real_schemes_kernel(SlicedLayout L, const uint32_t *__restrict__ gtab,
@@ -393,11 +387,10 @@ struct GlobalScratch {
   }
 };
 
-template <int D>
-cudaError_t real_schemes_sliced(const ts_tri *t, const uint64_t *signs, uint64_t n, uint64_t *codes,
+template <class K>
+cudaError_t real_schemes_blocks(const ts_tri *t, const uint64_t *signs, uint64_t n, uint64_t *codes,
                                 cudaStream_t st) {
-  typedef SlicedK<D> K;
-  const size_t smem = sliced_table_bytes(t->slay.words) + 128 + (size_t)tc_sl_words<K>(t->slay.chunks) * 4;
+  const size_t smem = tc_sl_bytes<K>(t->slay.words, t->slay.chunks);
   unsigned grid = 0;
   cudaError_t e = persistent_grid(t, 0, sliced_real_schemes_kernel<K>, K::T, smem, (n + K::T - 1) / K::T, &grid);
   if (e != cudaSuccess) return e;
@@ -405,12 +398,10 @@ cudaError_t real_schemes_sliced(const ts_tri *t, const uint64_t *signs, uint64_t
   return cudaGetLastError();
 }
 
-template <int D>
-cudaError_t enumerate_sliced(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *h,
+template <class K>
+cudaError_t enumerate_blocks(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *h,
                              cudaStream_t st) {
-  typedef SlicedK<D> K;
-  const size_t smem = sliced_table_bytes(t->slay.words) + 128 + (size_t)tc_sl_words<K>(t->slay.chunks) * 4 +
-                      (size_t)K::HASH * 16;
+  const size_t smem = tc_sl_bytes<K>(t->slay.words, t->slay.chunks) + (size_t)K::HASH * 16;
   const uint64_t total = hi - lo;
   unsigned grid = 0;
   cudaError_t e = persistent_grid(t, 1, sliced_enumerate_kernel<K>, K::T, smem, (total + K::T - 1) / K::T, &grid);
@@ -419,6 +410,22 @@ cudaError_t enumerate_sliced(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t
   if (e != cudaSuccess) return e;
   sliced_enumerate_kernel<K><<<grid, K::T, smem, st>>>(t->slay, t->d_stables, lo, total, flags, *h);
   return cudaGetLastError();
+}
+
+template <int D>
+cudaError_t real_schemes_sliced(const ts_tri *t, const uint64_t *signs, uint64_t n, uint64_t *codes,
+                                cudaStream_t st) {
+  return tc_sl_wide<D>(t->slay.words, t->slay.chunks)
+             ? real_schemes_blocks<TcSlWide<D>>(t, signs, n, codes, st)
+             : real_schemes_blocks<TcSlNarrow<D>>(t, signs, n, codes, st);
+}
+
+template <int D>
+cudaError_t enumerate_sliced(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *h,
+                             cudaStream_t st) {
+  return tc_sl_wide<D>(t->slay.words, t->slay.chunks)
+             ? enumerate_blocks<TcSlWide<D>>(t, lo, hi, flags, h, st)
+             : enumerate_blocks<TcSlNarrow<D>>(t, lo, hi, flags, h, st);
 }
 
 template <int D>

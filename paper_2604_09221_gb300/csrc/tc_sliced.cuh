@@ -729,3 +729,27 @@ __device__ __forceinline__ void tc_sl_classify(const TcSlMem &m, const TcSig<K::
   tc_sl_finish<K>(m, I, t, R, root, star, err, code);
 }
 #endif
+
+// ---- launch shape of the query, sweep and batch kernels ----
+// Bytes of shared memory of a block: tables, mbarrier and work slot, areas.
+template <class K>
+constexpr size_t tc_sl_bytes(u32 table_words, u32 chunks) {
+  return ((size_t)table_words * 4 + 127) / 128 * 128 + 128 + (size_t)tc_sl_words<K>(chunks) * 4;
+}
+// Blocks of 128 sign vectors; from d = 13 (130 to 195 KB) of 64, what limits
+// them being the sign vectors a multiprocessor's shared memory holds (d = 13:
+// three blocks of 64, one of 128; 0.40 against 0.28e9 schemes/s).
+template <int D>
+using TcSlNarrow = TcSlK<D, D <= 12 ? 4 : 2>;
+// Or, at d = 13 and 14, of 192 where that is more: one block of 192 against two
+// of 64 at d = 14 (2^21 queries 10.2 -> 7.4 ms; one thread per sign vector with
+// scratch in global memory 8.6; the same from 2^16 down).  Above, 192 do not fit.
+template <int D>
+using TcSlWide = TcSlK<D, D == 13 || D == 14 ? 6 : D <= 12 ? 4 : 2>;
+template <int D>
+constexpr bool tc_sl_wide(u32 table_words, u32 chunks) {
+  constexpr size_t BLOCK = 227 * 1024, SM = 228 * 1024, RESERVED = 1024;  // of a block
+  const size_t n = tc_sl_bytes<TcSlNarrow<D>>(table_words, chunks), w = tc_sl_bytes<TcSlWide<D>>(table_words, chunks);
+  return TcSlWide<D>::T > TcSlNarrow<D>::T && w <= BLOCK &&
+         SM / (w + RESERVED) * TcSlWide<D>::T > SM / (n + RESERVED) * TcSlNarrow<D>::T;
+}

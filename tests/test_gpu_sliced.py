@@ -156,3 +156,57 @@ def test_a_captured_sweep(eng, d, name, prepare):
     wcodes, wcounts, _ = want.read()
     np.testing.assert_array_equal(codes, wcodes)
     np.testing.assert_array_equal(counts, 2 * wcounts)
+
+
+@pytest.mark.parametrize("d", [13, 14])
+def test_ragged_blocks_of_64_and_192(eng, orc, d):
+    """Queries and sampled sweeps around the blocks' sizes, and nothing written
+    behind the last code."""
+    import torch
+    for edges in (ti.regular_triangulation(d, seed=d), greedy_triangulation(d, 3)):
+        tri = eng.Triangulation(d, edges)
+        otri = orc.triangles(d, edges)
+        want = orc.real_schemes(d, otri, ti.splitmix_sign_vectors(d, 77, 1000))
+        for n in (1, 63, 64, 65, 191, 192, 193, 1000):
+            out = torch.full((n + 4, tri.code_words), -7, dtype=torch.int64, device="cuda")
+            tri.real_schemes(eng.splitmix_masks(d, 77, n), out=out)
+            got = out.cpu().numpy()
+            assert (got[:n].view(np.uint64) == want[:n]).all(), n
+            assert (got[n:] == -7).all()
+            h = eng.Histogram(2048, tri.code_words)
+            eng.enumerate_schemes(tri, 77, 77 + n, h, eng.TS_ENUM_SPLITMIX)
+            codes, counts, failed = h.read()
+            assert failed == 0
+            assert ({eng.code_to_int(c): int(k) for c, k in zip(codes, counts)}
+                    == dict(collections.Counter(orc.code_to_int(c) for c in want[:n]))), n
+
+
+def _ms(run, reps=5):
+    """Least time of a call on the device, in ms."""
+    import torch
+    times = []
+    for _ in range(reps + 1):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        run()
+        b.record()
+        b.synchronize()
+        times.append(a.elapsed_time(b))
+    return min(times[1:])
+
+
+@pytest.mark.parametrize("d", [13, 14, 15])
+def test_long_queries_are_no_slower_than_one_thread_per_sign_vector(eng, d):
+    """2^20 sign vectors under AUTO against the kernels with scratch in global
+    memory (0.80, 0.85 and 0.91 of their time; with two blocks of 64 at d = 14
+    it was 1.19)."""
+    import torch
+    tri = eng.Triangulation(d, ti.regular_triangulation(d, seed=d))
+    signs = eng.splitmix_masks(d, 5, 1 << 20)
+    out = torch.empty((1 << 20, tri.code_words), dtype=torch.int64, device="cuda")
+    ms = {}
+    for kind, scratch in ((eng.TS_KERNEL_AUTO, 0), (eng.TS_KERNEL_TABLE, 2)):
+        tri.set_kernel(kind)
+        tri.set_scratch(scratch)
+        ms[kind] = _ms(lambda: tri.real_schemes(signs, out=out))
+    assert ms[eng.TS_KERNEL_AUTO] < 1.05 * ms[eng.TS_KERNEL_TABLE], ms

@@ -152,3 +152,21 @@ def test_the_host_knows_what_the_middle_phase_holds(open_exe, sliced_exe, tmp_pa
         assert (_block_sweep(sliced_exe["blocks"], tmp_path, d, edges, mode) == 128) == (n <= most)
         held.add(n <= most)
     assert held == {True, False}
+
+
+@pytest.mark.parametrize("d", [13, 14])
+def test_wide_blocks_on_the_host(tmp_path, d):
+    """Blocks of 192 sign vectors: standard, fan and a random triangulation."""
+    if not shutil.which("g++") or not os.path.exists(os.path.join(CUDA, "include", "cuda_runtime.h")):
+        pytest.skip("needs g++ and the CUDA headers")
+    csrc, exe = os.path.join(ROOT, "paper_2604_09221_gb300", "csrc"), tmp_path / "run"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-w", "-DTC_SL_GROUPS=6", f"-I{csrc}",
+                    f"-I{os.path.join(ROOT, 'oracle')}", f"-I{CUDA}/include", "-o", str(exe),
+                    os.path.join(HERE, "host", "run_sliced_sweep.cpp"),
+                    "-x", "c", os.path.join(ROOT, "oracle", "tcurve_oracle.c"), "-x", "none",
+                    f"-L{CUDA}/lib64", f"-Wl,-rpath,{CUDA}/lib64", "-lcudart", "-lpthread"],
+                   check=True, capture_output=True)
+    for edges in (ti.standard_triangulation(d), ti.fan_triangulation(d), greedy_triangulation(d, 3)):
+        np.savetxt(tmp_path / "tri.txt", edges, fmt="%d")
+        out = subprocess.run([str(exe), str(d), str(tmp_path / "tri.txt"), "2"], capture_output=True, text=True)
+        assert out.returncode == 0, out.stdout + out.stderr
