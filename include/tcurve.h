@@ -344,7 +344,8 @@ ts_status ts_batch_run(ts_batch *batch, int use_graph, void *stream);
  * kernel TS_KERNEL_TABLE or TS_KERNEL_WARP, 128 threads, its chunk, scratch
  * TS_SCRATCH_SHARED, and the registers, resident blocks and grid of its
  * tier's kernel.
- *   info  receives kernel (TS_KERNEL_*), threads per block, chunk (sign
+ *   info  receives kernel (TS_KERNEL_*), threads of the tile (bit-sliced
+ *         tiles: 128, with blocks of 64 or 192 at d = 13 and 14), chunk (sign
  *         vectors per work item), scratch (TS_SCRATCH_*), registers per
  *         thread, local_bytes (per-thread local memory: spills, call
  *         frames), blocks_per_sm (resident blocks of the launch) and grid

@@ -294,9 +294,10 @@ struct ts_batch {
   struct Group {  // all jobs of one degree
     int d = 0, threads = 64, chunk = 1024;
     bool global = false;        // per-thread scratch in global memory
-    bool sliced = false;        // the bit-sliced kernel (kSlicedThreads threads, shared memory)
-    uint32_t stable_words = 0;  // its tables (largest of the group's) and areas
-    size_t sarea = 0;
+    bool sliced = false;        // the bit-sliced kernel (shared memory)
+    SlicedLayout slargest{};    // its largest tables and most event chunks
+    uint64_t n = 0;             // sign vectors of its jobs
+    SlicedJobs splan;
     std::shared_ptr<JitJobsModule> jit;  // specialised kernel (null: table-driven)
     std::string jit_log;        // why the specialised kernel could not be built
     JobsFn fn = nullptr;        // the kernel of this tile, its launch shape
@@ -377,13 +378,13 @@ cudaError_t prepare_group(ts_batch::Group &g) {
   int per_sm = 0, sms = 0, dev = 0;
   cudaError_t e = cudaSuccess;
   if (!g.jit && g.sliced) {
-    const void *fn = sliced_jobs_fn(g.d);
-    if (!fn) return cudaErrorInvalidConfiguration;
+    g.splan = sliced_jobs(g.d, g.slargest, g.n);
+    if (!g.splan.fn) return cudaErrorInvalidConfiguration;
     g.fn = nullptr;
-    g.smem = ((size_t)g.stable_words * 4 + 127) / 128 * 128 + 128 + g.sarea;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxBlockSmem);
+    g.smem = g.splan.smem;
+    e = cudaFuncSetAttribute(g.splan.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxBlockSmem);
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, g.threads, g.smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, g.splan.fn, g.splan.threads, g.smem);
     if (e != cudaSuccess) return e;
   } else if (g.jit) {  // specialised: 128-thread blocks, global scratch, grid from its occupancy
     g.fn = nullptr;
@@ -425,9 +426,8 @@ cudaError_t launch_group(ts_batch *b, ts_batch::Group &g, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(g.d_work, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
   if (!g.jit && g.sliced)
-    return sliced_jobs_launch(g.d, g.grid, g.smem, (g.stable_words * 4 + 127) / 128 * 128, g.d_jobs,
-                              (uint32_t)g.jobs.size(), g.items, (uint32_t)g.chunk, g.d_work, b->d_err,
-                              b->d_failed, st);
+    return sliced_jobs_launch(g.splan, g.grid, g.d_jobs, (uint32_t)g.jobs.size(), g.items,
+                              (uint32_t)g.chunk, g.d_work, b->d_err, b->d_failed, st);
   if (g.jit)
     return jit_jobs_launch(*g.jit, g.grid, g.d_jobs, (uint32_t)g.jobs.size(), g.items,
                            (uint32_t)g.chunk, g.d_work, b->d_err, b->d_failed, g.scratch, st);
@@ -563,7 +563,7 @@ void table_tile(ts_batch::Group &g, int threads, int chunk, int scratch) {
 }
 void table_defaults(ts_batch::Group &g) {
   g.jit.reset();
-  table_tile(g, kSlicedThreads, kSlicedThreads * 8, TS_SCRATCH_AUTO);
+  table_tile(g, kSlicedThreads, (int)sliced_jobs(g.d, g.slargest, g.n).chunk, TS_SCRATCH_AUTO);
 }
 
 // TS_KERNEL_AUTO at creation: specialised code for groups of at least
@@ -698,7 +698,6 @@ ts_status ts_batch_create(int njobs, ts_tri *const *tris, const uint64_t *counts
       g.table_words = t->lay.words;
       g.off_fan = t->lay.off_fan;
       g.off_vext = t->lay.off_vext;
-      table_defaults(g);
       b->groups.push_back(g);
     }
     auto &grp = b->groups[gi[t->d]];
@@ -706,9 +705,11 @@ ts_status ts_batch_create(int njobs, ts_tri *const *tris, const uint64_t *counts
     grp.table_words = std::max(grp.table_words, t->lay.words);
     const uint32_t epw = (uint32_t)tc_layout(t->d, true, 32).epw;
     grp.ls_words = std::max(grp.ls_words, (t->lay.nslots + epw - 1) / epw);
-    grp.stable_words = std::max(grp.stable_words, t->slay.words);
-    grp.sarea = std::max(grp.sarea, fused_area_bytes(t->d, t->slay));
+    grp.slargest.words = std::max(grp.slargest.words, t->slay.words);
+    grp.slargest.chunks = std::max(grp.slargest.chunks, t->slay.chunks);
+    grp.n += counts[j];
   }
+  for (auto &g : b->groups) table_defaults(g);
   if (e == cudaSuccess) {
     std::vector<int> spec;
     for (size_t gi = 0; gi < b->groups.size(); ++gi)
@@ -942,13 +943,14 @@ ts_status ts_batch_info(const ts_batch *b, int d, ts_batch_group_info *info, cha
     if (g.jit) {
       jit_jobs_attrs(*g.jit, &x.registers, &x.local_bytes);
       x.blocks_per_sm = jit_jobs_blocks_per_sm(*g.jit);
-    } else if (const void *fn = g.sliced ? sliced_jobs_fn(g.d) : (const void *)g.fn) {
+    } else if (const void *fn = g.sliced ? g.splan.fn : (const void *)g.fn) {
       cudaFuncAttributes fa{};
       if (cudaFuncGetAttributes(&fa, fn) == cudaSuccess) {
         x.registers = fa.numRegs;
         x.local_bytes = (int)fa.localSizeBytes;
       }
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x.blocks_per_sm, fn, g.threads, g.smem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x.blocks_per_sm, fn,
+                                                    g.sliced ? (int)g.splan.threads : g.threads, g.smem);
     }
     *info = x;
     if (log && len) {

@@ -121,9 +121,10 @@ struct ts_tri {
   tcurve::Diamond dia;
   int kernel = 0;                // TS_KERNEL_*
   int scratch = 0;               // TS_SCRATCH_* (both kernel families)
-  // blocks the device holds of the bit-sliced query and sweep kernels (0: not
-  // asked yet); they depend on the degree and the tables alone
-  mutable std::atomic<uint32_t> resident[2] = {};
+  // blocks the device holds of the bit-sliced query and sweep kernels, then of
+  // their wide ones (0: not asked yet); they depend on the degree and the tables
+  // alone
+  mutable std::atomic<uint32_t> resident[4] = {};
   int occupancy = 0;             // target blocks per SM of the specialised kernels (0: default)
   std::mutex jit_mu;
   std::shared_ptr<tcurve::JitModule> jit;
@@ -238,13 +239,20 @@ struct DevJob {
 static_assert(sizeof(DevJob) == 88 && offsetof(DevJob, fn) == 64,
               "the job table layout of the generated batch kernels");
 
-// The bit-sliced kernel of a degree group (sliced_jobs.cu): smem = toff (the
-// tables, 128-byte aligned) + 128 + fused_area_bytes.
-constexpr int kSlicedThreads = 128;  // threads and sign vectors per block
-const void *sliced_jobs_fn(int d);
-cudaError_t sliced_jobs_launch(int d, unsigned grid, size_t smem, uint32_t toff, const DevJob *jobs,
-                               uint32_t njobs, uint64_t items, uint32_t chunk, unsigned long long *work,
-                               uint32_t *err, unsigned long long *failed, cudaStream_t st);
+// The bit-sliced kernel of a degree group (sliced_jobs.cu) for jobs with tables
+// and event chunks up to `largest` and n sign vectors in all: its threads per block, default sign vectors
+// per work item, the bytes of the staged tables, its shared memory.
+struct SlicedJobs {
+  const void *fn = nullptr;
+  unsigned threads = 0, chunk = 0;
+  uint32_t toff = 0;
+  size_t smem = 0;
+};
+constexpr int kSlicedThreads = 128;  // the tile (ts_batch_set_tile) that stands for it
+SlicedJobs sliced_jobs(int d, const SlicedLayout &largest, uint64_t n);
+cudaError_t sliced_jobs_launch(const SlicedJobs &p, unsigned grid, const DevJob *jobs, uint32_t njobs,
+                               uint64_t items, uint32_t chunk, unsigned long long *work, uint32_t *err,
+                               unsigned long long *failed, cudaStream_t st);
 
 // Fused batch plan (fused.cu): one persistent kernel per tier of degrees over
 // the batch's jobs, each degree with its own tile (bit-sliced or one warp per

@@ -387,24 +387,25 @@ struct GlobalScratch {
   }
 };
 
-template <class K>
+// WHICH: the kernel's place in ts_tri::resident.
+template <class K, int WHICH>
 cudaError_t real_schemes_blocks(const ts_tri *t, const uint64_t *signs, uint64_t n, uint64_t *codes,
                                 cudaStream_t st) {
   const size_t smem = tc_sl_bytes<K>(t->slay.words, t->slay.chunks);
   unsigned grid = 0;
-  cudaError_t e = persistent_grid(t, 0, sliced_real_schemes_kernel<K>, K::T, smem, (n + K::T - 1) / K::T, &grid);
+  cudaError_t e = persistent_grid(t, WHICH, sliced_real_schemes_kernel<K>, K::T, smem, (n + K::T - 1) / K::T, &grid);
   if (e != cudaSuccess) return e;
   sliced_real_schemes_kernel<K><<<grid, K::T, smem, st>>>(t->slay, t->d_stables, signs, n, codes, t->d_err);
   return cudaGetLastError();
 }
 
-template <class K>
+template <class K, int WHICH>
 cudaError_t enumerate_blocks(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *h,
                              cudaStream_t st) {
   const size_t smem = tc_sl_bytes<K>(t->slay.words, t->slay.chunks) + (size_t)K::HASH * 16;
   const uint64_t total = hi - lo;
   unsigned grid = 0;
-  cudaError_t e = persistent_grid(t, 1, sliced_enumerate_kernel<K>, K::T, smem, (total + K::T - 1) / K::T, &grid);
+  cudaError_t e = persistent_grid(t, WHICH, sliced_enumerate_kernel<K>, K::T, smem, (total + K::T - 1) / K::T, &grid);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(h->d_work, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
@@ -415,17 +416,17 @@ cudaError_t enumerate_blocks(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t
 template <int D>
 cudaError_t real_schemes_sliced(const ts_tri *t, const uint64_t *signs, uint64_t n, uint64_t *codes,
                                 cudaStream_t st) {
-  return tc_sl_wide<D>(t->slay.words, t->slay.chunks)
-             ? real_schemes_blocks<TcSlWide<D>>(t, signs, n, codes, st)
-             : real_schemes_blocks<TcSlNarrow<D>>(t, signs, n, codes, st);
+  return tc_sl_wide<D>(t->slay.words, t->slay.chunks, n)
+             ? real_schemes_blocks<TcSlWide<D>, 2>(t, signs, n, codes, st)
+             : real_schemes_blocks<TcSlNarrow<D>, 0>(t, signs, n, codes, st);
 }
 
 template <int D>
 cudaError_t enumerate_sliced(const ts_tri *t, uint64_t lo, uint64_t hi, uint32_t flags, ts_hist *h,
                              cudaStream_t st) {
-  return tc_sl_wide<D>(t->slay.words, t->slay.chunks)
-             ? enumerate_blocks<TcSlWide<D>>(t, lo, hi, flags, h, st)
-             : enumerate_blocks<TcSlNarrow<D>>(t, lo, hi, flags, h, st);
+  return tc_sl_wide<D>(t->slay.words, t->slay.chunks, hi - lo)
+             ? enumerate_blocks<TcSlWide<D>, 3>(t, lo, hi, flags, h, st)
+             : enumerate_blocks<TcSlNarrow<D>, 1>(t, lo, hi, flags, h, st);
 }
 
 template <int D>

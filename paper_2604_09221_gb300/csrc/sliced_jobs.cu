@@ -1,6 +1,6 @@
 // sliced_jobs.cu -- the bit-sliced kernel of a degree group of a batch
 // (ts_batch, one persistent kernel per degree; batch.cu plans and launches
-// it).  One kernel per degree, 128 sign vectors per block at a time.
+// it).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -11,14 +11,21 @@
 namespace tcurve {
 namespace {
 
-// The bit-sliced kernel of a degree group: 128 sign vectors per block at a
-// time (tc_sliced.cuh), everything in shared memory.  smem: tables (toff
-// bytes) | mbarrier, work slot (128 bytes) | the block's areas.
-template <int D>
-__global__ void __launch_bounds__(kSlicedThreads)
+// Work items of chunk sign vectors, K::T of them at a time (tc_sliced.cuh),
+// everything in shared memory.  smem: tables (toff bytes) | mbarrier, work slot
+// (128 bytes) | the block's areas.
+//
+// Blocks of 128, but at d = 13 and 14 of 64 or 192 (tc_sl_wide): 128 are one
+// block per multiprocessor there, and four jobs of 2^20 took 15.1 and 21.1 ms
+// against 14.0 and 18.9 with one thread per sign vector; now 10.4 and 15.1.
+// Their work items are two blocks long, so that short jobs wait for no more
+// phases.
+// (d = 15 and 16 have two blocks of 64 or one of 128: 20.2 and 27.6 ms with
+// 128, 19.7 and 27.6 with 64, whose short jobs take up to twice as long.)
+template <class K>
+__global__ void __launch_bounds__(K::T)
     sliced_jobs_kernel(const DevJob *__restrict__ jobs, u32 njobs, u64 total_items, u32 chunk, u32 toff,
                        unsigned long long *work, u32 *err_word, unsigned long long *failed_word) {
-  typedef TcSlK<D, kSlicedThreads / 32> K;
   extern __shared__ __align__(128) uint8_t smem[];
   u32 *tab = reinterpret_cast<u32 *>(smem);
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem + toff);
@@ -56,8 +63,8 @@ __global__ void __launch_bounds__(kSlicedThreads)
       cur = lo;
     }
     const TcSlMem M = tc_sl_carve<K>(tab, reinterpret_cast<u32 *>(smem + toff + 128), J.schunks);
-    const u64 first = (c - J.chunk0) * (u64)chunk;
-    for (u32 k = 0; k < chunk && first + k < J.n; k += K::T) {
+    const u64 first = (c - J.chunk0) * (u64)chunk, end = first + chunk < J.n ? first + chunk : J.n;
+    for (u32 k = 0; first + k < end; k += K::T) {
       // the sign vector of counter base + idx, as ts_splitmix_masks writes it
       TcSig<K::W> sg;
 #pragma unroll
@@ -68,7 +75,7 @@ __global__ void __launch_bounds__(kSlicedThreads)
       tc_sl_classify<K>(M, sg, t, e, code);
       const u64 idx = first + k + mine;
       u64 any = 0;
-      const bool live = idx < J.n;
+      const bool live = idx < end;
 #pragma unroll
       for (u32 w = 0; w < K::CW; ++w) {
         code[w] = live ? code[w] : 0ull;
@@ -93,27 +100,39 @@ __global__ void __launch_bounds__(kSlicedThreads)
 
 typedef void (*SlicedJobsFn)(const DevJob *, u32, u64, u32, u32, unsigned long long *, u32 *,
                              unsigned long long *);
-SlicedJobsFn kernel_of(int d) {
-  switch (d) {
-#define TC_CASE(x) \
-  case x: return sliced_jobs_kernel<x>;
-    TC_CASE(1) TC_CASE(2) TC_CASE(3) TC_CASE(4) TC_CASE(5) TC_CASE(6) TC_CASE(7) TC_CASE(8) TC_CASE(9)
-    TC_CASE(10) TC_CASE(11) TC_CASE(12) TC_CASE(13) TC_CASE(14) TC_CASE(15) TC_CASE(16)
-#undef TC_CASE
-    default: return nullptr;
-  }
+
+template <class K>
+SlicedJobs plan_k(const SlicedLayout &l) {
+  return SlicedJobs{(const void *)sliced_jobs_kernel<K>, K::T, K::T == 128 ? 1024 : 2 * K::T,
+                    (l.words * 4 + 127) / 128 * 128, tc_sl_bytes<K>(l.words, l.chunks)};
+}
+template <int D>
+SlicedJobs plan_d(const SlicedLayout &l, u64 n) {
+  if constexpr (D == 13 || D == 14)
+    return tc_sl_wide<D>(l.words, l.chunks, n) ? plan_k<TcSlWide<D>>(l) : plan_k<TcSlNarrow<D>>(l);
+  else
+    return plan_k<TcSlK<D, 4>>(l);
 }
 
 }  // namespace
 
-const void *sliced_jobs_fn(int d) { return (const void *)kernel_of(d); }
+SlicedJobs sliced_jobs(int d, const SlicedLayout &largest, uint64_t n) {
+  switch (d) {
+#define TC_CASE(x) \
+  case x: return plan_d<x>(largest, n);
+    TC_CASE(1) TC_CASE(2) TC_CASE(3) TC_CASE(4) TC_CASE(5) TC_CASE(6) TC_CASE(7) TC_CASE(8) TC_CASE(9)
+    TC_CASE(10) TC_CASE(11) TC_CASE(12) TC_CASE(13) TC_CASE(14) TC_CASE(15) TC_CASE(16)
+#undef TC_CASE
+    default: return SlicedJobs{};
+  }
+}
 
-cudaError_t sliced_jobs_launch(int d, unsigned grid, size_t smem, uint32_t toff, const DevJob *jobs,
-                               uint32_t njobs, uint64_t items, uint32_t chunk, unsigned long long *work,
-                               uint32_t *err, unsigned long long *failed, cudaStream_t st) {
-  const SlicedJobsFn fn = kernel_of(d);
-  if (!fn) return cudaErrorInvalidValue;
-  fn<<<grid, kSlicedThreads, smem, st>>>(jobs, njobs, items, chunk, toff, work, err, failed);
+cudaError_t sliced_jobs_launch(const SlicedJobs &p, unsigned grid, const DevJob *jobs, uint32_t njobs,
+                               uint64_t items, uint32_t chunk, unsigned long long *work, uint32_t *err,
+                               unsigned long long *failed, cudaStream_t st) {
+  if (!p.fn) return cudaErrorInvalidValue;
+  reinterpret_cast<SlicedJobsFn>(const_cast<void *>(p.fn))<<<grid, p.threads, p.smem, st>>>(
+      jobs, njobs, items, chunk, p.toff, work, err, failed);
   return cudaGetLastError();
 }
 

@@ -741,15 +741,19 @@ constexpr size_t tc_sl_bytes(u32 table_words, u32 chunks) {
 // three blocks of 64, one of 128; 0.40 against 0.28e9 schemes/s).
 template <int D>
 using TcSlNarrow = TcSlK<D, D <= 12 ? 4 : 2>;
-// Or, at d = 13 and 14, of 192 where that is more: one block of 192 against two
-// of 64 at d = 14 (2^21 queries 10.2 -> 7.4 ms; one thread per sign vector with
-// scratch in global memory 8.6; the same from 2^16 down).  Above, 192 do not fit.
+// Or, at d = 13 and 14, of 192 where that is more, so that the n sign vectors of
+// a launch are fewer waves of blocks (152 multiprocessors): one block of 192
+// against two of 64 at d = 14 (2^21 queries 10.2 -> 7.4 ms, one thread per sign
+// vector with scratch in global memory 8.6; 2^16 0.42 -> 0.35; as many waves,
+// 2^13 0.136 against 0.142, 2^15 0.23 against 0.24).  Above, 192 do not fit.
 template <int D>
 using TcSlWide = TcSlK<D, D == 13 || D == 14 ? 6 : D <= 12 ? 4 : 2>;
 template <int D>
-constexpr bool tc_sl_wide(u32 table_words, u32 chunks) {
+constexpr bool tc_sl_wide(u32 table_words, u32 chunks, u64 n) {
   constexpr size_t BLOCK = 227 * 1024, SM = 228 * 1024, RESERVED = 1024;  // of a block
-  const size_t n = tc_sl_bytes<TcSlNarrow<D>>(table_words, chunks), w = tc_sl_bytes<TcSlWide<D>>(table_words, chunks);
-  return TcSlWide<D>::T > TcSlNarrow<D>::T && w <= BLOCK &&
-         SM / (w + RESERVED) * TcSlWide<D>::T > SM / (n + RESERVED) * TcSlNarrow<D>::T;
+  constexpr u32 NT = TcSlNarrow<D>::T, WT = TcSlWide<D>::T;
+  const size_t nb = tc_sl_bytes<TcSlNarrow<D>>(table_words, chunks), wb = tc_sl_bytes<TcSlWide<D>>(table_words, chunks);
+  if (WT <= NT || wb > BLOCK) return false;
+  const u64 narrow = SM / (nb + RESERVED) * NT * 152, wide = SM / (wb + RESERVED) * WT * 152;  // a wave
+  return (n + wide - 1) / wide < (n + narrow - 1) / narrow;
 }

@@ -160,20 +160,20 @@ def test_a_captured_sweep(eng, d, name, prepare):
 
 @pytest.mark.parametrize("d", [13, 14])
 def test_ragged_blocks_of_64_and_192(eng, orc, d):
-    """Queries and sampled sweeps around the blocks' sizes, and nothing written
-    behind the last code."""
+    """Queries and sampled sweeps around the blocks' sizes, of one wave of narrow
+    blocks and more, and nothing written behind the last code."""
     import torch
     for edges in (ti.regular_triangulation(d, seed=d), greedy_triangulation(d, 3)):
         tri = eng.Triangulation(d, edges)
         otri = orc.triangles(d, edges)
-        want = orc.real_schemes(d, otri, ti.splitmix_sign_vectors(d, 77, 1000))
-        for n in (1, 63, 64, 65, 191, 192, 193, 1000):
+        want = orc.real_schemes(d, otri, ti.splitmix_sign_vectors(d, 77, 20001))
+        for n in (1, 63, 64, 65, 191, 192, 193, 1000, 152 * 128, 152 * 128 + 1, 20001):
             out = torch.full((n + 4, tri.code_words), -7, dtype=torch.int64, device="cuda")
             tri.real_schemes(eng.splitmix_masks(d, 77, n), out=out)
             got = out.cpu().numpy()
             assert (got[:n].view(np.uint64) == want[:n]).all(), n
             assert (got[n:] == -7).all()
-            h = eng.Histogram(2048, tri.code_words)
+            h = eng.Histogram(1 << 15, tri.code_words)
             eng.enumerate_schemes(tri, 77, 77 + n, h, eng.TS_ENUM_SPLITMIX)
             codes, counts, failed = h.read()
             assert failed == 0
@@ -210,3 +210,37 @@ def test_long_queries_are_no_slower_than_one_thread_per_sign_vector(eng, d):
         tri.set_scratch(scratch)
         ms[kind] = _ms(lambda: tri.real_schemes(signs, out=out))
     assert ms[eng.TS_KERNEL_AUTO] < 1.05 * ms[eng.TS_KERNEL_TABLE], ms
+
+
+@pytest.mark.parametrize("d,large", [(12, 2000), (13, 2000), (14, 2000), (14, 20001), (16, 2000)])
+def test_batch_groups_of_ragged_jobs(eng, d, large):
+    """Degree groups whose work items are no multiple of the blocks (64, 128 or
+    192 sign vectors), against sampled sweeps of the same streams."""
+    tris = [eng.Triangulation(d, e) for e in (ti.regular_triangulation(d, seed=d), greedy_triangulation(d, 3))]
+    counts = [1, 63, 192, 193, 1537, large]
+    jobs = [tris[j % 2] for j in range(len(counts))]
+    batch = eng.Batch(jobs, counts, [1000 * j for j in range(len(counts))], hist_capacity=1 << 15)
+    for chunk in (None, 128, 384, 1024):
+        if chunk:
+            batch.set_tile(d, 128, chunk)
+        batch.run()
+        for j, (tri, n) in enumerate(zip(jobs, counts)):
+            h = eng.Histogram(1 << 15, tri.code_words)
+            eng.enumerate_schemes(tri, 1000 * j, 1000 * j + n, h, eng.TS_ENUM_SPLITMIX)
+            codes, cnts, _ = h.read()
+            got, gcnt, failed = batch.read(j)
+            assert failed == 0 and int(gcnt.sum()) == n, (chunk, j)
+            np.testing.assert_array_equal(got.reshape(codes.shape), codes)
+            np.testing.assert_array_equal(gcnt, cnts)
+
+
+@pytest.mark.parametrize("d", [13, 14, 15])
+def test_large_batch_groups_are_no_slower_than_one_thread_per_sign_vector(eng, d):
+    """The default tile against the tile that was the default before it (128
+    threads, scratch in global memory), four jobs of 2^20 sign vectors (with
+    blocks of 128 at d = 13 and 14 it took 1.08 and 1.12 of its time)."""
+    tri = eng.Triangulation(d, ti.regular_triangulation(d, seed=d))
+    batch = eng.Batch([tri] * 4, [1 << 20] * 4, [j << 40 for j in range(4)], hist_capacity=1 << 18)
+    ms = _ms(batch.run, 3)
+    batch.set_tile(d, 128, 1024, eng.TS_SCRATCH_GLOBAL)
+    assert ms < 1.05 * _ms(batch.run, 3)
