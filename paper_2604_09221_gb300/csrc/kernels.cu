@@ -247,7 +247,8 @@ __global__ void __launch_bounds__(K::T)
     if (t == 0) *slot = atomicAdd(h.d_work, (unsigned long long)K::T);
     u32 e = 0;
     u64 code[K::CW];
-    tc_sl_classify<K>(M, tc_enum_sig<K::W>(lo + base + t, flags, K::D), t, e, code);
+    // threads behind the range take its last sign vector: no longer chains than its own
+    tc_sl_classify<K>(M, tc_enum_sig<K::W>(lo + (base + t < total ? base + t : total - 1), flags, K::D), t, e, code);
     u64 any = 0;
     const bool live = base + mine < total;
 #pragma unroll

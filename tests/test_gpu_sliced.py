@@ -244,3 +244,25 @@ def test_large_batch_groups_are_no_slower_than_one_thread_per_sign_vector(eng, d
     ms = _ms(batch.run, 3)
     batch.set_tile(d, 128, 1024, eng.TS_SCRATCH_GLOBAL)
     assert ms < 1.05 * _ms(batch.run, 3)
+
+
+def test_a_single_sampled_sign_vector_waits_for_its_own_chains(eng):
+    """A sweep of one sign vector takes less than one of a block (0.77 of it at
+    d = 10), whose longest joins and trees it would wait for if the threads
+    behind the range had sign vectors of their own."""
+    import time
+
+    import torch
+    tri = eng.Triangulation(10, ti.regular_triangulation(10, seed=10))
+    h = eng.Histogram(4096, tri.code_words)
+    us = {}
+    for n in (1, 128):
+        times = []
+        for _ in range(40):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            eng.enumerate_schemes(tri, 5, 5 + n, h, eng.TS_ENUM_SPLITMIX)
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - t)
+        us[n] = sorted(times)[20]
+    assert us[1] < 0.92 * us[128], us
