@@ -109,14 +109,14 @@ struct ts_tri {
   int device = 0;
   tcurve::TableLayout lay{};
   std::vector<uint32_t> host_tables;
-  uint32_t *d_tables = nullptr;  // lay.words words, 16-byte aligned
+  uint32_t *d_tables = nullptr;  // lay.words words, 16-byte aligned; the allocation of all four
   tcurve::WarpLayout wlay{};
   std::vector<uint32_t> host_wtables;
   uint32_t *d_wtables = nullptr;  // wlay.words words (warp-per-instance kernels)
   tcurve::SlicedLayout slay{};
   std::vector<uint32_t> host_stables;
   uint32_t *d_stables = nullptr;  // slay.words words (bit-sliced kernels)
-  uint32_t *d_err = nullptr;     // device error word (scratch, owned here)
+  uint32_t *d_err = nullptr;     // device error word
   int open = 0;                  // components next to the middle row (d <= 9)
   tcurve::Diamond dia;
   int kernel = 0;                // TS_KERNEL_*

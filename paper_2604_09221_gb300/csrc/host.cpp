@@ -536,20 +536,18 @@ ts_status ts_load_triangulation(int d, const int32_t *edges_ij, int n_edges, ts_
     return TS_ENOTTRI;
   }
   cudaError_t e = cudaGetDevice(&t->device);
-  if (e == cudaSuccess) e = cudaMalloc(&t->d_tables, t->lay.words * sizeof(uint32_t));
+  // the three tables (each padded to 16 bytes) and the error word, in one
+  // allocation and one copy
+  std::vector<uint32_t> all(t->host_tables);
+  all.insert(all.end(), t->host_wtables.begin(), t->host_wtables.end());
+  all.insert(all.end(), t->host_stables.begin(), t->host_stables.end());
+  all.push_back(0);
+  if (e == cudaSuccess) e = cudaMalloc(&t->d_tables, all.size() * sizeof(uint32_t));
   if (e == cudaSuccess)
-    e = cudaMemcpy(t->d_tables, t->host_tables.data(), t->lay.words * sizeof(uint32_t),
-                   cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&t->d_wtables, t->wlay.words * sizeof(uint32_t));
-  if (e == cudaSuccess)
-    e = cudaMemcpy(t->d_wtables, t->host_wtables.data(), t->wlay.words * sizeof(uint32_t),
-                   cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&t->d_stables, t->slay.words * sizeof(uint32_t));
-  if (e == cudaSuccess)
-    e = cudaMemcpy(t->d_stables, t->host_stables.data(), t->slay.words * sizeof(uint32_t),
-                   cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&t->d_err, sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMemset(t->d_err, 0, sizeof(uint32_t));
+    e = cudaMemcpy(t->d_tables, all.data(), all.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
+  t->d_wtables = t->d_tables + t->lay.words;
+  t->d_stables = t->d_wtables + t->wlay.words;
+  t->d_err = t->d_stables + t->slay.words;
   if (e != cudaSuccess) {
     ts_status s = cuda_status(e);
     ts_free_triangulation(t);
@@ -563,9 +561,6 @@ void ts_free_triangulation(ts_tri *t) {
   if (!t) return;
   jit_release(t);
   if (t->d_tables) cudaFree(t->d_tables);
-  if (t->d_wtables) cudaFree(t->d_wtables);
-  if (t->d_stables) cudaFree(t->d_stables);
-  if (t->d_err) cudaFree(t->d_err);
   delete t;
 }
 

@@ -2,7 +2,8 @@
 // devices (this program's definitions come before the shared library's).
 // Exit 0 when the copies of a read are ordered behind the kernel that packs
 // its entries, i.e. made with the batch's device current, whatever the
-// caller's is, and when a reader whose stream is busy holds up no other.
+// caller's is, when a reader whose stream is busy holds up no other, and when a
+// triangulation is loaded by one allocation and one copy.
 #include <cuda_runtime_api.h>
 
 #include <atomic>
@@ -29,6 +30,7 @@ const cudaStream_t kBusy = (cudaStream_t)0xA0, kIdle = (cudaStream_t)0xB0;
 std::mutex mu;
 std::condition_variable cv;
 bool waiting = false, released = false;
+int allocations = 0, uploads = 0;
 }  // namespace
 
 extern "C" {
@@ -61,6 +63,7 @@ cudaError_t cudaSetDevice(int d) {
   return cudaSuccess;
 }
 cudaError_t cudaMalloc(void **p, size_t n) {
+  ++allocations;
   *p = calloc(n, 1);
   return cudaSuccess;
 }
@@ -70,10 +73,12 @@ cudaError_t cudaFree(void *p) {
 }
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind k) {
   if (k == cudaMemcpyDeviceToHost) calls.push_back({'r', device});
+  else ++uploads;
   memcpy(d, s, n);
   return cudaSuccess;
 }
 cudaError_t cudaMemset(void *p, int v, size_t n) {
+  ++uploads;
   memset(p, v, n);
   return cudaSuccess;
 }
@@ -122,13 +127,17 @@ int main() {
   ts_batch *batch = nullptr;
   const uint64_t count = 1 << 20, base = 0;
   if (ts_load_triangulation(2, edges, 9, &tri) != TS_OK) return 2;
+  int bad = 0;
+  if (allocations != 1 || uploads != 1) {
+    printf("a load makes %d allocations, %d copies\n", allocations, uploads);
+    ++bad;
+  }
   if (ts_batch_create(1, &tri, &count, &base, nullptr, 1 << 15, &batch) != TS_OK) return 3;
   std::vector<uint64_t> codes(1 << 16), counts(1 << 16);
   auto read = [&](cudaStream_t st) {
     uint64_t n = 0, failed = 0;
     return ts_batch_read(batch, 0, codes.data(), counts.data(), codes.size(), &n, &failed, st);
   };
-  int bad = 0;
   for (int current : {0, 1})
     for (unsigned long long n : {3ull, 2000ull, 20000ull}) {  // one copy, two, the whole table
       packed = n;

@@ -1,4 +1,4 @@
-"""The order of ts_batch_read's work, over a fake of the CUDA runtime with two
+"""The order of ts_batch_read's work and the calls of a load, over a fake of the CUDA runtime with two
 devices (no GPU needed)."""
 import os
 import shutil
@@ -11,10 +11,10 @@ ROOT = os.path.dirname(HERE)
 CUDA = "/usr/local/cuda"
 
 
-def test_reads_are_ordered_on_the_batch_device(tmp_path):
+def test_reads_and_loads_over_a_fake_runtime(tmp_path):
     """The copies of a read are made on the batch's device, behind its pack
     kernel, whichever device is current; and a reader whose stream is busy
-    holds up no other reader."""
+    holds up no other reader.  A load makes one allocation and one copy."""
     if not shutil.which("g++") or not os.path.exists(os.path.join(CUDA, "include", "cuda_runtime.h")):
         pytest.skip("needs g++ and the CUDA headers")
     from paper_2604_09221_gb300 import build
