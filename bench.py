@@ -798,7 +798,7 @@ def mixed_run(steps, warmup, degrees=(5, 6, 7, 8, 9, 10), per_degree=32, seed=31
                        "fused": "one persistent kernel per tier of degrees (up to 6, 8, 10, 16; "
                                 "warp tiles), concurrent streams"}[plan],
             "plan_ms": order,
-            "fused_tiles": {str(d): [{1: "thread", 3: "warp"}.get(k, k), c]
+            "fused_tiles": {str(d): [{1: "bit-sliced", 3: "warp"}.get(k, k), c]
                             for d, (k, c) in sorted(ftiles.items())},
             "gpu_launches_per_step": fused_launches if plan == "fused" else len(degrees)}
 

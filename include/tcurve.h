@@ -119,7 +119,7 @@ ts_status ts_real_schemes(const ts_tri *tri, const uint64_t *signs, uint64_t n,
 /* Kernel families (ts_set_kernel).  All compute the same codes.
  *   TS_KERNEL_TABLE: one generic kernel per degree; the triangulation's
  *     tables are staged into shared memory by a bulk copy in every block.
- *     Blocks classify 64 or 128 sign vectors together, bit-sliced (with
+ *     Blocks classify 64, 128 or 192 sign vectors together, bit-sliced (with
  *     TS_SCRATCH_GLOBAL: one thread per sign vector).  Sweeps of at least 2^19
  *     masks that differ in the middle row block by block (4 <= d <= 9, not
  *     TS_ENUM_SPLITMIX) share the half-diamonds of each block.

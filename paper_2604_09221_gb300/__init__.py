@@ -366,7 +366,7 @@ class Batch:
 
     def set_fused_tile(self, d: int, kind: int, chunk: int):
         """Tile of degree d in the fused launch (ts_batch_set_fused_tile):
-        TS_KERNEL_TABLE (one thread per sign vector) or TS_KERNEL_WARP (one warp
+        TS_KERNEL_TABLE (bit-sliced) or TS_KERNEL_WARP (one warp
         per sign vector, d >= 7), and sign vectors per work item."""
         _check(_lib.ts_batch_set_fused_tile(self._h, int(d), int(kind), int(chunk)),
                "ts_batch_set_fused_tile")

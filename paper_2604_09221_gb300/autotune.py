@@ -3,15 +3,15 @@
 For every degree in a batch the persistent kernel has three knobs: threads
 per block, sign vectors per work item, and where the per-thread scratch
 lives: blocks of 128 threads with shared memory classify 128 sign vectors
-together (bit-sliced), the others one sign vector per thread.  A degree group that runs specialised code
-(ts_batch_info: compiled per triangulation, 128-thread blocks and global
-scratch fixed at compile time) has one knob, the sign vectors per work item.
-The tuner times candidate tiles on the batch's own jobs of that degree (a
-sub-batch, so degrees are tuned independently), keeps the fastest, and can
-store the choice in a JSON cache keyed by GPU name, degree and kernel family
-(path from the argument or the TCURVE_TILE_CACHE environment variable).  An
-entry holds the generation of the kernels it was timed with (GENERATION);
-entries of another one are timed again.
+together (bit-sliced), the others one sign vector per thread.  A degree
+group that runs specialised code (ts_batch_info: compiled per triangulation,
+128-thread blocks and global scratch fixed at compile time) has one knob, the
+sign vectors per work item.  The tuner times candidate tiles on the batch's
+own jobs of that degree (a sub-batch, so degrees are tuned independently),
+keeps the fastest, and can store the choice in a JSON cache keyed by GPU name,
+degree and kernel family (path from the argument or the TCURVE_TILE_CACHE
+environment variable).  An entry holds the generation of the kernels it was
+timed with (GENERATION); entries of another one are timed again.
 
 In the fused launch (ts_batch_set_fused: one kernel per tier of degrees) a
 degree's tile is the kind (bit-sliced or, from d = 7, one warp per sign

@@ -56,8 +56,11 @@ struct JobK : TcTableK<D_, T_, true> {
 
 
 // Degree groups of at least this many sign vectors run specialised code
-// (TS_KERNEL_AUTO): the compile at creation (about a second per
-// triangulation, in parallel) pays for itself.
+// (TS_KERNEL_AUTO, d <= kMaxBatchSpecialized), compiled at creation (about a
+// second per triangulation, in parallel).  The rule is from before the
+// bit-sliced kernels, which are faster now: four jobs of 2^20 at d = 3, 4, 5, 6
+// 0.43, 0.96, 1.30, 2.68 ms specialised, 0.25, 0.46, 0.48, 0.80 bit-sliced
+// (TS_KERNEL_TABLE or ts_batch_set_fused takes them).
 constexpr uint64_t kJitGroupMin = 1ull << 22;
 
 template <int D, int T, bool G>
@@ -184,7 +187,9 @@ JobsFn jobs_fn_tg(int t) {
     case 32: return jobs_fn<D, 32, G>();
     case 64: return jobs_fn<D, 64, G>();
     case 96: return jobs_fn<D, 96, G>();
-    case 128: return jobs_fn<D, 128, G>();
+    case 128:  // bit-sliced unless the scratch is global (table_tile)
+      if constexpr (G) return jobs_fn<D, 128, G>();
+      else return nullptr;
     case 192: return jobs_fn<D, 192, G>();
     case 256: return jobs_fn<D, 256, G>();
     default: return nullptr;

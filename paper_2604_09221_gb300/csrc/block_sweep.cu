@@ -118,7 +118,8 @@ __global__ void __launch_bounds__(128, D <= 7 ? 3 : 2)
       }
     }
     __syncthreads();
-    // at most 2^10 patterns per high part: counts stay below 2^32 for 2^15 items
+    // at most 2^10 patterns per high part: counts stay below 2^32 for fewer than
+    // 2^15 items
     if ((++items & 63u) == 0) flush();
   }
   __syncthreads();

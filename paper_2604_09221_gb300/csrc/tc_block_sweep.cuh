@@ -35,11 +35,10 @@
 // middle row alone, and every run has a node.
 //
 // The open comps are as many under every high part (open_components, engine.h):
-// d + 1 or fewer on the seeded regular triangulations up to d = 8, more the
-// more points the edges of the triangulation join to the x-axis.  Above K::NB
-// of them the block sweep is not launched (block_range).  High parts with more
-// than 32 comps (none seen below K::NB open ones) take the per-mask phases of
-// tc_sliced.cuh.
+// d on the standard triangulation, 12 on a seeded one at d = 9, up to 29 with
+// long edges at the x-axis.  Above K::NB of them the block sweep is not launched
+// (block_range).  High parts with more than 32 comps (none seen with up to K::NB
+// open ones) take the per-mask phases of tc_sliced.cuh.
 #pragma once
 
 #include "tc_sliced.cuh"
