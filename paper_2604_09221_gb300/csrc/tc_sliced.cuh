@@ -745,7 +745,8 @@ using TcSlNarrow = TcSlK<D, D <= 12 ? 4 : 2>;
 // a launch are fewer waves of blocks (152 multiprocessors): one block of 192
 // against two of 64 at d = 14 (2^21 queries 10.2 -> 7.4 ms, one thread per sign
 // vector with scratch in global memory 8.6; 2^16 0.42 -> 0.35; as many waves,
-// 2^13 0.136 against 0.142, 2^15 0.23 against 0.24).  Above, 192 do not fit.
+// 2^13 0.136 against 0.142, 2^15 0.23 against 0.24).  Bound by latency: six
+// warps per multiprocessor issue in 26 % of the slots.  Above, 192 do not fit.
 template <int D>
 using TcSlWide = TcSlK<D, D == 13 || D == 14 ? 6 : D <= 12 ? 4 : 2>;
 template <int D>
