@@ -103,7 +103,7 @@ bool build_diamond(int d, const std::vector<std::array<Pt, 3>> &tris, Diamond &D
   for (int v = 0; v < V; ++v) pos[verts[v]] = v;
 
   static const int qx[4] = {1, -1, -1, 1}, qy[4] = {1, 1, -1, -1};
-  std::set<std::array<int, 3>> dtris;
+  std::vector<std::array<int, 3>> dtris;  // of T^diamond, sorted
   std::vector<std::set<int>> adj(V);
   for (int q = 0; q < 4; ++q)
     for (auto &tr : tris) {
@@ -114,13 +114,15 @@ bool build_diamond(int d, const std::vector<std::array<Pt, 3>> &tris, Diamond &D
         adj[id[(k + 1) % 3]].insert(id[k]);
       }
       std::sort(id.begin(), id.end());
-      dtris.insert(id);
+      dtris.push_back(id);
     }
+  std::sort(dtris.begin(), dtris.end());
+  dtris.erase(std::unique(dtris.begin(), dtris.end()), dtris.end());
   if ((int)dtris.size() != 4 * d * d) return false;
   auto has_tri = [&](int a, int b, int c) {
     std::array<int, 3> id{a, b, c};
     std::sort(id.begin(), id.end());
-    return dtris.count(id) > 0;
+    return std::binary_search(dtris.begin(), dtris.end(), id);
   };
   D.d = d;
   D.V = V;
@@ -380,7 +382,8 @@ bool pack_sliced_tables(const Diamond &D, std::vector<uint32_t> &tables, SlicedL
   std::copy(mid_sites.begin(), mid_sites.end(), site.begin() + 32 * (nc1 + 1));
   // the boundary in cyclic order, p[t + 2d] antipodal to p[t]
   std::map<std::pair<int, int>, int> pos;
-  for (int v = 0; v < V; ++v) pos[{D.x[v], D.y[v]}] = v;
+  for (int v = 0; v < V; ++v)
+    if (std::abs(D.x[v]) + std::abs(D.y[v]) == d) pos[{D.x[v], D.y[v]}] = v;
   std::vector<int> p;
   for (int t = 0; t < d; ++t) p.push_back(pos.at({d - t, t}));
   for (int t = 0; t < d; ++t) p.push_back(pos.at({-t, d - t}));
